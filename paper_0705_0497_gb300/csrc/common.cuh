@@ -204,6 +204,25 @@ __device__ __forceinline__ uint32_t cic_r(float frac) {
     return (uint32_t)(frac * 65536.0f);
 }
 
+// The same cell, fraction and weight for x in [0, L) without float-integer
+// conversions (a quarter-rate unit): adding 2^23 with rounding down leaves the
+// truncated value in the low mantissa bits, exactly, for values in [0, 2^22).
+constexpr float TRUNC_MAGIC = 8388608.0f;   // 2^23
+constexpr int TRUNC_BITS = 0x4B000000;      // its bit pattern
+
+__device__ __forceinline__ float cell_limit(int Nc) { return TRUNC_MAGIC + (float)(Nc - 1); }
+
+__device__ __forceinline__ void cell_of_inside(float x, float inv_dx, float limit, int& j, float& frac) {
+    const float s = x * inv_dx;
+    const float t = fminf(__fadd_rd(s, TRUNC_MAGIC), limit);
+    j = __float_as_int(t) - TRUNC_BITS;
+    frac = s - (t - TRUNC_MAGIC);
+}
+
+__device__ __forceinline__ uint32_t cic_r_inside(float frac) {
+    return (uint32_t)(__float_as_int(__fadd_rd(frac * 65536.0f, TRUNC_MAGIC)) - TRUNC_BITS);
+}
+
 __device__ __forceinline__ bool is_dead(float x) { return x != x; }
 
 __device__ __forceinline__ float dead_marker() { return __uint_as_float(0x7FC00000u); }

@@ -136,6 +136,7 @@ struct Params {
     SpeciesBuf sp[NSP];
     // rate tables (cumulative, FP32), [NGRID][nproc]
     const float* cum[NSP];
+    const float* tot[NSP];       // [NGRID] the last cumulative column (total rate)
     int nproc[NSP];
     int kind[NSP][MAXPROC];
     float thr[NSP][MAXPROC];

@@ -10,12 +10,19 @@
 //     The common path reads x, vx, tc (12 B) and writes x, vx (8 B); id,
 //     vy, vz are read for collision candidates only.
 //   * a persistent grid; each warp owns one contiguous, 128-aligned slot range
-//     and walks it in rounds of 128 (lane l takes slots l, l+32, l+64, l+96:
-//     every load and store is one coalesced 128-byte line per array).  No
-//     block-wide barrier between the set-up and the final flush.
+//     (O2+: takes rounds of the whole array in turn) and walks it in rounds of
+//     128, a lane taking four neighbouring slots with one 16-byte load and
+//     store per array, the next round's loads in flight while it works on this
+//     one.  No block-wide barrier between the set-up and the final flush.
+//   * what bounds it: on large arrays HBM (20 B per particle; 4.65e7 O2+ on
+//     2048 cells 198 -> 180 us, 5.2 TB/s against 6.8 of a plain copy), on small ones the
+//     instructions (80 per 32 particles, before 122: integer deposit counters
+//     of 32 bits instead of a 64-bit compare-and-swap loop, no conversion on
+//     the FP64 unit, one branch per round for all that is rare) and the tail
+//     of collisions;
 //   * the gather field and the deposit live in shared memory; the deposit is
-//     one 64-bit atomic per particle holding (count, sum of CIC weights) per
-//     cell, turned into node charges when the block flushes;
+//     a count and a sum of CIC weights per cell, turned into node charges when
+//     the block flushes (one 64-bit add per node);
 //   * free flights (Sec. 2: "the durations of the free flights ... from
 //     elementary kinetic considerations"): each particle carries the step of
 //     its next null-collision candidate (tc, read with x and v_x), so the
@@ -36,15 +43,16 @@
 //     the end-of-step kernel places them in parent order.
 #include "common.cuh"
 
-// Launch shape of the particle kernels: minimum resident blocks per SM (caps
-// the registers; 4 timed fastest of 2, 3, 4 on the 512-cell, 1.6e7-particle
-// workload) and unrolling of the four particles a lane handles per round.
+// Launch shape of the particle kernels: minimum resident blocks per SM, which
+// caps the registers (80 at 3: room for the round in flight).  Per launch, 4, 3
+// and 2 blocks: electrons 24.7, 22.4, 22.8 us (1.5e6 on 512 cells) and 207, 206,
+// 228 us (2.6e7 on 2048 cells), O2+ 183, 180, 195 us (4.65e7 on 2048 cells).
 #ifndef O2PIC_PUSH_MIN_BLOCKS
-#define O2PIC_PUSH_MIN_BLOCKS 4
+#define O2PIC_PUSH_MIN_BLOCKS 3
 #endif
 // The electron kernel also runs the kinematics of its real collisions.
 #ifndef O2PIC_PUSH_E_MIN_BLOCKS
-#define O2PIC_PUSH_E_MIN_BLOCKS 4
+#define O2PIC_PUSH_E_MIN_BLOCKS 3
 #endif
 // Ion candidates filtered (gas target, energy against the total rate) and
 // their real collisions handled inside the particle kernel, as for the
@@ -56,15 +64,6 @@
 #ifndef O2PIC_FUSE_IONS
 #define O2PIC_FUSE_IONS 0
 #endif
-// Deposit: one 64-bit shared-memory atomic per particle (0), or lanes of a
-// warp that hit the same cell first summed over __match_any_sync peers and
-// added by one lane (1).  Integers: both give the same charge.  The
-// aggregated form was far slower on the 512-cell discharge (76.7 against
-// 46.3 ms per RF cycle): the lanes of a warp rarely share a cell, and the
-// match and the shuffles cost more than the atomics they save.
-#ifndef O2PIC_DEPOSIT_AGG
-#define O2PIC_DEPOSIT_AGG 0
-#endif
 // The particle kernel that runs the kinematics stages the species' cumulative
 // rate table in shared memory when that keeps its resident blocks per SM (1),
 // or reads it from global memory through L1 (0).  Both give the same results;
@@ -73,9 +72,6 @@
 // the electrons' 34 KB table each step, and the kinematics read a few rows.
 #ifndef O2PIC_CUM_SMEM
 #define O2PIC_CUM_SMEM 0
-#endif
-#ifndef O2PIC_PUSH_UNROLL
-#define O2PIC_PUSH_UNROLL 4
 #endif
 // Minimum resident blocks per SM of the kinematics kernel (caps its registers
 // at 85, no spills; 3 timed fastest of 2, 3, 4 on the same workload).
@@ -94,7 +90,6 @@ template <> struct SpeciesTraits<SP_OP> { static constexpr uint32_t tag = TAG_OP
 
 constexpr int WARPS = BLOCK / 32;           // 8
 constexpr int ROUND = 128;                  // slots per warp round (4 per lane)
-constexpr int PUSH_UNROLL = O2PIC_PUSH_UNROLL;
 
 struct PushShared {
     unsigned long long jsum;     // block's sum of trunc(256 v_x^{n+1/2})
@@ -105,6 +100,20 @@ struct PushShared {
     unsigned wtries;
     unsigned events[MAXPROC];    // electrons: real collisions per process
 };
+
+// First record of particle-kernel warp gw (of W) in its species' candidate list:
+// the warp's first slot, or, where warps take rounds in turn (O2+), the number
+// of slots in the rounds of the warps before it; never fewer records than the
+// slots it handles lie between two warps' starts.
+template <int S>
+__device__ __forceinline__ unsigned list_start(unsigned gw, unsigned W, unsigned nslots) {
+    if (S == SP_OP) {
+        const unsigned rounds = (nslots + ROUND - 1) / ROUND, q = rounds / W, rem = rounds % W;
+        return ROUND * (gw * q + (gw < rem ? gw : rem));
+    }
+    const unsigned R = warp_range_len(nslots, W);
+    return (gw * (unsigned long long)R < nslots) ? gw * R : nslots;
+}
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
 
@@ -309,9 +318,35 @@ __device__ __forceinline__ bool ion_is_real(const Params& P, const float* tot, u
 
 // Total-rate column (the last cumulative column) of species S into shared memory.
 __device__ __forceinline__ void stage_total(const Params& P, int S, float* tot) {
-    const int np = P.nproc[S];
-    const float* __restrict__ cum = P.cum[S];
-    for (int i = threadIdx.x; i < NGRID; i += blockDim.x) tot[i] = np > 0 ? cum[(size_t)i * np + np - 1] : 0.0f;
+    const float* __restrict__ g = P.tot[S];
+    for (int i = threadIdx.x; i < NGRID; i += blockDim.x) tot[i] = g[i];
+}
+
+// (long long)v for |v| >= 2^31 (and infinities, NaN) in integer arithmetic: a
+// 64-bit conversion runs on the FP64 unit, also where its predicate is false.
+__device__ __forceinline__ long long trunc_s64_large(float v) {
+    const uint32_t b = __float_as_uint(v);
+    const int e = (int)((b >> 23) & 0xFFu) - 150;                  // v = +-m 2^e, e >= 8
+    if (e > 39) return (v > 0.0f) ? 0x7FFFFFFFFFFFFFFFll : (long long)0x8000000000000000ull;
+    const long long m = (long long)((b & 0x007FFFFFu) | 0x00800000u) << e;
+    return (b >> 31) ? -m : m;
+}
+
+// The block's deposit: per cell the count of its particles and the sum of
+// their CIC weights r (32-bit counters: shared memory adds 32-bit words in one
+// instruction, 64-bit words in a compare-and-swap loop).  A weight sum that
+// wraps hands its 2^32 to the node charges at once: the one operation that
+// wrapped sees it in the old value, so no block is too large for the counters.
+__device__ __forceinline__ void weight_wrapped(unsigned long long* Q, int c, int sign) {
+    const unsigned long long w = (unsigned long long)((long long)sign << 32);
+    atomicAdd(&Q[c], 0ull - w);
+    atomicAdd(&Q[c + 1], w);
+}
+
+__device__ __forceinline__ void cell_sub(unsigned* cnt, unsigned* rsum, int c, uint32_t r, unsigned long long* Q) {
+    atomicSub(&cnt[c], 1u);
+    const unsigned old = atomicSub(&rsum[c], r);
+    if (old < r) weight_wrapped(Q, c, -1);
 }
 
 // Real collisions of the list of one particle-kernel warp (records r0 ..
@@ -323,8 +358,8 @@ __device__ __forceinline__ void stage_total(const Params& P, int S, float* tot) 
 // Philox stream is drawn again; ion records carry the slot, id, v and that
 // block (its first word, the candidate draw, is spent), x is read from the
 // array.  `cum` is the species' cumulative rate table (global or shared
-// memory).  A removed particle's charge comes off the block's histogram when
-// `hist` is given (the particle kernel: the particle was deposited there),
+// memory).  A removed particle's charge comes off the block's deposit when
+// `cnt` is given (the particle kernel: the particle was deposited there),
 // else off the step's deposit in global memory.  Births are ranked with
 // ballots within the segment and staged at the particle warp's slot range;
 // nb1, nb2 count them.
@@ -333,7 +368,8 @@ __device__ __forceinline__ void collide_list(const Params& P, const float* cum, 
                                              unsigned long long step,
                                              unsigned r0, unsigned n, unsigned nmax, unsigned sl,
                                              unsigned seg_mask, unsigned lt_mask, unsigned* events,
-                                             unsigned long long* hist, unsigned& nb1, unsigned& nb2,
+                                             unsigned* cnt, unsigned* rsum, unsigned long long* Qcopy,
+                                             unsigned& nb1, unsigned& nb2,
                                              unsigned& nremoved, unsigned& wtries, unsigned& wemax) {
     const int np = P.nproc[S];
     const unsigned cb = P.ctrl->cur[S];
@@ -374,10 +410,10 @@ __device__ __forceinline__ void collide_list(const Params& P, const float* cum, 
                     VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
                 } else {
                     X[slot] = dead_marker();
-                    if (hist) {
+                    if (cnt) {
                         int j; float f;
                         cell_of(x, inv_dx, Nc, j, f);
-                        atomicAdd(&hist[j], 0ull - ((1ull << 40) + (unsigned long long)cic_r(f)));
+                        cell_sub(cnt, rsum, j, cic_r(f), Qcopy);
                     } else {
                         deposit_sub_global(P.Qf[S], x, inv_dx, Nc);
                     }
@@ -414,13 +450,12 @@ __device__ __forceinline__ void collide_list(const Params& P, const float* cum, 
     }
 }
 
-// Candidate queue of one warp of the particle kernel (shared memory): slot,
-// x and v_x after the push of up to QN candidates in slot order.
-constexpr int QN = 64;
+// Candidate queue of one warp of the particle kernel (shared memory): the slots
+// of its candidates in slot order.  Fewer than 32 stay from one round to the
+// next and a round adds at most ROUND.
+constexpr int QN = 32 + ROUND;
 struct PushQueue {
     unsigned slot[WARPS][QN];
-    float x[WARPS][QN];
-    float vx[WARPS][QN];
 };
 
 // Body of the particle kernel for block blk of nblk blocks (the launch's own
@@ -431,9 +466,9 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const int np = P.nproc[S];
     PushShared& sh = *reinterpret_cast<PushShared*>(smem);
     float* Es = reinterpret_cast<float*>(smem + align16(sizeof(PushShared)));
-    unsigned long long* hist =
-        reinterpret_cast<unsigned long long*>(smem + align16(align16(sizeof(PushShared)) + sizeof(float) * P.Ng));
-    PushQueue& Q = *reinterpret_cast<PushQueue*>(hist + P.Ng);
+    unsigned* cnt = reinterpret_cast<unsigned*>(Es + P.Ng);
+    unsigned* rsum = cnt + P.Ng;
+    PushQueue& Q = *reinterpret_cast<PushQueue*>(rsum + P.Ng);
     float* Tt = reinterpret_cast<float*>(&Q + 1);        // total-rate column (filter in the kernel)
     float* Ct = Tt + NGRID;                              // cumulative table (if staged)
     constexpr bool fused = (S == SP_E) || (O2PIC_FUSE_IONS != 0);
@@ -442,8 +477,6 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned* qs = Q.slot[warp];
-    float* qx = Q.x[warp];
-    float* qv = Q.vx[warp];
 
     DevCtrl* C = P.ctrl;
     const unsigned long long step = C->step;
@@ -461,31 +494,52 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const float inv_lnq = P.inv_lnq[S], kcap = P.kcap[S];
     const unsigned sub = P.sub[S];
     const int Nc = P.Nc, Ng = P.Ng;
+    const float jmax = cell_limit(Nc);
+    unsigned long long* __restrict__ Qcopy = P.Qf[S] + (size_t)(blk & (QCOPIES - 1)) * Ng;
     const PhiloxPre pre = philox_pre(step_lo, SpeciesTraits<S>::tag, (uint32_t)(step >> 32), P.seed);
 
     // this warp's contiguous slot range, and its first round of x, v_x, tc
-    // requested before the block's set-up (their latency overlaps it)
+    // requested before the block's set-up (their latency overlaps it).  A lane
+    // takes four neighbouring slots of a round, one 16-byte word per array
+    // (ranges start on multiples of 128 slots); the last round of the slots in
+    // use is read slot by slot.
     const unsigned W = nblk * WARPS;
     const unsigned gw = blk * WARPS + warp;
     const unsigned R = warp_range_len(nslots, W);
     const unsigned r0 = (gw * (unsigned long long)R < nslots) ? gw * R : nslots;
     const unsigned r1 = (r0 + R < nslots) ? r0 + R : nslots;
+    // O2+ have no births, so nothing asks for their order: their warps take the
+    // rounds of the whole array in turn, and the grid sweeps it front to back
+    // (5.1 against 4.7 TB/s for 4.65e7 O2+ on 2048 cells).  Births are placed in
+    // parent order, so the other species' warps keep contiguous ranges.
+    constexpr bool in_turn = S == SP_OP;
+    const unsigned stride = in_turn ? W * ROUND : ROUND;
+    const unsigned ga = in_turn ? gw * ROUND : r0, gz = in_turn ? nslots : r1;
+    const unsigned rec0 = in_turn ? list_start<S>(gw, W, nslots) : r0;
     float xs[4], vxs[4];
     uint32_t tcs[4];
-    auto load_round = [&](unsigned g0) {
-        const bool full = g0 + ROUND <= r1;
+    auto load_round = [&](unsigned g0, float (&xs)[4], float (&vxs)[4], uint32_t (&tcs)[4]) {
+        const unsigned i0 = g0 + 4u * lane;
+        if (g0 + ROUND <= gz) {
+            const float4 a = *reinterpret_cast<const float4*>(X + i0);
+            const float4 b = *reinterpret_cast<const float4*>(VX + i0);
+            const uint4 c = *reinterpret_cast<const uint4*>(TC + i0);
+            xs[0] = a.x; xs[1] = a.y; xs[2] = a.z; xs[3] = a.w;
+            vxs[0] = b.x; vxs[1] = b.y; vxs[2] = b.z; vxs[3] = b.w;
+            tcs[0] = c.x; tcs[1] = c.y; tcs[2] = c.z; tcs[3] = c.w;
+        } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const unsigned i = g0 + 32u * k + lane;
-            const bool inr = full || i < r1;
-            xs[k] = inr ? X[i] : dead_marker();
-            vxs[k] = inr ? VX[i] : 0.0f;
-            tcs[k] = inr ? TC[i] : 0u;
+            for (int k = 0; k < 4; ++k) {
+                const bool inr = i0 + k < gz;
+                xs[k] = inr ? X[i0 + k] : dead_marker();
+                vxs[k] = inr ? VX[i0 + k] : 0.0f;
+                tcs[k] = inr ? TC[i0 + k] : 0u;
+            }
         }
     };
-    if (r0 < r1) load_round(r0);
+    if (ga < gz) load_round(ga, xs, vxs, tcs);
 
-    for (int j = tid; j < Ng; j += BLOCK) { Es[j] = P.Ef[j]; hist[j] = 0ull; }
+    for (int j = tid; j < Ng; j += BLOCK) { Es[j] = P.Ef[j]; cnt[j] = 0u; rsum[j] = 0u; }
     if (fused) stage_total(P, S, Tt);
     if (cum_staged) {
         const float* __restrict__ g = P.cum[S];
@@ -503,20 +557,22 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     unsigned nrec = 0;    // warp-uniform: records of this warp so far
     unsigned qn = 0;      // warp-uniform: queued candidates
 
-    // The first m (<= 32) queued candidates, one per lane: the candidate's
+    // m (<= 32) queued candidates from entry h on, one per lane: the candidate's
     // stream at this step (block 0) draws its next free flight (word 0) and
     // the real/null test (word 1 against the total rate at the particle's
     // energy; ions: relative to a target from the gas Maxwellian); records go
     // to the warp's list in slot order, two uint4 each: electrons {slot, id,
     // x, vx}{vy, vz, -, -}, ions {slot, id, vx, vy}{vz, w1, w2, w3} (the real
     // collisions; with the ion filter in its own kernel, every ion candidate).
-    auto flush = [&](unsigned m) {
+    auto flush = [&](unsigned h, unsigned m) {
         const bool has = (unsigned)lane < m;
-        const unsigned slot = has ? qs[lane] : 0u;
-        const float cx = has ? qx[lane] : 0.0f, cvx = has ? qv[lane] : 0.0f;
+        const unsigned slot = has ? qs[h + lane] : 0u;
         uint32_t id = 0u;
-        float cvy = 0.0f, cvz = 0.0f;
-        if (has) { id = ID[slot]; cvy = VY[slot]; cvz = VZ[slot]; }
+        float cx = 0.0f, cvx = 0.0f, cvy = 0.0f, cvz = 0.0f;
+        if (has) {
+            id = ID[slot]; cvx = VX[slot]; cvy = VY[slot]; cvz = VZ[slot];   // (x, v_x: as this warp just stored them)
+            if (S == SP_E) cx = X[slot];
+        }
         bool rec = false;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         if (has) {
@@ -527,7 +583,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         }
         const unsigned cm = __ballot_sync(0xffffffffu, rec);
         if (rec) {
-            const size_t q = r0 + nrec + __popc(cm & lt_mask);
+            const size_t q = rec0 + nrec + __popc(cm & lt_mask);
             if (S == SP_E) {
                 CAND[2 * q] = make_uint4(slot, id, __float_as_uint(cx), __float_as_uint(cvx));
                 CAND[2 * q + 1] = make_uint4(__float_as_uint(cvy), __float_as_uint(cvz), 0u, 0u);
@@ -539,70 +595,116 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         nrec += __popc(cm);
     };
 
-    for (unsigned g0 = r0; g0 < r1; g0 += ROUND) {
-        if (g0 != r0) load_round(g0);
-#pragma unroll PUSH_UNROLL
+    for (unsigned g0 = ga; g0 < gz; g0 += stride) {
+        float xn[4], vxn[4];
+        uint32_t tcn[4];
+        if (g0 + stride < gz) load_round(g0 + stride, xn, vxn, tcn);   // in flight meanwhile
+        const unsigned i0 = g0 + 4u * lane;
+        // the four slots without branches (a dead slot's NaN falls through the
+        // arithmetic and takes part in nothing); what is rare is flagged and
+        // handled once per round: bit k of `out`: the particle left the gap,
+        // `wide`: its current term does not fit 32 bits, `wrap`: its weight
+        // sum wrapped, `cand`: its free flight ends at this step
+        unsigned cand = 0u, out = 0u, wide = 0u, wrap = 0u;
+#pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const unsigned i = g0 + 32u * k + lane;
             float x = xs[k], vx = vxs[k];
-            bool cand = false;
-            int dcell = -1;                  // cell deposited into (-1: none)
-            unsigned long long dval = 0ull;
-            if (!is_dead(x)) {
-                int j; float frac;
-                cell_of(x, inv_dx, Nc, j, frac);
-                const float Ep = fmaf(frac, Es[j + 1] - Es[j], Es[j]);
-                vx = fmaf(qmdt, Ep, vx);
-                x = fmaf(vx, dts, x);
+            const bool live = !is_dead(x);
+            int j; float frac;
+            cell_of_inside(x, inv_dx, jmax, j, frac);
+            const float Ep = fmaf(frac, Es[j + 1] - Es[j], Es[j]);
+            vx = fmaf(qmdt, Ep, vx);
+            x = fmaf(vx, dts, x);
+            // exact scaling by 2^8, then truncation
+            const float jv = vx * 256.0f;
+            if (live) {
                 ++psteps;
-                jacc += (long long)(vx * 256.0f);   // exact scaling by 2^8, then truncation
-                if (x < 0.0f) { ++nabs0; x = dead_marker(); }
-                else if (x >= Lf) { ++nabs1; x = dead_marker(); }
-                else if (!(x >= 0.0f) || !isfinite(vx)) { ++nnf; x = dead_marker(); }
-                else {
-                    // CIC deposit as (count, sum of r) per cell: node c gets
-                    // 2^16 count_c - rsum_c, node c+1 gets rsum_c
-                    int j2; float f2;
-                    cell_of(x, inv_dx, Nc, j2, f2);
-                    dcell = j2;
-                    dval = (1ull << 40) + (unsigned long long)cic_r(f2);
-                    if (!O2PIC_DEPOSIT_AGG) atomicAdd(&hist[j2], dval);
-                    // its free flight ends at this step: a collision candidate
-                    cand = (np > 0) && (tcs[k] == step_lo);
+                jacc += (long long)__float2int_rz(jv);
+                if (!(fabsf(jv) < 2147483648.0f)) wide |= 1u << k;
+            }
+            if (x >= 0.0f && x < Lf) {
+                // (a finite x here has a finite v_x.)  CIC deposit as (count,
+                // sum of r) per cell: node c gets 2^16 count_c - rsum_c, node
+                // c+1 gets rsum_c
+                int j2; float f2;
+                cell_of_inside(x, inv_dx, jmax, j2, f2);
+                const uint32_t r = cic_r_inside(f2);
+                atomicAdd(&cnt[j2], 1u);
+                const unsigned old = atomicAdd(&rsum[j2], r);
+                if (old + r < old) wrap |= 1u << k;
+                if (tcs[k] == step_lo) cand |= 1u << k;
+            } else if (live) {
+                out |= 1u << k;
+            }
+            xs[k] = x;
+            vxs[k] = vx;
+        }
+        if (out | wide | wrap) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if ((wide >> k) & 1u) {
+                    const float jv = vxs[k] * 256.0f;
+                    jacc += trunc_s64_large(jv) - (long long)__float2int_rz(jv);
                 }
-                X[i] = x;
-                VX[i] = vx;
+                if ((wrap >> k) & 1u) {
+                    int j2; float f2;
+                    cell_of_inside(xs[k], inv_dx, jmax, j2, f2);
+                    weight_wrapped(Qcopy, j2, 1);
+                }
+                if ((out >> k) & 1u) {
+                    if (xs[k] < 0.0f) ++nabs0;
+                    else if (xs[k] >= Lf) ++nabs1;
+                    else ++nnf;
+                    xs[k] = dead_marker();
+                }
             }
-            if (O2PIC_DEPOSIT_AGG) {
-                // the lanes of one cell add their values (peer by peer, in
-                // lane order) and the lowest of them adds the sum
-                const unsigned peers = __match_any_sync(0xffffffffu, dcell);
-                unsigned long long sum = 0ull;
-                for (unsigned m = peers; m; m &= m - 1u) sum += __shfl_sync(peers, dval, __ffs(m) - 1);
-                if (dcell >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[dcell], sum);
+        }
+        if (g0 + ROUND <= gz) {
+            *reinterpret_cast<float4*>(X + i0) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+            *reinterpret_cast<float4*>(VX + i0) = make_float4(vxs[0], vxs[1], vxs[2], vxs[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i0 + k < gz) { X[i0 + k] = xs[k]; VX[i0 + k] = vxs[k]; }
+        }
+        const unsigned some = np > 0 ? __ballot_sync(0xffffffffu, cand != 0u) : 0u;
+        if (some) {
+            // queue them in slot order (lane by lane, four slots each); most
+            // rounds have at most one in a lane
+            if (!__any_sync(0xffffffffu, (cand & (cand - 1u)) != 0u)) {
+                if (cand) qs[qn + __popc(some & lt_mask)] = i0 + (unsigned)__ffs(cand) - 1u;
+                qn += __popc(some);
+            } else {
+                unsigned below = 0u, all = 0u;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned b = __ballot_sync(0xffffffffu, (cand >> k) & 1u);
+                    below += __popc(b & lt_mask);
+                    all += __popc(b);
+                }
+                unsigned q = qn + below;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((cand >> k) & 1u) qs[q++] = i0 + k;
+                qn += all;
             }
-            const unsigned cm = __ballot_sync(0xffffffffu, cand);
-            if (cand) {
-                const unsigned q = qn + __popc(cm & lt_mask);
-                qs[q] = i; qx[q] = x; qv[q] = vx;
-            }
-            qn += __popc(cm);
             if (qn >= 32u) {
                 __syncwarp();
-                flush(32u);
-                const unsigned rest = qn - 32u;    // < 32: lane q moves entry 32 + q
-                unsigned s0 = 0u;
-                float x0 = 0.0f, v0 = 0.0f;
-                if ((unsigned)lane < rest) { s0 = qs[32 + lane]; x0 = qx[32 + lane]; v0 = qv[32 + lane]; }
+                unsigned h = 0u;
+                do { flush(h, 32u); h += 32u; } while (qn - h >= 32u);
+                const unsigned rest = qn - h;      // < 32: lane q moves entry h + q
+                const unsigned s0 = ((unsigned)lane < rest) ? qs[h + lane] : 0u;
                 __syncwarp();
-                if ((unsigned)lane < rest) { qs[lane] = s0; qx[lane] = x0; qv[lane] = v0; }
+                if ((unsigned)lane < rest) qs[lane] = s0;
                 qn = rest;
                 __syncwarp();
             }
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { xs[k] = xn[k]; vxs[k] = vxn[k]; tcs[k] = tcn[k]; }
     }
     __syncwarp();
-    if (qn > 0u) flush(qn);
+    if (qn > 0u) flush(0u, qn);
     unsigned nrm = 0;
     if (fused) {
         // the real collisions, by the warp that recorded them (its lanes'
@@ -612,8 +714,8 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         // counted the warnings of the part it shares with the kinematics.
         __syncwarp();
         unsigned nb1 = 0, nb2 = 0, wt2 = 0, we2 = 0;
-        collide_list<S, 32>(P, cum, pre, step, r0, nrec, nrec, (unsigned)lane, 0xffffffffu, lt_mask, sh.events, hist,
-                            nb1, nb2, nrm, wt2, we2);
+        collide_list<S, 32>(P, cum, pre, step, rec0, nrec, nrec, (unsigned)lane, 0xffffffffu, lt_mask, sh.events, cnt,
+                            rsum, Qcopy, nb1, nb2, nrm, wt2, we2);
         wtries += wt2;
         if (P.births_possible[S] && lane == 0) {
             if (S == SP_E) {
@@ -640,14 +742,12 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     if (wnumax) atomicAdd(&C->cnt.warn_numax, (unsigned long long)wnumax);
     __syncthreads();
     if (fused && tid < np && sh.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)sh.events[tid]);
-    unsigned long long* __restrict__ Qcopy = P.Qf[S] + (size_t)(blk & (QCOPIES - 1)) * Ng;
-    for (int c = tid; c < Nc; c += BLOCK) {
-        const unsigned long long v = hist[c];
-        if (v) {
-            const unsigned long long count = v >> 40, rsum = v & ((1ull << 40) - 1);
-            atomicAdd(&Qcopy[c], (count << 16) - rsum);
-            if (rsum) atomicAdd(&Qcopy[c + 1], rsum);
-        }
+    // one 64-bit add per node: what its two cells give it
+    for (int j = tid; j < Ng; j += BLOCK) {
+        unsigned long long v = 0ull;
+        if (j < Nc) v = ((unsigned long long)cnt[j] << 16) - rsum[j];
+        if (j > 0) v += rsum[j - 1];
+        if (v) atomicAdd(&Qcopy[j], v);
     }
     if (tid == 0) {
         if (sh.absorbed[0]) atomicAdd(&C->cnt.absorbed[S][0], (unsigned long long)sh.absorbed[0]);
@@ -711,11 +811,10 @@ __device__ __forceinline__ void filter_body(const Params& P, unsigned blk, unsig
     const unsigned nslots = (unsigned)((C->slots[S] < P.sp[S].cap) ? C->slots[S] : P.sp[S].cap);
     uint4* CAND = P.cand[S];
     const unsigned W = P.push_warps[S];
-    const unsigned R = warp_range_len(nslots, W);
     const float numax = P.numax[S], kap = P.kappa[S], sig = P.sig_gas;
     unsigned wtries = 0, wemax = 0, wnumax = 0;
     for (unsigned gw = blk * WARPS + warp; gw < W; gw += nblk * WARPS) {
-        const unsigned r0 = (gw * (unsigned long long)R < nslots) ? gw * R : nslots;
+        const unsigned r0 = list_start<S>(gw, W, nslots);
         const unsigned n = P.ccount[S][gw];
         unsigned nreal = 0;   // warp-uniform
         for (unsigned c0 = 0; c0 < n; c0 += 64) {
@@ -800,19 +899,18 @@ __device__ __forceinline__ void cand_body(const Params& P, unsigned blk, unsigne
     unsigned* cnt1 = (S == SP_E) ? P.wcount[B_E_FROM_E] : nullptr;
     unsigned* cnt2 = (S == SP_E) ? P.wcount[B_OM_FROM_E] : (S == SP_OM ? P.wcount[B_E_FROM_OM] : nullptr);
     const unsigned W = P.push_warps[S];
-    const unsigned R = warp_range_len(nslots, W);
     const PhiloxPre pre = philox_pre((uint32_t)step, SpeciesTraits<S>::tag, (uint32_t)(step >> 32), P.seed);
     unsigned wtries = 0, wemax = 0, nremoved = 0;
 
     for (unsigned gb = (blk * WARPS + warp) * SEGS; gb < W; gb += nblk * WARPS * SEGS) {
         const unsigned gw = gb + seg;                  // this half-warp's list
         const bool valid = gw < W;
-        const unsigned r0 = !valid ? 0u : ((gw * (unsigned long long)R < nslots) ? gw * R : nslots);
+        const unsigned r0 = valid ? list_start<S>(gw, W, nslots) : 0u;
         const unsigned n = valid ? P.ccount[S][gw] : 0u;
         const unsigned nmax = max(n, __shfl_xor_sync(0xffffffffu, n, SEG));
         unsigned nb1 = 0, nb2 = 0;   // half-warp-uniform
-        collide_list<S, SEG>(P, P.cum[S], pre, step, r0, n, nmax, sl, seg_mask, lt_mask, events, nullptr, nb1, nb2,
-                             nremoved, wtries, wemax);
+        collide_list<S, SEG>(P, P.cum[S], pre, step, r0, n, nmax, sl, seg_mask, lt_mask, events, nullptr, nullptr,
+                             nullptr, nb1, nb2, nremoved, wtries, wemax);
         if (births && valid && sl == 0) {
             if (cnt1) cnt1[gw] = nb1;
             if (cnt2) cnt2[gw] = nb2;
@@ -927,8 +1025,7 @@ __global__ void __launch_bounds__(BLOCK) k_deposit(Params P) {
 }  // namespace
 
 size_t push_smem_bytes(int species, const Params& P) {
-    const size_t base = align16(align16(sizeof(PushShared)) + sizeof(float) * P.Ng) +
-                        sizeof(unsigned long long) * P.Ng + sizeof(PushQueue);
+    const size_t base = align16(sizeof(PushShared)) + (sizeof(float) + 2 * sizeof(unsigned)) * P.Ng + sizeof(PushQueue);
     if (!(species == SP_E || O2PIC_FUSE_IONS)) return base;
     const size_t table = P.cum_smem[species] ? sizeof(float) * NGRID * (size_t)P.nproc[species] : 0;
     return base + sizeof(float) * NGRID + table;

@@ -494,6 +494,9 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
         float* cum;
         TRY(ctx_alloc(c, &cum, (size_t)NGRID * MAXPROC));
         P.cum[s] = cum;
+        float* tot;
+        TRY(ctx_alloc(c, &tot, NGRID));
+        P.tot[s] = tot;
         TRY(ctx_alloc(c, &P.Q[s], Ng));
         TRY(ctx_alloc(c, &P.Qf[s], (size_t)QCOPIES * Ng));
         TRY(ctx_alloc(c, &P.Qb[s], Ng));
@@ -686,6 +689,10 @@ int o2pic_set_processes(o2pic_ctx* c, const o2pic_process* procs, int nproc) {
             e = cudaMemcpy((void*)P.cum[s], cum.data(), sizeof(float) * cum.size(), cudaMemcpyHostToDevice);
             if (e != cudaSuccess) return cuda_fail(c, e);
         }
+        std::vector<float> tot(NGRID, 0.0f);
+        for (int i = 0; i < NGRID && np > 0; ++i) tot[i] = cum[(size_t)i * np + np - 1];
+        e = cudaMemcpy((void*)P.tot[s], tot.data(), sizeof(float) * NGRID, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_fail(c, e);
     }
     std::vector<float> K(NGRID, 0.0f);
     float kmax = 0.0f;
