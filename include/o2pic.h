@@ -302,7 +302,7 @@ int o2pic_compact_particles(const float* x, const float* vx, const float* vy, co
                             uint32_t* oid, uint64_t* n_out, void* stream);
 
 /* Failure detection of the bounded device waits: runs the decoupled
- * look-back wait that the compaction kernels use (one thread waiting, as tile
+ * look-back wait that the compaction kernels use (one warp waiting, as tile
  * 1, for a tile 0 whose flag nothing ever sets) on `stream`.  The wait must
  * give up after its spin limit, record the timeout and return, so that the
  * context stays usable; *seconds (may be NULL) gets the kernel's duration.

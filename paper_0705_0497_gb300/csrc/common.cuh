@@ -276,13 +276,7 @@ __device__ __forceinline__ void load_params(Params& dst, const Params* src) {
     __syncthreads();
 }
 
-// ------------------------------------------------------- decoupled look-back
-// Per tile: a flag word = (epoch << 2) | state (1 = aggregate published,
-// 2 = inclusive prefix published) and two value words (val[2t] = aggregate,
-// val[2t+1] = inclusive prefix), each holding two 32-bit counts.  A value is
-// stored before its flag (release) and read after the flag (acquire); the
-// aggregate word is never rewritten, so a reader that saw state 1 reads the
-// aggregate even if the tile has meanwhile published its prefix.
+// ------------------------------------------------ ordered loads and stores
 __device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -298,59 +292,6 @@ __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long lon
 }
 __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long pack2(unsigned a, unsigned b) {
-    return (unsigned long long)a | ((unsigned long long)b << 32);
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long x, unsigned long long y) {
-    return pack2((unsigned)x + (unsigned)y, (unsigned)(x >> 32) + (unsigned)(y >> 32));
-}
-
-// Called by one thread.  Publishes the tile's aggregate, walks back to the
-// nearest inclusive prefix, publishes its own inclusive prefix and returns
-// the exclusive prefix.  Tiles are claimed in increasing order by running
-// blocks, so every predecessor is being processed; the wait is still bounded:
-// on giving up the error flag is set, *ok = false and the caller skips its
-// writes.
-constexpr unsigned LOOKBACK_SPIN_LIMIT = 1u << 22;
-
-__device__ __forceinline__ unsigned long long lookback(unsigned long long* flag, unsigned long long* val,
-                                                       unsigned tile, unsigned long long agg,
-                                                       unsigned long long epoch, unsigned long long* err,
-                                                       bool* ok) {
-    *ok = true;
-    if (tile == 0) {
-        st_relaxed(&val[1], agg);
-        st_release(&flag[0], (epoch << 2) | 2ull);
-        return 0ull;
-    }
-    st_relaxed(&val[2 * tile], agg);
-    st_release(&flag[tile], (epoch << 2) | 1ull);
-    unsigned long long excl = 0ull;
-    unsigned spins = 0;
-    int j = (int)tile - 1;
-    while (j >= 0) {
-        const unsigned long long f = ld_acquire(&flag[j]);
-        if ((f >> 2) != epoch) {
-            if (++spins > LOOKBACK_SPIN_LIMIT) {
-                atomicOr(err, ERR_TIMEOUT);
-                *ok = false;
-                return 0ull;
-            }
-            if (spins > 64) __nanosleep(64);
-            continue;
-        }
-        if ((f & 3ull) == 2ull) {
-            excl = add2(excl, ld_relaxed(&val[2 * j + 1]));
-            break;
-        }
-        excl = add2(excl, ld_relaxed(&val[2 * j]));
-        --j;
-    }
-    st_relaxed(&val[2 * tile + 1], add2(excl, agg));
-    st_release(&flag[tile], (epoch << 2) | 2ull);
-    return excl;
 }
 
 }  // namespace o2

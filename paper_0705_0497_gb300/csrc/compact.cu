@@ -1,90 +1,47 @@
 // Stable compaction of a caller's particle arrays (the removal half of the
 // method's births/removal step): particles whose x is NaN (the library's
 // marker of a removed particle) are dropped, the others are written in their
-// original order to the output arrays.  One pass over tiles of TILE
-// particles claimed in increasing order; each tile's live count is combined
-// with the earlier tiles' by a decoupled look-back.  The look-back state and
-// the tile ticket are the kernel's scratch memory.
-#include "common.cuh"
+// original order to the output arrays (compact_tiles).  The look-back state
+// and the tile ticket are the kernel's scratch memory.
+#include "compact.cuh"
 
 namespace o2 {
 
 namespace {
 
-__global__ void __launch_bounds__(BLOCK) k_compact_arrays(const float* __restrict__ X, const float* __restrict__ VX,
-                                                          const float* __restrict__ VY, const float* __restrict__ VZ,
-                                                          const uint32_t* __restrict__ ID, unsigned long long n,
-                                                          float* OX, float* OVX, float* OVY, float* OVZ, uint32_t* OID,
-                                                          unsigned long long* n_out, unsigned long long* ticket,
-                                                          unsigned long long* count, unsigned long long* flag,
-                                                          unsigned long long* val, unsigned long long epoch,
-                                                          unsigned long long* err) {
-    __shared__ unsigned ws[32];
-    __shared__ unsigned sh_tile;
-    __shared__ unsigned long long sh_excl;
-    __shared__ int sh_ok;
-    const unsigned ntiles = (unsigned)ceil_div(n, TILE);
-    const int tid = threadIdx.x;
-    for (;;) {
-        if (tid == 0) sh_tile = (unsigned)atomicAdd(ticket, 1ull);
-        __syncthreads();
-        const unsigned tile = sh_tile;
-        __syncthreads();
-        if (tile >= ntiles) break;
-        const unsigned long long base = (unsigned long long)tile * TILE;
-        const unsigned long long end = (base + TILE < n) ? base + TILE : n;
-        unsigned cnt = 0;
-        for (int c = 0; c < CHUNKS_PER_TILE; ++c) {
-            const unsigned long long i0 = base + (unsigned long long)c * CHUNK + 4ull * tid;
+__global__ void __launch_bounds__(CMP_T, 2) k_compact_arrays(const float* __restrict__ X, const float* __restrict__ VX,
+                                                            const float* __restrict__ VY, const float* __restrict__ VZ,
+                                                            const uint32_t* __restrict__ ID, unsigned long long n,
+                                                            float* OX, float* OVX, float* OVY, float* OVZ,
+                                                            uint32_t* OID, unsigned long long* n_out,
+                                                            unsigned long long* ticket, unsigned long long* count,
+                                                            unsigned long long* flag, unsigned long long* val,
+                                                            unsigned long long epoch, unsigned long long* err) {
+    __shared__ CompactShared sh;
+    compact_tiles(
+        sh, X, n, reinterpret_cast<unsigned*>(ticket), flag, val, epoch, err,
+        [&](unsigned long long p) {
+            prefetch_l2(VX + p); prefetch_l2(VY + p); prefetch_l2(VZ + p); prefetch_l2(ID + p);
+        },
+        [&](const float (&x)[CMP_I], unsigned long long base, unsigned long long d, const unsigned (&off)[CMP_I],
+            unsigned in) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + k < end && !is_dead(X[i0 + k])) ++cnt;
-        }
-        unsigned tile_total;
-        (void)block_excl_scan<BLOCK>(cnt, ws, &tile_total);
-        if (tid == 0) {
-            bool ok;
-            sh_excl = lookback(flag, val, tile, pack2(tile_total, 0u), epoch, err, &ok);
-            sh_ok = ok ? 1 : 0;
-            if (ok && tile == ntiles - 1) {
-                const unsigned long long total = (unsigned)sh_excl + (unsigned long long)tile_total;
-                *count = total;
-                *n_out = total;
-            }
-        }
-        __syncthreads();
-        if (sh_ok) {
-            unsigned long long run = (unsigned)sh_excl;
-            for (int c = 0; c < CHUNKS_PER_TILE; ++c) {
-                const unsigned long long i0 = base + (unsigned long long)c * CHUNK + 4ull * tid;
-                unsigned m = 0;
-                bool lv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { lv[k] = (i0 + k < end) && !is_dead(X[i0 + k]); m += lv[k] ? 1u : 0u; }
-                unsigned ctot;
-                const unsigned off = block_excl_scan<BLOCK>(m, ws, &ctot);
-                unsigned long long d = run + off;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (!lv[k]) continue;
-                    OX[d] = X[i0 + k]; OVX[d] = VX[i0 + k]; OVY[d] = VY[i0 + k]; OVZ[d] = VZ[i0 + k];
-                    OID[d] = ID[i0 + k];
-                    ++d;
-                }
-                run += ctot;
-            }
-        }
-        __syncthreads();
-    }
+            for (int i = 0; i < CMP_I; ++i)
+                if ((in >> i) & 1u) OX[d + off[i]] = x[i];
+            move_array(OVX, VX, base, d, off, in, ~0ull);
+            move_array(OVY, VY, base, d, off, in, ~0ull);
+            move_array(OVZ, VZ, base, d, off, in, ~0ull);
+            move_array(OID, ID, base, d, off, in, ~0ull);
+        },
+        [&](unsigned long long kept) { *count = kept; *n_out = kept; });
 }
 
-// One thread waits, as tile 1 of a look-back, for tile 0, whose flag nothing
+// One warp waits, as tile 1 of a look-back, for tile 0, whose flag nothing
 // ever sets (epoch 1 against the zeroed flag): the bounded wait must give up,
 // set the timeout bit and return.  words = [err, flag[2], val[4]].
 __global__ void k_lookback_probe(unsigned long long* words) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     bool ok;
-    (void)lookback(words + 1, words + 3, 1u, pack2(1u, 0u), 1ull, words, &ok);
+    (void)lookback(words + 1, words + 3, 1u, 1ull, 1ull, words, &ok);
 }
 
 }  // namespace
@@ -98,8 +55,10 @@ size_t compact_scratch_words(unsigned long long n) {
 void launch_compact_arrays(const float* x, const float* vx, const float* vy, const float* vz, const uint32_t* id,
                            unsigned long long n, float* ox, float* ovx, float* ovy, float* ovz, uint32_t* oid,
                            unsigned long long* n_out, unsigned long long* words, unsigned long long tiles,
-                           unsigned long long epoch, int grid, cudaStream_t s) {
-    k_compact_arrays<<<grid, BLOCK, 0, s>>>(x, vx, vy, vz, id, n, ox, ovx, ovy, ovz, oid, n_out, &words[0], &words[1],
+                           unsigned long long epoch, int sms, cudaStream_t s) {
+    // two blocks per SM are resident; fewer where there are fewer tiles
+    const int grid = (int)(ceil_div(n, TILE) < 2ull * sms ? ceil_div(n, TILE) : 2ull * sms);
+    k_compact_arrays<<<grid, CMP_T, 0, s>>>(x, vx, vy, vz, id, n, ox, ovx, ovy, ovz, oid, n_out, &words[0], &words[1],
                                             &words[3], &words[3 + tiles], epoch, &words[2]);
 }
 
@@ -153,7 +112,7 @@ extern "C" int o2pic_compact_particles(const float* x, const float* vx, const fl
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && n > 0) {
         launch_compact_arrays(x, vx, vy, vz, id, n, ox, ovx, ovy, ovz, oid, (unsigned long long*)n_out, scratch, tiles,
-                              1ull, 4 * sms, s);
+                              1ull, sms, s);
         e = cudaGetLastError();
     }
     unsigned long long err = 0;

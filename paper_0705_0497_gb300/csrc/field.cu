@@ -20,7 +20,7 @@
 // only rounding is in the final FP64 expressions, each evaluated in the order
 // written here.  |S| <= 2^47 and |T| <= 2^58 for up to 2^31 particles and 8192
 // cells, so int64 holds both exactly.
-#include "common.cuh"
+#include "compact.cuh"
 
 namespace o2 {
 
@@ -495,115 +495,41 @@ __device__ __forceinline__ void field_body(const Params& P, int mode, int pushed
     }
 }
 
-// Stable compaction of the live slots of one species into the other buffer
-// (mode 0, when more than a fraction of the slots is dead), or a stable copy
-// of the live particles into caller buffers (mode 1).  Tiles of TILE slots in
-// increasing order, decoupled look-back on the live counts.
-template <int S>
-__device__ __forceinline__ void compact_body(const Params& P, int mode, unsigned long long epoch_arg,
-                                             unsigned* ticket_arg, unsigned long long* flag_arg,
-                                             unsigned long long* val_arg, float* ox, float* ovx, float* ovy,
-                                             float* ovz, uint32_t* oid, uint32_t* otc, unsigned long long ocap,
-                                             unsigned long long* out_count) {
-    __shared__ unsigned ws[32];
-    __shared__ unsigned sh_tile;
-    __shared__ unsigned long long sh_excl;
-    __shared__ int sh_ok;
+// Stable compaction of the live slots of one species into the other buffer,
+// when more than a fraction of the slots is dead.
+__device__ __forceinline__ void compact_body(const Params& P, int S, CompactShared& sh) {
     DevCtrl* C = P.ctrl;
     const unsigned long long nslots = C->slots[S];
     const unsigned long long live = C->live[S];
-    if (mode == 0) {
-        const unsigned long long dead = nslots - live;
-        const bool many_dead = (double)dead > (double)P.compact_dead_frac * (double)nslots;
-        const bool near_full = dead > 0 && 4 * nslots > 3 * P.sp[S].cap;
-        if (!many_dead && !near_full) return;
-    }
-    const unsigned cb = C->cur[S];
-    const float* X = P.sp[S].x[cb];
-    const float* VX = P.sp[S].vx[cb];
-    const float* VY = P.sp[S].vy[cb];
-    const float* VZ = P.sp[S].vz[cb];
-    const uint32_t* ID = P.sp[S].id[cb];
-    const uint32_t* TCS = P.sp[S].tc[cb];
-    float *DX, *DVX, *DVY, *DVZ; uint32_t *DID, *DTC;
-    unsigned long long dcap;
-    unsigned* ticket; unsigned long long *flag, *val, epoch;
-    if (mode == 0) {
-        DX = P.sp[S].x[cb ^ 1u]; DVX = P.sp[S].vx[cb ^ 1u]; DVY = P.sp[S].vy[cb ^ 1u]; DVZ = P.sp[S].vz[cb ^ 1u];
-        DID = P.sp[S].id[cb ^ 1u]; DTC = P.sp[S].tc[cb ^ 1u]; dcap = P.sp[S].cap;
-        ticket = &C->ticket[NKK + S];
-        flag = P.lb_flag[KK_COMPACT]; val = P.lb_val[KK_COMPACT];
-        epoch = (C->epoch << 2) | (unsigned long long)S;
-    } else {
-        DX = ox; DVX = ovx; DVY = ovy; DVZ = ovz; DID = oid; DTC = otc; dcap = ocap;
-        ticket = ticket_arg; flag = flag_arg; val = val_arg; epoch = epoch_arg;
-    }
-    const unsigned ntiles = (unsigned)ceil_div(nslots, TILE);
-    const int tid = threadIdx.x;
-    for (;;) {
-        if (tid == 0) sh_tile = atomicAdd(ticket, 1u);
-        __syncthreads();
-        const unsigned tile = sh_tile;
-        __syncthreads();
-        if (tile >= ntiles) break;
-        const unsigned long long base = (unsigned long long)tile * TILE;
-        const unsigned long long end = (base + TILE < nslots) ? base + TILE : nslots;
-        // pass 1: live count of the tile
-        unsigned cnt = 0;
-        for (int c = 0; c < CHUNKS_PER_TILE; ++c) {
-            const unsigned long long i0 = base + (unsigned long long)c * CHUNK + 4ull * tid;
+    const unsigned long long dead = nslots - live;
+    const bool many_dead = (double)dead > (double)P.compact_dead_frac * (double)nslots;
+    const bool near_full = dead > 0 && 4 * nslots > 3 * P.sp[S].cap;
+    if (!many_dead && !near_full) return;
+    const SpeciesBuf& B = P.sp[S];
+    const unsigned cb = C->cur[S], nb = cb ^ 1u;
+    const unsigned long long cap = B.cap;
+    compact_tiles(
+        sh, B.x[cb], nslots, &C->ticket[NKK + S], P.lb_flag[S], P.lb_val[S], C->epoch, &C->error_flags,
+        [&](unsigned long long p) {
+            prefetch_l2(B.vx[cb] + p); prefetch_l2(B.vy[cb] + p); prefetch_l2(B.vz[cb] + p);
+            prefetch_l2(B.id[cb] + p); prefetch_l2(B.tc[cb] + p);
+        },
+        [&](const float (&x)[CMP_I], unsigned long long base, unsigned long long d, const unsigned (&off)[CMP_I],
+            unsigned in) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + k < end && !is_dead(X[i0 + k])) ++cnt;
-        }
-        unsigned tile_total;
-        (void)block_excl_scan<BLOCK>(cnt, ws, &tile_total);
-        if (tid == 0) {
-            bool ok;
-            sh_excl = lookback(flag, val, tile, pack2(tile_total, 0u), epoch, &C->error_flags, &ok);
-            sh_ok = ok ? 1 : 0;
-            if (ok && tile == ntiles - 1) {
-                const unsigned long long total = (unsigned)sh_excl + (unsigned long long)tile_total;
-                if (mode == 0) {
-                    C->slots[S] = total;
-                    C->live[S] = total;
-                    C->cur[S] = cb ^ 1u;
-                } else {
-                    *out_count = total;
-                }
-            }
-        }
-        __syncthreads();
-        if (sh_ok) {
-            // pass 2: destinations in slot order, chunk by chunk in (thread, k) order
-            unsigned long long run = (unsigned)sh_excl;
-            for (int c = 0; c < CHUNKS_PER_TILE; ++c) {
-                const unsigned long long i0 = base + (unsigned long long)c * CHUNK + 4ull * tid;
-                unsigned m = 0;
-                bool lv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { lv[k] = (i0 + k < end) && !is_dead(X[i0 + k]); m += lv[k] ? 1u : 0u; }
-                unsigned ctot;
-                const unsigned off = block_excl_scan<BLOCK>(m, ws, &ctot);
-                unsigned long long d = run + off;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (!lv[k]) continue;
-                    if (d < dcap) {
-                        // a gather (mode 1) may ask for the flights only
-                        if (DX) {
-                            DX[d] = X[i0 + k]; DVX[d] = VX[i0 + k]; DVY[d] = VY[i0 + k]; DVZ[d] = VZ[i0 + k];
-                            DID[d] = ID[i0 + k];
-                        }
-                        if (DTC) DTC[d] = TCS[i0 + k];
-                    }
-                    ++d;
-                }
-                run += ctot;
-            }
-        }
-        __syncthreads();
-    }
+            for (int i = 0; i < CMP_I; ++i)
+                if (((in >> i) & 1u) && d + off[i] < cap) B.x[nb][d + off[i]] = x[i];
+            move_array(B.vx[nb], B.vx[cb], base, d, off, in, cap);
+            move_array(B.vy[nb], B.vy[cb], base, d, off, in, cap);
+            move_array(B.vz[nb], B.vz[cb], base, d, off, in, cap);
+            move_array(B.id[nb], B.id[cb], base, d, off, in, cap);
+            move_array(B.tc[nb], B.tc[cb], base, d, off, in, cap);
+        },
+        [&](unsigned long long kept) {
+            C->slots[S] = kept;
+            C->live[S] = kept;
+            C->cur[S] = nb;
+        });
 }
 
 __global__ void __launch_bounds__(FT) k_field(Params P, int mode, int pushed_mask) {
@@ -621,23 +547,55 @@ __global__ void __launch_bounds__(FT) k_field_b(const Params* __restrict__ all, 
     field_body(sP, mode, pushed_mask, (int)(blockIdx.x & 1u));
 }
 
-template <int S>
-__global__ void __launch_bounds__(BLOCK) k_compact(Params P, int mode, unsigned long long epoch_arg, unsigned* ticket_arg,
-                                                   unsigned long long* flag_arg, unsigned long long* val_arg, float* ox,
-                                                   float* ovx, float* ovy, float* ovz, uint32_t* oid, uint32_t* otc,
-                                                   unsigned long long ocap, unsigned long long* out_count) {
+// The compaction check of all species: blockIdx.y is the species.
+__global__ void __launch_bounds__(CMP_T, 2) k_compact(Params P) {
+    __shared__ CompactShared sh;
     pdl_wait();
-    compact_body<S>(P, mode, epoch_arg, ticket_arg, flag_arg, val_arg, ox, ovx, ovy, ovz, oid, otc, ocap, out_count);
+    compact_body(P, (int)blockIdx.y, sh);
 }
 
-// batched compaction check (mode 0): the blocks of map[b].x claim that
-// discharge's tiles by its own ticket
-template <int S>
-__global__ void __launch_bounds__(BLOCK) k_compact_b(const Params* __restrict__ all, const uint4* __restrict__ map) {
-    __shared__ Params sP;
+// batched: the blocks of map[b].x claim that discharge's tiles of species
+// map[b].w by its own ticket
+__global__ void __launch_bounds__(CMP_T, 2) k_compact_b(const Params* __restrict__ all, const uint4* __restrict__ map) {
+    __shared__ CompactShared sh;
     pdl_wait();
-    load_params(sP, all + map[blockIdx.x].x);
-    compact_body<S>(sP, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr);
+    const uint4 m = map[blockIdx.x];
+    compact_body(all[m.x], (int)m.w, sh);
+}
+
+// Stable copy of the live particles of a species into caller buffers (a
+// caller may ask for the flights alone).
+__global__ void __launch_bounds__(CMP_T, 2) k_gather(Params P, int S, unsigned long long epoch, unsigned* ticket,
+                                                     unsigned long long* flag, unsigned long long* val, float* ox,
+                                                     float* ovx, float* ovy, float* ovz, uint32_t* oid, uint32_t* otc,
+                                                     unsigned long long ocap, unsigned long long* out_count) {
+    __shared__ CompactShared sh;
+    DevCtrl* C = P.ctrl;
+    const SpeciesBuf& B = P.sp[S];
+    const unsigned cb = C->cur[S];
+    compact_tiles(
+        sh, B.x[cb], C->slots[S], ticket, flag, val, epoch, &C->error_flags,
+        [&](unsigned long long p) {
+            if (ox) {
+                prefetch_l2(B.vx[cb] + p); prefetch_l2(B.vy[cb] + p); prefetch_l2(B.vz[cb] + p);
+                prefetch_l2(B.id[cb] + p);
+            }
+            if (otc) prefetch_l2(B.tc[cb] + p);
+        },
+        [&](const float (&x)[CMP_I], unsigned long long base, unsigned long long d, const unsigned (&off)[CMP_I],
+            unsigned in) {
+            if (ox) {
+#pragma unroll
+                for (int i = 0; i < CMP_I; ++i)
+                    if (((in >> i) & 1u) && d + off[i] < ocap) ox[d + off[i]] = x[i];
+                move_array(ovx, B.vx[cb], base, d, off, in, ocap);
+                move_array(ovy, B.vy[cb], base, d, off, in, ocap);
+                move_array(ovz, B.vz[cb], base, d, off, in, ocap);
+                move_array(oid, B.id[cb], base, d, off, in, ocap);
+            }
+            if (otc) move_array(otc, B.tc[cb], base, d, off, in, ocap);
+        },
+        [&](unsigned long long kept) { *out_count = kept; });
 }
 
 // Validation of freshly loaded particles (x in [0, L), finite velocities)
@@ -705,9 +663,8 @@ void launch_field_batched(const Params* all, int n, size_t smem, int mode, int p
     launch_pdl(k_field_b, 2 * n, FT, smem, s, all, mode, pushed_mask);
 }
 
-void launch_compact_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
-    auto k = species == SP_E ? k_compact_b<SP_E> : (species == SP_OM ? k_compact_b<SP_OM> : k_compact_b<SP_OP>);
-    launch_pdl(k, nblocks, BLOCK, 0, s, all, map);
+void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
+    launch_pdl(k_compact_b, nblocks, CMP_T, 0, s, all, map);
 }
 
 void launch_field(const Params& P, int mode, int pushed_mask, cudaStream_t s) {
@@ -720,22 +677,15 @@ cudaError_t configure_field_smem(size_t bytes) {
     return e;
 }
 
-void launch_compact(int species, const Params& P, int grid, cudaStream_t s) {
-    auto k = species == SP_E ? k_compact<SP_E> : (species == SP_OM ? k_compact<SP_OM> : k_compact<SP_OP>);
-    launch_pdl(k, grid, BLOCK, 0, s, P, 0, 0ull, (unsigned*)nullptr, (unsigned long long*)nullptr,
-               (unsigned long long*)nullptr, (float*)nullptr, (float*)nullptr, (float*)nullptr, (float*)nullptr,
-               (uint32_t*)nullptr, (uint32_t*)nullptr, 0ull, (unsigned long long*)nullptr);
+// `grid` blocks per species (two per SM are resident)
+void launch_compact(const Params& P, int grid, cudaStream_t s) {
+    launch_pdl(k_compact, dim3(grid, NSP), CMP_T, 0, s, P);
 }
 
 void launch_gather(int species, const Params& P, int grid, unsigned long long epoch, unsigned* ticket,
                    unsigned long long* flag, unsigned long long* val, float* x, float* vx, float* vy, float* vz,
                    uint32_t* id, uint32_t* tc, unsigned long long cap, unsigned long long* out_count, cudaStream_t s) {
-    if (species == SP_E)
-        k_compact<SP_E><<<grid, BLOCK, 0, s>>>(P, 1, epoch, ticket, flag, val, x, vx, vy, vz, id, tc, cap, out_count);
-    else if (species == SP_OM)
-        k_compact<SP_OM><<<grid, BLOCK, 0, s>>>(P, 1, epoch, ticket, flag, val, x, vx, vy, vz, id, tc, cap, out_count);
-    else
-        k_compact<SP_OP><<<grid, BLOCK, 0, s>>>(P, 1, epoch, ticket, flag, val, x, vx, vy, vz, id, tc, cap, out_count);
+    k_gather<<<grid, CMP_T, 0, s>>>(P, species, epoch, ticket, flag, val, x, vx, vy, vz, id, tc, cap, out_count);
 }
 
 void launch_load_check(int species, const Params& P, unsigned long long n, cudaStream_t s) {

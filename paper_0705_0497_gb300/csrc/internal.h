@@ -45,15 +45,11 @@ constexpr float GRID_EMIN = 0.0009765625f;                       // 2^-10
 constexpr float GRID_EMAX = 4096.0f;                             // 2^12
 
 constexpr int BLOCK = 256;              // threads of the particle kernels
-constexpr int ITEMS = 4;                // particles per thread per chunk (one float4)
-constexpr int CHUNK = BLOCK * ITEMS;    // 1024
 constexpr int TILE = 8192;              // slots per tile (compaction, neutralization histograms)
 constexpr int WTILE = 2048;             // slots per warp work unit of the particle kernels
-constexpr int CHUNKS_PER_TILE = TILE / CHUNK;
 constexpr int FLUSH_TILES = 7;          // tiles between deposit flushes (7*8192*2^16 < 2^32)
 constexpr int MAX_TRIES = 32;           // rejection-loop cap
 constexpr uint32_t FIX_ONE = 65536u;    // CIC fixed point per particle
-constexpr int QCAP = BLOCK - 1 + CHUNK; // candidate queue capacity
 constexpr int MAX_NODES = 8193;         // grid limit (smem field and histograms)
 constexpr int JRING = 8192;             // steps of conduction-current sums kept on the device
 // Copies of a species' fresh deposit Qf (Ng each): the particle kernel's
@@ -174,9 +170,9 @@ struct Params {
     float dt_s[NSP], qmdt[NSP], kappa[NSP], a_m[NSP], a_M[NSP], sig_birth[NSP];
     float delta_el, sig_gas, kappa_n, pair_factor;
     uint32_t seed;
-    // decoupled look-back state: per kernel kind, flag and value words per tile
-    unsigned long long* lb_flag[NKK];
-    unsigned long long* lb_val[NKK];
+    // look-back state of the compaction: per species, flag and value words per tile
+    unsigned long long* lb_flag[NSP];
+    unsigned long long* lb_val[NSP];
     unsigned int max_tiles;
     // births staging, [wtile * WTILE + rank] per BirthSlot, and the number
     // staged by each warp work unit (B_OP_FROM_E shares B_E_FROM_E's counts)
@@ -283,14 +279,14 @@ void launch_edet_apply_batched(const Params* all, const PairSpec* specs, int n, 
 void launch_push_batched(int species, const Params* all, const uint4* map, int nblocks, size_t smem, cudaStream_t s);
 void launch_cand_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_field_batched(const Params* all, int n, size_t smem, int mode, int pushed_mask, cudaStream_t s);
-void launch_compact_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
+void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_pair_hist_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,
                               cudaStream_t s);
 void launch_pair_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, cudaStream_t s);
 void launch_pair_apply_batched(const Params* all, const PairSpec* specs, int n, cudaStream_t s);
 void launch_field(const Params& P, int mode, int pushed_mask, cudaStream_t s);
 void launch_phi(const Params& P, cudaStream_t s);
-void launch_compact(int species, const Params& P, int grid, cudaStream_t s);
+void launch_compact(const Params& P, int grid, cudaStream_t s);   // all species
 void launch_deposit(int species, const Params& P, int grid, cudaStream_t s);
 void launch_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, unsigned long long n, cudaStream_t s);
 void launch_ln(const float* x, float* out, unsigned long long n, cudaStream_t s);

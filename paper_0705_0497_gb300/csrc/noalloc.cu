@@ -19,7 +19,7 @@ size_t compact_scratch_words(unsigned long long n);
 void launch_compact_arrays(const float* x, const float* vx, const float* vy, const float* vz, const uint32_t* id,
                            unsigned long long n, float* ox, float* ovx, float* ovy, float* ovz, uint32_t* oid,
                            unsigned long long* n_out, unsigned long long* words, unsigned long long tiles,
-                           unsigned long long epoch, int grid, cudaStream_t s);
+                           unsigned long long epoch, int sms, cudaStream_t s);
 }  // namespace o2
 
 using namespace o2;
@@ -77,7 +77,7 @@ extern "C" int o2pic_compact_particles_noalloc(const float* x, const float* vx, 
     if (e == cudaSuccess) e = cudaMemsetAsync(n_out, 0, sizeof(uint64_t), s);
     if (e == cudaSuccess && n > 0) {
         launch_compact_arrays(x, vx, vy, vz, id, n, ox, ovx, ovy, ovz, oid, (unsigned long long*)n_out, scratch,
-                              NOALLOC_TILES, epoch, 4 * sms, s);
+                              NOALLOC_TILES, epoch, sms, s);
         e = cudaGetLastError();
     }
     unsigned long long err = 0;

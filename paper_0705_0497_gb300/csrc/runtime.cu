@@ -398,8 +398,7 @@ void enqueue_steps(o2pic_ctx* c, uint64_t nsteps, cudaStream_t s) {
         launch(c, KK_FIELD, s, [&] { launch_field(P, 0, ion ? 7 : 1, s); });
         c->host_step += 1;
         if (++c->since_check >= c->cfg.compact_check) {
-            for (int sp = 0; sp < NSP; ++sp)
-                launch(c, KK_COMPACT, s, [&] { launch_compact(sp, P, c->grid_compact, s); });
+            launch(c, KK_COMPACT, s, [&] { launch_compact(P, 2 * c->num_sms, s); });
             c->since_check = 0;
         }
     }
@@ -517,7 +516,7 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     TRY(ctx_alloc(c, &P.fU, Ng));
     TRY(ctx_alloc(c, &P.fVD, 2));
     TRY(ctx_alloc(c, &P.jring, (size_t)JRING * NSP));
-    for (int k = 0; k < NKK; ++k) {
+    for (int k = 0; k < NSP; ++k) {
         TRY(ctx_alloc(c, &P.lb_flag[k], max_tiles));
         TRY(ctx_alloc(c, &P.lb_val[k], 2 * max_tiles));
     }
@@ -909,7 +908,7 @@ int o2pic_read_particles(o2pic_ctx* c, int species, float* x, float* vx, float* 
     }
     c->gepoch += 1;
     cudaMemsetAsync(c->d_gticket, 0, sizeof(unsigned), s);
-    launch_gather(species, c->P, c->grid_compact, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
+    launch_gather(species, c->P, 2 * c->num_sms, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
                   dx_, dvx, dvy, dvz, did, nullptr, m, c->d_gcount, s);
     c->launches += 1;
     e = cudaStreamSynchronize(s);
@@ -1019,7 +1018,7 @@ int o2pic_read_flight(o2pic_ctx* c, int species, uint32_t* tc, uint64_t cap, uin
     }
     c->gepoch += 1;
     cudaMemsetAsync(c->d_gticket, 0, sizeof(unsigned), s);
-    launch_gather(species, c->P, c->grid_compact, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
+    launch_gather(species, c->P, 2 * c->num_sms, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
                   nullptr, nullptr, nullptr, nullptr, nullptr, dtc, m, c->d_gcount, s);
     c->launches += 1;
     e = cudaStreamSynchronize(s);
@@ -1223,9 +1222,9 @@ struct o2pic_batch {
     PairSpec* dD = nullptr;               // [n] (22)
     PairSpec* dN = nullptr;               // [n] (17)
     uint4* dmap = nullptr;                // block maps, concatenated
-    size_t map_push[NSP] = {0, 0, 0}, map_comp[NSP] = {0, 0, 0}, map_rh = 0, map_rp = 0, map_nh = 0, map_np = 0;
+    size_t map_push[NSP] = {0, 0, 0}, map_comp = 0, map_rh = 0, map_rp = 0, map_nh = 0, map_np = 0;
     size_t map_dh = 0, map_dp = 0;
-    int nb_push[NSP] = {0, 0, 0}, nb_comp[NSP] = {0, 0, 0}, nb_rh = 0, nb_rp = 0, nb_nh = 0, nb_np = 0;
+    int nb_push[NSP] = {0, 0, 0}, nb_comp = 0, nb_rh = 0, nb_rp = 0, nb_nh = 0, nb_np = 0;
     int nb_dh = 0, nb_dp = 0;
     bool any_recomb = false, any_neutral = false, any_edet = false;
     size_t smem_push = 0, smem_field = 0, smem_hist = 0;
@@ -1272,11 +1271,15 @@ int fused_tables(o2pic_batch* b) {
         b->smem_field = std::max(b->smem_field, field_smem_bytes(P));
         b->smem_hist = std::max(b->smem_hist, 3 * sizeof(unsigned) * (size_t)P.Nc);
     }
-    for (int sp = 0; sp < NSP; ++sp) {
+    for (int sp = 0; sp < NSP; ++sp)
         add_map(b->map_push[sp], b->nb_push[sp], [&](o2pic_ctx* c) { return c->grid_push[sp]; });
-        add_map(b->map_comp[sp], b->nb_comp[sp],
-                [&](o2pic_ctx* c) { return std::min<unsigned long long>(tiles(c->P.sp[sp].cap), 16); });
-    }
+    b->map_comp = map.size();
+    for (size_t i = 0; i < n; ++i)
+        for (unsigned sp = 0; sp < NSP; ++sp) {
+            const unsigned k = (unsigned)std::min<unsigned long long>(tiles(b->ctx[i]->P.sp[sp].cap), 16);
+            for (unsigned j = 0; j < k; ++j) map.push_back(make_uint4((unsigned)i, j, k, sp));
+        }
+    b->nb_comp = (int)(map.size() - b->map_comp);
     add_map(b->map_dh, b->nb_dh, [&](o2pic_ctx* c) {
         return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap) + tiles(c->P.sp[SP_E].cap), 32); });
     add_map(b->map_dp, b->nb_dp, [&](o2pic_ctx* c) { return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap), 64); });
@@ -1352,9 +1355,8 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
         launches += 1;
         step += 1;
         if (++since >= c0->cfg.compact_check) {
-            for (int sp = 0; sp < NSP; ++sp)
-                launch_compact_batched(sp, b->dP, b->dmap + b->map_comp[sp], b->nb_comp[sp], s);
-            launches += 3;
+            launch_compact_batched(b->dP, b->dmap + b->map_comp, b->nb_comp, s);
+            launches += 1;
             since = 0;
         }
     }
