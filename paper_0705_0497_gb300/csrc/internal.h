@@ -143,7 +143,6 @@ struct Params {
     float inv_lnq[NSP], kcap[NSP];
     unsigned sub[NSP];
     int births_possible[NSP];
-    int cum_smem[NSP];           // particle kernel stages the cumulative table in shared memory
     // (17)
     const float* Ktab;           // [NGRID] sigma_n g
     float Kmax_hi;               // max(Ktab) inflated so the prefilter bounds every interpolant
@@ -259,12 +258,6 @@ __host__ __device__ inline unsigned warp_range_len(unsigned n, unsigned W) {
 // (defined in the kernel translation units, called by the runtime)
 void launch_push(int species, const Params& P, int grid, cudaStream_t s);
 void launch_cand(int species, const Params& P, int grid, cudaStream_t s);   // ion species
-// true when the ion filter and kinematics run inside the ion particle kernels
-// (then the filter and kinematics kernels are not launched)
-bool ions_fused();
-// true when the particle kernel may stage the cumulative rate table in shared
-// memory (it does when the table keeps its resident blocks per SM)
-bool cum_smem_allowed();
 void launch_filter(int species, const Params& P, int grid, cudaStream_t s);
 void launch_filter_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_pair_hist(const Params& P, const PairSpec& S, int grid, cudaStream_t s);

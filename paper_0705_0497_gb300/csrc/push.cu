@@ -54,25 +54,6 @@
 #ifndef O2PIC_PUSH_E_MIN_BLOCKS
 #define O2PIC_PUSH_E_MIN_BLOCKS 3
 #endif
-// Ion candidates filtered (gas target, energy against the total rate) and
-// their real collisions handled inside the particle kernel, as for the
-// electrons (1), or by the separate filter and kinematics kernels (0).  Both
-// give the same results; on the 512-cell, 1.6e7-particle discharge at its
-// periodic state the separate kernels were faster (48.4 against 49.1 ms per
-// RF cycle): the ion filter's Maxwellian target draws weigh on the particle
-// kernel's registers.
-#ifndef O2PIC_FUSE_IONS
-#define O2PIC_FUSE_IONS 0
-#endif
-// The particle kernel that runs the kinematics stages the species' cumulative
-// rate table in shared memory when that keeps its resident blocks per SM (1),
-// or reads it from global memory through L1 (0).  Both give the same results;
-// on the 512-cell, 1.6e7-particle discharge at its periodic state the global
-// table was faster (46.3 against 47.5 ms per RF cycle): every block copies
-// the electrons' 34 KB table each step, and the kinematics read a few rows.
-#ifndef O2PIC_CUM_SMEM
-#define O2PIC_CUM_SMEM 0
-#endif
 // Minimum resident blocks per SM of the kinematics kernel (caps its registers
 // at 85, no spills; 3 timed fastest of 2, 3, 4 on the same workload).
 #ifndef O2PIC_CAND_MIN_BLOCKS
@@ -99,6 +80,10 @@ struct PushShared {
     unsigned nonfinite;
     unsigned wtries;
     unsigned events[MAXPROC];    // electrons: real collisions per process
+    // electrons: the block's pool of collisions (see push_body)
+    unsigned first[WARPS], start[WARPS + 1];   // first pooled record of each warp, its place in the pool
+    unsigned nb1[WARPS], nb2[WARPS];           // births of each warp's own passes (ionizations, attachments)
+    unsigned m1[WARPS], m2[WARPS];             // births of the pool, by thread
 };
 
 // First record of particle-kernel warp gw (of W) in its species' candidate list:
@@ -117,40 +102,12 @@ __device__ __forceinline__ unsigned list_start(unsigned gw, unsigned W, unsigned
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
 
-// One real collision (a candidate its filter kept) through process selection
-// and kinematics, exactly in the order of the oracle.  The filter already
-// counted the warnings of the part it shares with this function (the ions'
-// target sample, the energy above the grid), so they are not counted again.
-// Returns the event index, or -1 for a null collision (the selected
-// process's threshold above E; the rate test itself repeats the filter's).
-// bkind: 0 none, 1 ionization (two births), 2 attachment / detachment (one).
-template <int S>
-__device__ __forceinline__ int collide(const Params& P, const float* cum, int np, unsigned long long step,
-                                       uint32_t id, uint4 w0, float x, float& vx, float& vy, float& vz,
-                                       bool& alive, int& bkind, float4& b1, float4& b2,
-                                       unsigned& warn_tries, unsigned& warn_emax) {
-    alive = true;
-    bkind = 0;
-    Stream st;
-    st.resume(id, P.seed, step, SpeciesTraits<S>::tag, w0, 1);
-    const float u1 = uniform(st.next());
-    float vtx = 0.0f, vty = 0.0f, vtz = 0.0f;
-    float gx = vx, gy = vy, gz = vz;
-    if (S != SP_E) {
-        unsigned counted_by_filter = 0;
-        maxwellian(st, P.sig_gas, vtx, vty, vtz, counted_by_filter);
-        gx = vx - vtx; gy = vy - vty; gz = vz - vtz;
-    }
-    const float E = P.kappa[S] * dot3(gx, gy, gz, gx, gy, gz);
-    int i; float w; bool above;
-    grid_locate(E, i, w, above);
-    (void)warn_emax;
-    // null collision unless u1 nu_max falls below the total rate; then the
-    // first process whose cumulative rate exceeds it (the last one if
-    // rounding leaves none)
-    // the cumulative rates are read four processes at a time (loads in
-    // flight together); each value is grid_interp(cum, np, kk, i, w)
-    const float target = u1 * P.numax[S];
+// Process of a real collision (a candidate its filter kept): the total rate is
+// above u1 nu_max, and the first process whose cumulative rate exceeds it is
+// chosen (the last one if rounding leaves none).  -1: null (rounding).  The
+// cumulative rates are read four processes at a time (loads in flight
+// together); each value is grid_interp(cum, np, kk, i, w).
+__device__ __forceinline__ int select_process(const float* __restrict__ cum, int np, float target, int i, float w) {
     const bool last = i >= NGRID - 1;
     const float* row = cum + (size_t)(last ? NGRID - 1 : i) * np;
     auto interp = [&](float a, float b) { return last ? a : fmaf(w, b - a, a); };
@@ -162,7 +119,6 @@ __device__ __forceinline__ int collide(const Params& P, const float* cum, int np
         b[j] = (j < np - 1 && !last) ? row[np + j] : 0.0f;
     }
     if (!(target < interp(ta, tb))) return -1;
-    int k = np - 1;
     for (int k0 = 0; k0 < np - 1; k0 += 4) {
         if (k0 > 0) {
 #pragma unroll
@@ -178,66 +134,157 @@ __device__ __forceinline__ int collide(const Params& P, const float* cum, int np
             const int kk = k0 + j;
             if (f < 0 && kk < np - 1 && target < interp(a[j], b[j])) f = kk;
         }
-        if (f >= 0) { k = f; break; }
+        if (f >= 0) return f;
     }
+    return np - 1;
+}
+
+// One real collision of an electron: process selection and kinematics, with the
+// random words and the arithmetic in the order of the oracle.  w0: block 0 of
+// its stream (word 0, the candidate draw, is spent).  Returns the event index,
+// or -1 for a null collision (the selected process's threshold above E; the
+// rate test itself repeats the filter's).  bkind: 0 none, 1 ionization (two
+// births), 2 attachment (one).
+//
+// The directions (points of the unit disk) and normals (the same without the
+// centre) a lane needs are drawn by one rejection loop, task after task: 0, 1
+// directions, 2, 3 pairs of normals; elastic and excited electrons need task
+// 0, an ionization 0-3 (after the share of the energy), an attachment 2-3.  A
+// warp passes the loop as often as its longest lane needs in all, not in each
+// task, and the code holds one Philox block instead of nine.
+__device__ __forceinline__ int collide_electron(const Params& P, const float* __restrict__ cum, int np,
+                                                unsigned long long step, uint32_t id, uint4 w0, float x, float& vx,
+                                                float& vy, float& vz, bool& alive, int& bkind, float4& b1, float4& b2,
+                                                unsigned& warn_tries) {
+    alive = true;
+    bkind = 0;
+    const float E = P.kappa[SP_E] * dot3(vx, vy, vz, vx, vy, vz);
+    int i; float w; bool above;
+    grid_locate(E, i, w, above);
+    const int k = select_process(cum, np, uniform(w0.y) * P.numax[SP_E], i, w);
+    if (k < 0) return -1;
+    const float thr = P.thr[SP_E][k];
+    if (E < thr) return -1;
+    const int kind = P.kind[SP_E][k];
+    const bool ionize = kind == K_IONIZE, attach = kind == K_ATTACH;
+    uint4 buf = w0;
+    uint32_t block = 0;
+    int pos = 2;
+    float u = 0.0f;
+    if (ionize) { u = uniform(buf.z); pos = 3; }
+    float a0 = 0.0f, c0 = 0.0f, s0 = 0.0f, a1 = 0.0f, c1 = 0.0f, s1 = 0.0f, a2 = 0.0f, c2 = 0.0f, s2 = 0.5f,
+          a3 = 0.0f, s3 = 0.5f;
+    const int last_task = (ionize || attach) ? 4 : 1;
+    int task = attach ? 2 : 0, tries = 0;
+    while (task < last_task) {
+        // the next two words
+        const uint32_t held = pos == 2 ? buf.z : (pos == 3 ? buf.w : (pos == 0 ? buf.x : buf.y));
+        uint32_t wa = held, wb;
+        if (pos <= 2) {
+            wb = pos == 2 ? buf.w : (pos == 1 ? buf.z : buf.y);
+            pos += 2;
+        } else {
+            ++block;
+            buf = philox4x32_10(make_uint4((uint32_t)step, SpeciesTraits<SP_E>::tag, block, (uint32_t)(step >> 32)),
+                                make_uint2(id, P.seed));
+            wa = pos == 3 ? held : buf.x;
+            wb = pos == 3 ? buf.x : buf.y;
+            pos = pos == 3 ? 1 : 2;
+        }
+        float a = 2.0f * uniform(wa) - 1.0f;
+        float b = 2.0f * uniform(wb) - 1.0f;
+        float s = fmaf(a, a, b * b);
+        if (!(s < 1.0f && (task < 2 || s > 0.0f))) {
+            if (++tries < MAX_TRIES) continue;
+            ++warn_tries;              // gives up: direction (0, 0, 1), normals 0
+            a = 0.0f; b = 0.0f; s = task < 2 ? 0.0f : 0.5f;
+        }
+        if (task == 0) { a0 = a; c0 = b; s0 = s; }
+        else if (task == 1) { a1 = a; c1 = b; s1 = s; }
+        else if (task == 2) { a2 = a; c2 = b; s2 = s; }
+        else { a3 = a; s3 = s; }
+        ++task;
+        tries = 0;
+    }
+    if (ionize || attach) {
+        const float sig = P.sig_birth[ionize ? SP_OP : SP_OM];
+        const float f2 = sqrtf((-2.0f * ln_series(s2)) / s2), f3 = sqrtf((-2.0f * ln_series(s3)) / s3);
+        b2 = make_float4(x, sig * (a2 * f2), sig * (c2 * f2), sig * (a3 * f3));
+        if (attach) {
+            b1 = b2;
+            bkind = 2;
+            alive = false;
+            return k;
+        }
+    }
+    const float h0 = 2.0f * sqrtf(1.0f - s0);
+    const float nx = a0 * h0, ny = c0 * h0, nz = 1.0f - 2.0f * s0;
+    float vn;
+    if (kind == K_ELASTIC) {
+        const float vm = sqrtf(dot3(vx, vy, vz, vx, vy, vz));
+        const float cosx = (vm > 0.0f) ? dot3(nx, ny, nz, vx, vy, vz) / vm : 0.0f;
+        const float fac = 1.0f - P.delta_el * (1.0f - cosx);
+        vn = vm * sqrtf(fac);
+    } else {
+        const float Er = E - thr;
+        float Ep = Er;
+        if (ionize) {
+            const float Es = u * Er;
+            Ep = Er - Es;
+            const float h1 = 2.0f * sqrtf(1.0f - s1);
+            const float vs = sqrtf(Es / P.kappa[SP_E]);
+            b1 = make_float4(x, vs * (a1 * h1), vs * (c1 * h1), vs * (1.0f - 2.0f * s1));
+            bkind = 1;
+        }
+        vn = sqrtf(Ep / P.kappa[SP_E]);
+    }
+    vx = vn * nx; vy = vn * ny; vz = vn * nz;
+    return k;
+}
+
+// One real collision of an ion, exactly in the order of the oracle (its filter
+// already counted the warnings of the target sample and the energy).  Returns
+// as collide_electron; bkind 2: detachment (the electron in b1).
+template <int S>
+__device__ __forceinline__ int collide_ion(const Params& P, const float* __restrict__ cum, int np,
+                                           unsigned long long step, uint32_t id, uint4 w0, float x, float& vx,
+                                           float& vy, float& vz, bool& alive, int& bkind, float4& b1,
+                                           unsigned& warn_tries) {
+    alive = true;
+    bkind = 0;
+    Stream st;
+    st.resume(id, P.seed, step, SpeciesTraits<S>::tag, w0, 1);
+    const float u1 = uniform(st.next());
+    float vtx, vty, vtz;
+    unsigned counted_by_filter = 0;
+    maxwellian(st, P.sig_gas, vtx, vty, vtz, counted_by_filter);
+    const float gx = vx - vtx, gy = vy - vty, gz = vz - vtz;
+    const float E = P.kappa[S] * dot3(gx, gy, gz, gx, gy, gz);
+    int i; float w; bool above;
+    grid_locate(E, i, w, above);
+    const int k = select_process(cum, np, u1 * P.numax[S], i, w);
+    if (k < 0) return -1;
     const float thr = P.thr[S][k];
     if (E < thr) return -1;
     const int kind = P.kind[S][k];
+    if (kind == K_CX) {
+        vx = vtx; vy = vty; vz = vtz;
+        return k;
+    }
+    float nx, ny, nz;
+    isotropic(st, nx, ny, nz, warn_tries);
     if (kind == K_ELASTIC) {
-        float nx, ny, nz;
-        isotropic(st, nx, ny, nz, warn_tries);
-        if (S == SP_E) {
-            const float v2 = dot3(vx, vy, vz, vx, vy, vz);
-            const float vm = sqrtf(v2);
-            const float cosx = (vm > 0.0f) ? dot3(nx, ny, nz, vx, vy, vz) / vm : 0.0f;
-            const float fac = 1.0f - P.delta_el * (1.0f - cosx);
-            const float vn = vm * sqrtf(fac);
-            vx = vn * nx; vy = vn * ny; vz = vn * nz;
-        } else {
-            const float gm = sqrtf(dot3(gx, gy, gz, gx, gy, gz));
-            const float cmx = fmaf(P.a_m[S], vx, P.a_M[S] * vtx);
-            const float cmy = fmaf(P.a_m[S], vy, P.a_M[S] * vty);
-            const float cmz = fmaf(P.a_m[S], vz, P.a_M[S] * vtz);
-            const float f = P.a_M[S] * gm;
-            vx = fmaf(f, nx, cmx); vy = fmaf(f, ny, cmy); vz = fmaf(f, nz, cmz);
-        }
-    } else if (kind == K_EXCITE) {
-        const float Ep = E - thr;
-        float nx, ny, nz;
-        isotropic(st, nx, ny, nz, warn_tries);
-        const float vn = sqrtf(Ep / P.kappa[S]);
-        vx = vn * nx; vy = vn * ny; vz = vn * nz;
-    } else if (kind == K_IONIZE) {
-        const float Er = E - thr;
-        const float u = uniform(st.next());
-        const float Es = u * Er;
-        const float Epr = Er - Es;
-        float n1x, n1y, n1z, n2x, n2y, n2z, vix, viy, viz;
-        isotropic(st, n1x, n1y, n1z, warn_tries);
-        isotropic(st, n2x, n2y, n2z, warn_tries);
-        maxwellian(st, P.sig_birth[SP_OP], vix, viy, viz, warn_tries);
-        const float vp = sqrtf(Epr / P.kappa[SP_E]);
-        const float vs = sqrtf(Es / P.kappa[SP_E]);
-        vx = vp * n1x; vy = vp * n1y; vz = vp * n1z;
-        b1 = make_float4(x, vs * n2x, vs * n2y, vs * n2z);
-        b2 = make_float4(x, vix, viy, viz);
-        bkind = 1;
-    } else if (kind == K_ATTACH) {
-        float vix, viy, viz;
-        maxwellian(st, P.sig_birth[SP_OM], vix, viy, viz, warn_tries);
-        b1 = make_float4(x, vix, viy, viz);
-        bkind = 2;
-        alive = false;
-    } else if (kind == K_DETACH) {
-        const float Er = E - thr;
-        float nx, ny, nz;
-        isotropic(st, nx, ny, nz, warn_tries);
-        const float vn = sqrtf(Er / P.kappa[SP_E]);
+        const float gm = sqrtf(dot3(gx, gy, gz, gx, gy, gz));
+        const float cmx = fmaf(P.a_m[S], vx, P.a_M[S] * vtx);
+        const float cmy = fmaf(P.a_m[S], vy, P.a_M[S] * vty);
+        const float cmz = fmaf(P.a_m[S], vz, P.a_M[S] * vtz);
+        const float f = P.a_M[S] * gm;
+        vx = fmaf(f, nx, cmx); vy = fmaf(f, ny, cmy); vz = fmaf(f, nz, cmz);
+    } else if (S == SP_OM && kind == K_DETACH) {
+        const float vn = sqrtf((E - thr) / P.kappa[SP_E]);
         b1 = make_float4(x, vn * nx, vn * ny, vn * nz);
         bkind = 2;
         alive = false;
-    } else if (kind == K_CX) {
-        vx = vtx; vy = vty; vz = vtz;
     }
     return k;
 }
@@ -293,29 +340,6 @@ __device__ __forceinline__ bool electron_is_real(const Params& P, const float* t
     return (u1 * P.numax[SP_E]) < total;
 }
 
-// Filter of an ion candidate: the target sampled from the gas Maxwellian
-// (words 2, 3 of block 0 and the blocks after), the relative energy, and the
-// total rate on the table grid against u1 nu_max (word 1): the same
-// arithmetic as the start of collide().
-template <int S>
-__device__ __forceinline__ bool ion_is_real(const Params& P, const float* tot, unsigned long long step, uint32_t id,
-                                            uint4 w, float vx, float vy, float vz, unsigned& wtries,
-                                            unsigned& wemax, unsigned& wnumax) {
-    Stream st;
-    st.resume(id, P.seed, step, SpeciesTraits<S>::tag, w, 1);
-    const float u1 = uniform(st.next());
-    float vtx, vty, vtz;
-    maxwellian(st, P.sig_gas, vtx, vty, vtz, wtries);
-    const float gx = vx - vtx, gy = vy - vty, gz = vz - vtz;
-    const float E = P.kappa[S] * dot3(gx, gy, gz, gx, gy, gz);
-    int i; float wt; bool above;
-    grid_locate(E, i, wt, above);
-    if (above) ++wemax;
-    const float total = grid_interp(tot, 1, 0, i, wt);
-    if (total > P.numax[S]) ++wnumax;   // above a capped majorant
-    return (u1 * P.numax[S]) < total;
-}
-
 // Total-rate column (the last cumulative column) of species S into shared memory.
 __device__ __forceinline__ void stage_total(const Params& P, int S, float* tot) {
     const float* __restrict__ g = P.tot[S];
@@ -349,29 +373,21 @@ __device__ __forceinline__ void cell_sub(unsigned* cnt, unsigned* rsum, int c, u
     if (old < r) weight_wrapped(Q, c, -1);
 }
 
-// Real collisions of the list of one particle-kernel warp (records r0 ..
-// r0 + n - 1, in slot order), taken SEGW records per pass by the SEGW lanes
-// of one segment of the calling warp (seg_mask: its lanes; sl: this lane's
-// index in it; lt_mask: the segment's lanes below this one; nmax: the longest
-// list among the warp's segments, so that every lane makes the same passes).
-// Electron records carry the particle (slot, id, x, v) and block 0 of its
-// Philox stream is drawn again; ion records carry the slot, id, v and that
-// block (its first word, the candidate draw, is spent), x is read from the
-// array.  `cum` is the species' cumulative rate table (global or shared
-// memory).  A removed particle's charge comes off the block's deposit when
-// `cnt` is given (the particle kernel: the particle was deposited there),
-// else off the step's deposit in global memory.  Births are ranked with
-// ballots within the segment and staged at the particle warp's slot range;
-// nb1, nb2 count them.
+// Real collisions of the list of one ion-push warp (records r0 .. r0 + n - 1, in
+// slot order), taken SEGW records per pass by the SEGW lanes of one segment of
+// the calling warp (seg_mask: its lanes; sl: this lane's index in it; lt_mask:
+// the segment's lanes below this one; nmax: the longest list among the warp's
+// segments, so that every lane makes the same passes).  Records carry the
+// slot, id, v and block 0 of the Philox stream (its first word, the candidate
+// draw, is spent); x is read from the array.  A removed particle's charge
+// comes off the step's deposit.  Births are ranked with ballots within the
+// segment and staged at the push warp's slot range; nb counts them.
 template <int S, int SEGW>
-__device__ __forceinline__ void collide_list(const Params& P, const float* cum, const PhiloxPre& pre,
-                                             unsigned long long step,
-                                             unsigned r0, unsigned n, unsigned nmax, unsigned sl,
-                                             unsigned seg_mask, unsigned lt_mask, unsigned* events,
-                                             unsigned* cnt, unsigned* rsum, unsigned long long* Qcopy,
-                                             unsigned& nb1, unsigned& nb2,
-                                             unsigned& nremoved, unsigned& wtries, unsigned& wemax) {
+__device__ __forceinline__ void collide_list(const Params& P, unsigned long long step, unsigned r0, unsigned n,
+                                             unsigned nmax, unsigned sl, unsigned seg_mask, unsigned lt_mask,
+                                             unsigned* events, unsigned& nb, unsigned& nremoved, unsigned& wtries) {
     const int np = P.nproc[S];
+    const float* __restrict__ cum = P.cum[S];
     const unsigned cb = P.ctrl->cur[S];
     float* __restrict__ X = P.sp[S].x[cb];
     float* __restrict__ VX = P.sp[S].vx[cb];
@@ -380,74 +396,51 @@ __device__ __forceinline__ void collide_list(const Params& P, const float* cum, 
     const uint4* __restrict__ CAND = P.cand[S];
     const float inv_dx = P.inv_dx;
     const int Nc = P.Nc;
-    const bool births = P.births_possible[S] != 0;
+    const bool births = S == SP_OM && P.births_possible[S] != 0;
     for (unsigned c0 = 0; c0 < nmax; c0 += SEGW) {
         const unsigned ci = c0 + sl;
         const bool has = ci < n;
-        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-        if (has) { a = CAND[2 * (size_t)(r0 + ci)]; b = CAND[2 * (size_t)(r0 + ci) + 1]; }
-        const unsigned slot = a.x;
-        float x, vx, vy, vz;
-        uint4 w0;
-        if (S == SP_E) {
-            x = __uint_as_float(a.z); vx = __uint_as_float(a.w);
-            vy = __uint_as_float(b.x); vz = __uint_as_float(b.y);
-            w0 = has ? philox_id(pre, a.y) : make_uint4(0u, 0u, 0u, 0u);
-        } else {
-            x = has ? X[slot] : 0.0f;
-            vx = __uint_as_float(a.z); vy = __uint_as_float(a.w); vz = __uint_as_float(b.x);
-            w0 = make_uint4(0u, b.y, b.z, b.w);
-        }
-        w0.x = a.y;   // word 0 (the candidate draw) is spent: it carries the id
         int bkind = 0;
-        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = b1;
+        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f);
         if (has) {
+            const uint4 a = CAND[2 * (size_t)(r0 + ci)], b = CAND[2 * (size_t)(r0 + ci) + 1];
+            const unsigned slot = a.x;
+            const float x = X[slot];
+            float vx = __uint_as_float(a.z), vy = __uint_as_float(a.w), vz = __uint_as_float(b.x);
             bool alive;
-            const int k = collide<S>(P, cum, np, step, a.y, w0, x, vx, vy, vz, alive, bkind, b1, b2, wtries, wemax);
+            const int k = collide_ion<S>(P, cum, np, step, a.y, make_uint4(a.y, b.y, b.z, b.w), x, vx, vy, vz, alive,
+                                         bkind, b1, wtries);
             if (k >= 0) {
                 atomicAdd(&events[k], 1u);
                 if (alive) {
                     VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
                 } else {
                     X[slot] = dead_marker();
-                    if (cnt) {
-                        int j; float f;
-                        cell_of(x, inv_dx, Nc, j, f);
-                        cell_sub(cnt, rsum, j, cic_r(f), Qcopy);
-                    } else {
-                        deposit_sub_global(P.Qf[S], x, inv_dx, Nc);
-                    }
+                    deposit_sub_global(P.Qf[S], x, inv_dx, Nc);
                     ++nremoved;
                 }
             }
         }
         if (births) {
-            const unsigned m1 = __ballot_sync(0xffffffffu, bkind == 1) & seg_mask;
-            const unsigned m2 = __ballot_sync(0xffffffffu, bkind == 2) & seg_mask;
             // staged for the end-of-step kernel, which places them; their
             // charge goes to Qb now
-            if (S == SP_E) {
-                if (bkind == 1) {
-                    const unsigned r = nb1 + __popc(m1 & lt_mask);
-                    P.stage[B_E_FROM_E][r0 + r] = b1;
-                    P.stage[B_OP_FROM_E][r0 + r] = b2;
-                    deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
-                    deposit_add_global(P.Qb[SP_OP], b2.x, inv_dx, Nc);
-                } else if (bkind == 2) {
-                    P.stage[B_OM_FROM_E][r0 + nb2 + __popc(m2 & lt_mask)] = b1;
-                    deposit_add_global(P.Qb[SP_OM], b1.x, inv_dx, Nc);
-                }
-            } else if (S == SP_OM) {
-                if (bkind == 2) {
-                    P.stage[B_E_FROM_OM][r0 + nb2 + __popc(m2 & lt_mask)] = b1;
-                    deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
-                }
+            const unsigned m = __ballot_sync(0xffffffffu, bkind == 2) & seg_mask;
+            if (bkind == 2) {
+                P.stage[B_E_FROM_OM][r0 + nb + __popc(m & lt_mask)] = b1;
+                deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
             }
-            nb1 += __popc(m1);
-            nb2 += __popc(m2);
+            nb += __popc(m);
         }
         __syncwarp();
     }
+}
+
+// Set bits [a, b) of the 32-bit words in m (b - a <= 32).
+__device__ __forceinline__ unsigned bits_between(const unsigned* m, unsigned a, unsigned b) {
+    if (a >= b) return 0u;
+    const unsigned wa = a >> 5, wb = (b - 1u) >> 5;
+    const unsigned lo = 0xffffffffu << (a & 31u), hi = 0xffffffffu >> (31u - ((b - 1u) & 31u));
+    return wa == wb ? __popc(m[wa] & lo & hi) : __popc(m[wa] & lo) + __popc(m[wb] & hi);
 }
 
 // Candidate queue of one warp of the particle kernel (shared memory): the slots
@@ -469,11 +462,8 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     unsigned* cnt = reinterpret_cast<unsigned*>(Es + P.Ng);
     unsigned* rsum = cnt + P.Ng;
     PushQueue& Q = *reinterpret_cast<PushQueue*>(rsum + P.Ng);
-    float* Tt = reinterpret_cast<float*>(&Q + 1);        // total-rate column (filter in the kernel)
-    float* Ct = Tt + NGRID;                              // cumulative table (if staged)
-    constexpr bool fused = (S == SP_E) || (O2PIC_FUSE_IONS != 0);
-    const bool cum_staged = fused && P.cum_smem[S] != 0;
-    const float* cum = cum_staged ? Ct : P.cum[S];
+    float* Tt = reinterpret_cast<float*>(&Q + 1);        // electrons: total-rate column
+    constexpr bool electrons = S == SP_E;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned* qs = Q.slot[warp];
@@ -485,11 +475,11 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const unsigned nslots = (unsigned)((C->slots[S] < P.sp[S].cap) ? C->slots[S] : P.sp[S].cap);
     float* __restrict__ X = P.sp[S].x[cb];
     float* __restrict__ VX = P.sp[S].vx[cb];
-    const float* __restrict__ VY = P.sp[S].vy[cb];
-    const float* __restrict__ VZ = P.sp[S].vz[cb];
+    float* __restrict__ VY = P.sp[S].vy[cb];
+    float* __restrict__ VZ = P.sp[S].vz[cb];
     const uint32_t* __restrict__ ID = P.sp[S].id[cb];
     uint32_t* __restrict__ TC = P.sp[S].tc[cb];
-    uint4* __restrict__ CAND = P.cand[S];
+    uint4* CAND = P.cand[S];          // written by one warp, read by others of the block
     const float qmdt = P.qmdt[S], dts = P.dt_s[S], inv_dx = P.inv_dx, Lf = P.Lf;
     const float inv_lnq = P.inv_lnq[S], kcap = P.kcap[S];
     const unsigned sub = P.sub[S];
@@ -540,16 +530,12 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     if (ga < gz) load_round(ga, xs, vxs, tcs);
 
     for (int j = tid; j < Ng; j += BLOCK) { Es[j] = P.Ef[j]; cnt[j] = 0u; rsum[j] = 0u; }
-    if (fused) stage_total(P, S, Tt);
-    if (cum_staged) {
-        const float* __restrict__ g = P.cum[S];
-        for (int j = tid; j < NGRID * np; j += BLOCK) Ct[j] = g[j];
-    }
+    if (electrons) stage_total(P, S, Tt);
     if (tid == 0) {
         sh.absorbed[0] = sh.absorbed[1] = 0u; sh.removed = 0u; sh.psteps = 0u; sh.nonfinite = 0u; sh.wtries = 0u;
         sh.jsum = 0ull;
     }
-    if (fused && tid < MAXPROC) sh.events[tid] = 0u;
+    if (electrons && tid < MAXPROC) sh.events[tid] = 0u;
     __syncthreads();
 
     unsigned psteps = 0, nabs0 = 0, nabs1 = 0, nnf = 0, wemax = 0, wtries = 0, wnumax = 0;
@@ -559,11 +545,10 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
 
     // m (<= 32) queued candidates from entry h on, one per lane: the candidate's
     // stream at this step (block 0) draws its next free flight (word 0) and
-    // the real/null test (word 1 against the total rate at the particle's
-    // energy; ions: relative to a target from the gas Maxwellian); records go
-    // to the warp's list in slot order, two uint4 each: electrons {slot, id,
-    // x, vx}{vy, vz, -, -}, ions {slot, id, vx, vy}{vz, w1, w2, w3} (the real
-    // collisions; with the ion filter in its own kernel, every ion candidate).
+    // the electrons' real/null test (word 1 against the total rate at the
+    // particle's energy); records go to the warp's list in slot order, two uint4 each: electrons {slot, id,
+    // x, vx}{vy, vz, -, -} per real collision, ions {slot, id, vx, vy}{vz, w1,
+    // w2, w3} per candidate.
     auto flush = [&](unsigned h, unsigned m) {
         const bool has = (unsigned)lane < m;
         const unsigned slot = has ? qs[h + lane] : 0u;
@@ -578,8 +563,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         if (has) {
             w = philox_id(pre, id);
             TC[slot] = step_lo + sub * (1u + flight_gap(w.x, inv_lnq, kcap));
-            if (S == SP_E) rec = electron_is_real(P, Tt, w.y, cvx, cvy, cvz, wemax, wnumax);
-            else rec = !fused || ion_is_real<S>(P, Tt, step, id, w, cvx, cvy, cvz, wtries, wemax, wnumax);
+            rec = !electrons || electron_is_real(P, Tt, w.y, cvx, cvy, cvz, wemax, wnumax);
         }
         const unsigned cm = __ballot_sync(0xffffffffu, rec);
         if (rec) {
@@ -706,24 +690,95 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     __syncwarp();
     if (qn > 0u) flush(0u, qn);
     unsigned nrm = 0;
-    if (fused) {
-        // the real collisions, by the warp that recorded them (its lanes'
-        // records are visible to the whole warp after the barrier): the
-        // kinematics run while other warps still push, and a removed
-        // particle's charge comes off this block's histogram.  The filter
+    if (electrons) {
+        // The real collisions: each warp takes its own records 32 at a time,
+        // and what is left (fewer than 32 per warp) is pooled over the block,
+        // in warp order, one record per thread, so that short lists still fill
+        // their warps (1.5e6 electrons: 11 records per warp).  A removed
+        // particle's charge comes off this block's deposit.  The filter
         // counted the warnings of the part it shares with the kinematics.
-        __syncwarp();
-        unsigned nb1 = 0, nb2 = 0, wt2 = 0, we2 = 0;
-        collide_list<S, 32>(P, cum, pre, step, rec0, nrec, nrec, (unsigned)lane, 0xffffffffu, lt_mask, sh.events, cnt,
-                            rsum, Qcopy, nb1, nb2, nrm, wt2, we2);
-        wtries += wt2;
-        if (P.births_possible[S] && lane == 0) {
-            if (S == SP_E) {
-                P.wcount[B_E_FROM_E][gw] = nb1;
-                P.wcount[B_OM_FROM_E][gw] = nb2;
-            } else if (S == SP_OM) {
-                P.wcount[B_E_FROM_OM][gw] = nb2;
+        // Births are staged at their warp's slot range in slot order: those of
+        // its own passes, then those of its pooled records.
+        const unsigned own = nrec & ~31u;
+        unsigned nb1 = 0, nb2 = 0;   // warp-uniform: births of its own passes
+        if (lane == 0) { sh.first[warp] = rec0 + own; sh.start[warp + 1] = nrec - own; }
+        __syncthreads();
+        if (warp == 0) {
+            unsigned v = lane < WARPS ? sh.start[lane + 1] : 0u;
+#pragma unroll
+            for (int o = 1; o < WARPS; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += y;
             }
+            if (lane < WARPS) sh.start[lane + 1] = v;
+            if (lane == 0) sh.start[0] = 0u;
+        }
+        __syncthreads();
+        const unsigned pooled = sh.start[WARPS];
+        const bool births = P.births_possible[S] != 0;
+        int bkind = 0;
+        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = b1;
+        unsigned u = (unsigned)warp;              // the warp whose record this is
+        for (unsigned c = 0;; c += 32u) {
+            const bool pool = c >= own;
+            bool has = true;
+            unsigned rec = rec0 + c + lane;
+            if (pool) {
+                has = (unsigned)tid < pooled;
+                for (u = 0; u < WARPS - 1 && (unsigned)tid >= sh.start[u + 1]; ++u) {}
+                rec = sh.first[u] + ((unsigned)tid - sh.start[u]);
+            }
+            bkind = 0;
+            if (has) {
+                const uint4 a = CAND[2 * (size_t)rec], b = CAND[2 * (size_t)rec + 1];
+                const unsigned slot = a.x;
+                const float x = __uint_as_float(a.z);
+                float vx = __uint_as_float(a.w), vy = __uint_as_float(b.x), vz = __uint_as_float(b.y);
+                bool alive;
+                const int k = collide_electron(P, P.cum[S], np, step, a.y, philox_id(pre, a.y), x, vx, vy, vz, alive,
+                                               bkind, b1, b2, wtries);
+                if (k >= 0) {
+                    atomicAdd(&sh.events[k], 1u);
+                    if (alive) {
+                        VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
+                    } else {
+                        X[slot] = dead_marker();
+                        int j; float f;
+                        cell_of(x, inv_dx, Nc, j, f);
+                        cell_sub(cnt, rsum, j, cic_r(f), Qcopy);
+                        ++nrm;
+                    }
+                }
+            }
+            const unsigned m1 = __ballot_sync(0xffffffffu, bkind == 1), m2 = __ballot_sync(0xffffffffu, bkind == 2);
+            unsigned rank1 = nb1 + __popc(m1 & lt_mask), rank2 = nb2 + __popc(m2 & lt_mask), s0 = r0;
+            if (pool) {
+                if (lane == 0) { sh.nb1[warp] = nb1; sh.nb2[warp] = nb2; sh.m1[warp] = m1; sh.m2[warp] = m2; }
+                __syncthreads();
+                if (bkind) {
+                    rank1 = sh.nb1[u] + bits_between(sh.m1, sh.start[u], (unsigned)tid);
+                    rank2 = sh.nb2[u] + bits_between(sh.m2, sh.start[u], (unsigned)tid);
+                    s0 = (blk * WARPS + u) * R;
+                }
+            }
+            // staged for the end-of-step kernel, which places them; their
+            // charge goes to Qb now
+            if (bkind == 1) {
+                P.stage[B_E_FROM_E][s0 + rank1] = b1;
+                P.stage[B_OP_FROM_E][s0 + rank1] = b2;
+                deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
+                deposit_add_global(P.Qb[SP_OP], b2.x, inv_dx, Nc);
+            } else if (bkind == 2) {
+                P.stage[B_OM_FROM_E][s0 + rank2] = b1;
+                deposit_add_global(P.Qb[SP_OM], b1.x, inv_dx, Nc);
+            }
+            if (pool) break;
+            nb1 += __popc(m1);
+            nb2 += __popc(m2);
+        }
+        if (births && tid < WARPS) {
+            P.wcount[B_E_FROM_E][blk * WARPS + tid] = sh.nb1[tid] + bits_between(sh.m1, sh.start[tid], sh.start[tid + 1]);
+            P.wcount[B_OM_FROM_E][blk * WARPS + tid] = sh.nb2[tid] + bits_between(sh.m2, sh.start[tid], sh.start[tid + 1]);
         }
     } else if (lane == 0) {
         P.ccount[S][gw] = nrec;
@@ -741,7 +796,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     if (wemax) atomicAdd(&C->cnt.warn_emax, (unsigned long long)wemax);
     if (wnumax) atomicAdd(&C->cnt.warn_numax, (unsigned long long)wnumax);
     __syncthreads();
-    if (fused && tid < np && sh.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)sh.events[tid]);
+    if (electrons && tid < np && sh.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)sh.events[tid]);
     // one 64-bit add per node: what its two cells give it
     for (int j = tid; j < Ng; j += BLOCK) {
         unsigned long long v = 0ull;
@@ -882,25 +937,22 @@ constexpr int SEGS = 32 / SEG;
 template <int S>
 __device__ __forceinline__ void cand_body(const Params& P, unsigned blk, unsigned nblk) {
     __shared__ unsigned events[MAXPROC];
-    __shared__ unsigned sh_removed, sh_wtries, sh_wemax;
+    __shared__ unsigned sh_removed, sh_wtries;
     const int np = P.nproc[S];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned seg = (unsigned)lane / SEG, sl = (unsigned)lane % SEG;
     const unsigned seg_mask = ((1u << SEG) - 1u) << (seg * SEG);
     const unsigned lt_mask = ((1u << lane) - 1u) & seg_mask;   // lanes below, same half-warp
     if (tid < MAXPROC) events[tid] = 0u;
-    if (tid == 0) { sh_removed = 0u; sh_wtries = 0u; sh_wemax = 0u; }
+    if (tid == 0) { sh_removed = 0u; sh_wtries = 0u; }
     __syncthreads();
 
     DevCtrl* C = P.ctrl;
     const unsigned long long step = C->step;
     const unsigned nslots = (unsigned)((C->slots[S] < P.sp[S].cap) ? C->slots[S] : P.sp[S].cap);
-    const bool births = P.births_possible[S] != 0;
-    unsigned* cnt1 = (S == SP_E) ? P.wcount[B_E_FROM_E] : nullptr;
-    unsigned* cnt2 = (S == SP_E) ? P.wcount[B_OM_FROM_E] : (S == SP_OM ? P.wcount[B_E_FROM_OM] : nullptr);
+    const bool births = S == SP_OM && P.births_possible[S] != 0;
     const unsigned W = P.push_warps[S];
-    const PhiloxPre pre = philox_pre((uint32_t)step, SpeciesTraits<S>::tag, (uint32_t)(step >> 32), P.seed);
-    unsigned wtries = 0, wemax = 0, nremoved = 0;
+    unsigned wtries = 0, nremoved = 0;
 
     for (unsigned gb = (blk * WARPS + warp) * SEGS; gb < W; gb += nblk * WARPS * SEGS) {
         const unsigned gw = gb + seg;                  // this half-warp's list
@@ -908,24 +960,18 @@ __device__ __forceinline__ void cand_body(const Params& P, unsigned blk, unsigne
         const unsigned r0 = valid ? list_start<S>(gw, W, nslots) : 0u;
         const unsigned n = valid ? P.ccount[S][gw] : 0u;
         const unsigned nmax = max(n, __shfl_xor_sync(0xffffffffu, n, SEG));
-        unsigned nb1 = 0, nb2 = 0;   // half-warp-uniform
-        collide_list<S, SEG>(P, P.cum[S], pre, step, r0, n, nmax, sl, seg_mask, lt_mask, events, nullptr, nullptr,
-                             nullptr, nb1, nb2, nremoved, wtries, wemax);
-        if (births && valid && sl == 0) {
-            if (cnt1) cnt1[gw] = nb1;
-            if (cnt2) cnt2[gw] = nb2;
-        }
+        unsigned nb = 0;   // half-warp-uniform
+        collide_list<S, SEG>(P, step, r0, n, nmax, sl, seg_mask, lt_mask, events, nb, nremoved, wtries);
+        if (births && valid && sl == 0) P.wcount[B_E_FROM_OM][gw] = nb;
     }
     pdl_trigger();
     if (nremoved) atomicAdd(&sh_removed, nremoved);
     if (wtries) atomicAdd(&sh_wtries, wtries);
-    if (wemax) atomicAdd(&sh_wemax, wemax);
     __syncthreads();
     if (tid < np && events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)events[tid]);
     if (tid == 0) {
         if (sh_removed) atomicAdd(&C->removed[S], (unsigned long long)sh_removed);
         if (sh_wtries) atomicAdd(&C->cnt.warn_tries, (unsigned long long)sh_wtries);
-        if (sh_wemax) atomicAdd(&C->cnt.warn_emax, (unsigned long long)sh_wemax);
     }
 }
 
@@ -1026,14 +1072,8 @@ __global__ void __launch_bounds__(BLOCK) k_deposit(Params P) {
 
 size_t push_smem_bytes(int species, const Params& P) {
     const size_t base = align16(sizeof(PushShared)) + (sizeof(float) + 2 * sizeof(unsigned)) * P.Ng + sizeof(PushQueue);
-    if (!(species == SP_E || O2PIC_FUSE_IONS)) return base;
-    const size_t table = P.cum_smem[species] ? sizeof(float) * NGRID * (size_t)P.nproc[species] : 0;
-    return base + sizeof(float) * NGRID + table;
+    return base + (species == SP_E ? sizeof(float) * NGRID : 0);
 }
-
-bool ions_fused() { return O2PIC_FUSE_IONS != 0; }
-
-bool cum_smem_allowed() { return O2PIC_CUM_SMEM != 0; }
 
 void launch_flight_init(int species, const Params& P, cudaStream_t s) {
     const unsigned long long cap = P.sp[species].cap;

@@ -357,12 +357,12 @@ void enqueue_steps(o2pic_ctx* c, uint64_t nsteps, cudaStream_t s) {
         launch(c, KK_PUSH_E, s, [&] { launch_push(SP_E, P, c->grid_push[SP_E], s); });
         if (ion) {
             launch(c, KK_PUSH_OM, so, [&] { launch_push(SP_OM, P, c->grid_push[SP_OM], so); });
-            if (P.nproc[SP_OM] && !ions_fused()) {
+            if (P.nproc[SP_OM]) {
                 launch(c, KK_FILT_OM, so, [&] { launch_filter(SP_OM, P, c->grid_push[SP_OM], so); });
                 launch(c, KK_CAND_OM, so, [&] { launch_cand(SP_OM, P, c->grid_push[SP_OM], so); });
             }
             launch(c, KK_PUSH_OP, sp2, [&] { launch_push(SP_OP, P, c->grid_push[SP_OP], sp2); });
-            if (P.nproc[SP_OP] && !ions_fused()) {
+            if (P.nproc[SP_OP]) {
                 launch(c, KK_FILT_OP, sp2, [&] { launch_filter(SP_OP, P, c->grid_push[SP_OP], sp2); });
                 launch(c, KK_CAND_OP, sp2, [&] { launch_cand(SP_OP, P, c->grid_push[SP_OP], sp2); });
             }
@@ -564,16 +564,11 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     TRY(ctx_alloc(c, &c->d_gcount, 1));
     // kernel shared-memory opt-in and launch shapes
     size_t smax = 0;
-    for (int s = 0; s < NSP; ++s) {
-        P.nproc[s] = MAXPROC;
-        P.cum_smem[s] = 1;
-        smax = std::max(smax, push_smem_bytes(s, P));
-    }
+    for (int s = 0; s < NSP; ++s) smax = std::max(smax, push_smem_bytes(s, P));
     smax = std::max(smax, sizeof(unsigned) * (size_t)Ng);
     TRY(configure_push_smem(smax));
     TRY(configure_field_smem(field_smem_bytes(P)));
     TRY(configure_pair_hist_smem(Nc));
-    for (int s = 0; s < NSP; ++s) { P.nproc[s] = 0; P.cum_smem[s] = 0; }
     c->grid_pair = (int)std::max<unsigned long long>(1, std::min<unsigned long long>(tiles_ion, 8ull * c->num_sms));
     c->grid_pair_e = (int)std::max<unsigned long long>(
         1, std::min<unsigned long long>(ceil_div(cfg->capacity[SP_E], TILE) + 1, 8ull * c->num_sms));
@@ -745,15 +740,8 @@ int o2pic_set_processes(o2pic_ctx* c, const o2pic_process* procs, int nproc) {
     if (e != cudaSuccess) return cuda_fail(c, e);
     for (int s = 0; s < NSP; ++s) {
         int bps = 0;
-        P.cum_smem[s] = 0;
         if (push_occupancy(s, P, &bps) || bps < 1) bps = 1;
         if (bps > MAX_PUSH_BLOCKS_PER_SM) bps = MAX_PUSH_BLOCKS_PER_SM;
-        // the kinematics' table in shared memory when the blocks per SM stay
-        if (cum_smem_allowed() && P.nproc[s] > 0 && (s == SP_E || ions_fused())) {
-            int b2 = 0;
-            P.cum_smem[s] = 1;
-            if (push_occupancy(s, P, &b2) || std::min(b2, MAX_PUSH_BLOCKS_PER_SM) < bps) P.cum_smem[s] = 0;
-        }
         c->grid_push[s] = std::max(bps * c->num_sms, min_push_blocks(P.sp[s].cap));
         P.push_warps[s] = (unsigned)c->grid_push[s] * (BLOCK / 32);
     }
@@ -1327,11 +1315,9 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
             for (int sp = SP_OM; sp <= SP_OP; ++sp) {
                 launch_push_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], b->smem_push, s);
                 launches += 1;
-                if (!ions_fused()) {
-                    launch_filter_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
-                    launch_cand_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
-                    launches += 2;
-                }
+                launch_filter_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
+                launch_cand_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
+                launches += 2;
             }
             if (b->any_edet) {
                 launch_pair_hist_batched(b->dP, b->dD, b->dmap + b->map_dh, b->nb_dh, b->smem_hist, s);
