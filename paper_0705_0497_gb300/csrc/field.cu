@@ -26,22 +26,48 @@ namespace o2 {
 
 namespace {
 
-// The end-of-step kernel is two independent blocks of FT threads, each on its
-// own SM (twice the memory-level parallelism of one): block 0 commits the
-// charge and solves the field, block 1 places the births and commits the step.
-// They share nothing; block 0 keeps its own copy of the step counter
-// (field_step) for U sin(2 pi f t).
-constexpr int FT = 512;
-constexpr int GA = FT;                            // threads of the charge block
-constexpr int GB = FT;                            // threads of the births block
+// The end-of-step kernel is two independent clusters of FC blocks of FT threads
+// (one pair per discharge of a batched launch): cluster 0 commits the charge
+// and solves the field, cluster 1 places the births and commits the step.  They
+// share nothing; cluster 0 keeps its own copy of the step counter (field_step)
+// for U sin(2 pi f t).
+//
+// Bound by latency (a few dependent L2 round trips of 0.45 us) and, in a
+// single block, by one SM's FP64 and int64 conversion rate (513 nodes: 0.8
+// us) and outstanding misses.  So the nodes, and the births, are spread over
+// the FC SMs of a cluster; the field's blocks exchange their partial sums
+// once through distributed shared memory, and the births' blocks each scan
+// all counts (a thread takes whole particle-kernel blocks of 8 warps).  512
+// cells: 13.3 us between events (two blocks of 512 threads) -> 10.5, of which
+// the launch is about 4.8; 2048 cells 26 -> 12.6.
+constexpr int FT = 256;
+constexpr int FC = 8;                             // blocks of a cluster
+constexpr int FW = FT / 32;
+constexpr int FN = (MAX_NODES + FC * FT - 1) / (FC * FT);   // nodes per thread, at most (5)
+constexpr int PW = BLOCK / 32;                    // warps of a particle-kernel block
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v into the same shared-memory word of block `rank` of the cluster
+__device__ __forceinline__ void store_remote(long long* p, unsigned rank, long long v) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("{ .reg .b32 r; mapa.shared::cluster.u32 r, %0, %1; st.shared::cluster.s64 [r], %2; }" ::"r"(a),
+                 "r"(rank), "l"(v)
+                 : "memory");
+}
 
 // Births of one step, placed in the order the method defines (source species
 // e then O-, parent order, e before O2+ for an ionization): each warp of a
 // particle kernel staged the births of its slot range [u R, ...) with their
 // count (their charge already went to Qb there).  The counts are scanned into
-// per-warp offsets in shared memory, and every thread of the births block
-// then places single births (found by a binary search over the offsets), so
-// the work spreads over the block however the births cluster.
+// per-block offsets in shared memory, and every thread of the births cluster
+// then places single births (found by a binary search over the offsets and the
+// counts of the block's warps), so the work spreads however the births cluster.
 // A newborn of step n starts a free flight at its first push after n (step
 // n + 1 for electrons, the next ion step for ions), drawn from its own stream
 // at step n with tag TAG_FLIGHT + d.
@@ -69,14 +95,13 @@ __device__ void place_birth(const Params& P, DevCtrl* C, const unsigned cur[NSP]
     B.tc[cb][slot] = nf + sub * flight_gap(w.x, P.inv_lnq[d], P.kcap[d]);
 }
 
-// Exclusive scan over the births block of two 64-bit values per thread, with
-// the totals.
-__device__ __forceinline__ void groupB_excl_scan_pair(unsigned long long v, unsigned long long w,
-                                                      unsigned long long* ws, unsigned long long& ev,
-                                                      unsigned long long& ew, unsigned long long& tv,
-                                                      unsigned long long& tw) {
-    const int tB = threadIdx.x, lane = tB & 31, warp = tB >> 5;
-    constexpr int NW = GB / 32;
+// Exclusive scan over the block of two 64-bit values per thread (words: two
+// 32-bit counts each), with the totals.
+__device__ __forceinline__ void block_excl_scan_pair(unsigned long long v, unsigned long long w,
+                                                     unsigned long long* ws, unsigned long long& ev,
+                                                     unsigned long long& ew, unsigned long long& tv,
+                                                     unsigned long long& tw) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long x = v, y = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -84,113 +109,46 @@ __device__ __forceinline__ void groupB_excl_scan_pair(unsigned long long v, unsi
         const unsigned long long yo = __shfl_up_sync(0xffffffffu, y, o);
         if (lane >= o) { x += xo; y += yo; }
     }
-    if (lane == 31) { ws[warp] = x; ws[NW + warp] = y; }
+    if (lane == 31) { ws[warp] = x; ws[FW + warp] = y; }
     __syncthreads();
-    if (warp == 0) {
-        unsigned long long a = (lane < NW) ? ws[lane] : 0ull, b = (lane < NW) ? ws[NW + lane] : 0ull;
+    ev = x - v;
+    ew = y - w;
+    tv = tw = 0ull;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long ao = __shfl_up_sync(0xffffffffu, a, o);
-            const unsigned long long bo = __shfl_up_sync(0xffffffffu, b, o);
-            if (lane >= o) { a += ao; b += bo; }
+    for (int k = 0; k < FW; ++k) {
+        const unsigned long long a = ws[k], b = ws[FW + k];
+        if (k < warp) { ev += a; ew += b; }
+        tv += a;
+        tw += b;
+    }
+}
+
+// The birth counts of one particle-kernel block's PW warps.
+struct WarpCounts {
+    uint4 a, b;
+    __device__ __forceinline__ void load(const unsigned* c, unsigned blk) {
+        const uint4* p = reinterpret_cast<const uint4*>(c + (size_t)blk * PW);
+        a = p[0];
+        b = p[1];
+    }
+    __device__ __forceinline__ unsigned sum() const { return a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w; }
+    // the warp that staged the block's birth number r (r < sum()); r becomes its
+    // rank among that warp's
+    __device__ __forceinline__ unsigned warp_of(unsigned& r) const {
+        const unsigned n[PW] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        unsigned u = 0;
+        bool found = false;
+#pragma unroll
+        for (int k = 0; k < PW; ++k) {
+            if (!found && r < n[k]) { u = k; found = true; }
+            if (!found) r -= n[k];
         }
-        if (lane < NW) { ws[lane] = a; ws[NW + lane] = b; }
+        return u;
     }
-    __syncthreads();
-    ev = (warp == 0 ? 0ull : ws[warp - 1]) + x - v;
-    ew = (warp == 0 ? 0ull : ws[NW + warp - 1]) + y - w;
-    tv = ws[NW - 1];
-    tw = ws[2 * NW - 1];
-    __syncthreads();
-}
+};
+static_assert(PW == 8, "two 16-byte words of counts per block");
 
-// Offsets of the per-warp birth counts: c1, c2 of the electron kernel's nu1
-// warps into p1, p2 [0..nu1], c3 of the O- kernel's nu3 warps into p3
-// [0..nu3] (nu1 or nu3 may be 0), by one scan over the births block; returns
-// the totals (c1 | c2 << 32 and c3).  A thread owns a range of a multiple of 4
-// units, read as 16-byte vectors (the count arrays are 256-byte aligned).
-__device__ __forceinline__ void unit_range(unsigned nu, unsigned& u0, unsigned& u1) {
-    const unsigned tB = threadIdx.x;
-    const unsigned per = (((nu + GB - 1) / GB) + 3u) & ~3u;
-    u0 = tB * per < nu ? tB * per : nu;
-    u1 = (u0 + per < nu) ? u0 + per : nu;
-}
-
-__device__ __forceinline__ uint4 count4(const unsigned* c, unsigned u, unsigned nu) {
-    if (u + 4 <= nu) return *reinterpret_cast<const uint4*>(c + u);
-    uint4 r = make_uint4(0u, 0u, 0u, 0u);
-    if (u < nu) r.x = c[u];
-    if (u + 1 < nu) r.y = c[u + 1];
-    if (u + 2 < nu) r.z = c[u + 2];
-    return r;
-}
-
-__device__ void unit_offsets(const unsigned* c1, const unsigned* c2, unsigned nu1, const unsigned* c3, unsigned nu3,
-                             unsigned* p1, unsigned* p2, unsigned* p3, unsigned long long* ws,
-                             unsigned long long& tot12, unsigned long long& tot3) {
-    const int tB = threadIdx.x;
-    unsigned u0, u1;
-    unit_range(nu1 > nu3 ? nu1 : nu3, u0, u1);
-    unsigned long long m12 = 0, m3 = 0;
-    for (unsigned ub = u0; ub < u1; ub += 8) {
-        uint4 a[2], b[2], d[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {       // all loads first
-            const unsigned u = ub + 4u * k;
-            const bool in = u < u1;
-            a[k] = in ? count4(c1, u, nu1) : make_uint4(0u, 0u, 0u, 0u);
-            b[k] = in ? count4(c2, u, nu1) : make_uint4(0u, 0u, 0u, 0u);
-            d[k] = in ? count4(c3, u, nu3) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const unsigned u = ub + 4u * k;
-            const unsigned av[4] = {a[k].x, a[k].y, a[k].z, a[k].w}, bv[4] = {b[k].x, b[k].y, b[k].z, b[k].w},
-                           dv[4] = {d[k].x, d[k].y, d[k].z, d[k].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const bool mine = u + e < u1;   // the next thread's units are its own
-                if (mine && u + e < nu1) { p1[u + e] = av[e]; p2[u + e] = bv[e]; }
-                if (mine && u + e < nu3) p3[u + e] = dv[e];
-                m12 += (unsigned long long)av[e] | ((unsigned long long)bv[e] << 32);
-                m3 += dv[e];
-            }
-        }
-    }
-    unsigned long long e12, e3;
-    groupB_excl_scan_pair(m12, m3, ws, e12, e3, tot12, tot3);
-    unsigned r1 = (unsigned)e12, r2 = (unsigned)(e12 >> 32), r3 = (unsigned)e3;
-    for (unsigned u = u0; u < u1; ++u) {
-        if (u < nu1) { const unsigned x = p1[u], y = p2[u]; p1[u] = r1; p2[u] = r2; r1 += x; r2 += y; }
-        if (u < nu3) { const unsigned z = p3[u]; p3[u] = r3; r3 += z; }
-    }
-    if (tB == 0) { p1[nu1] = (unsigned)tot12; p2[nu1] = (unsigned)(tot12 >> 32); p3[nu3] = (unsigned)tot3; }
-    __syncthreads();
-}
-
-// Start moving a line into this SM's L1 (the loads that follow hit it).
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-// Prefetch a births-block thread's share [u0, u1) of the per-warp counts
-// (the lines of its first and last unit: a share spans at most two lines
-// while it holds at most 32 units).
-__device__ __forceinline__ void prefetch_units(const unsigned* c1, const unsigned* c2, unsigned nu1, const unsigned* c3,
-                                               unsigned nu3) {
-    unsigned u0, u1;
-    unit_range(nu1 > nu3 ? nu1 : nu3, u0, u1);
-    if (u0 >= u1) return;
-    const unsigned ends[2] = {u0, u1 - 1};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const unsigned u = ends[k];
-        if (u < nu1) { prefetch_l1(c1 + u); prefetch_l1(c2 + u); }
-        if (u < nu3) prefetch_l1(c3 + u);
-    }
-}
-
-// The warp that staged birth number b (largest u with p[u] <= b).
+// The block whose births hold number b (largest u with p[u] <= b).
 __device__ __forceinline__ unsigned find_unit(const unsigned* p, unsigned nu, unsigned b) {
     unsigned lo = 0, hi = nu;
     while (hi - lo > 1) {
@@ -206,246 +164,248 @@ struct CtrlSnap {
     unsigned cur[NSP], removals, births22;
 };
 
-// Over the charge block: the inclusive scan S_j of R_j held in a[0..n)
-// (a[0] = 0; in place), and U_j = sum_{k<=j} k R_k straight to global U[j]
-// (its only readers are the potential and D0, which gets U_{n-2} in *u_last).
-// Blocked: thread t owns [t*per, (t+1)*per); the two scans share their
-// warp shuffles and barriers.
-__device__ __forceinline__ void groupA_scan_SU(long long* a, int n, long long* ws, long long* U, long long* u_last) {
-    const int t = threadIdx.x;
-    const int per = (n + GA - 1) / GA;
-    const int j0 = t * per;
-    long long ra = 0, rb = 0;
-    for (int i = 0; i < per; ++i) {
+// The charge commit, cycle moments and field solve of one block (rank cr) of
+// the field cluster: nodes [cr per, (cr + 1) per), a few neighbouring ones per
+// thread.  mode 0: end of a step (pushed_mask = species pushed this step);
+// mode 1: after a load (all species freshly deposited into Qf).
+__device__ __forceinline__ void field_solve(const Params& P, int mode, int pushed_mask, unsigned cr) {
+    __shared__ long long ws[2 * FW];
+    __shared__ long long part[2 * FC];     // the cluster's partial sums, written by its blocks
+    DevCtrl* C = P.ctrl;
+    const int N = P.Nc, Ng = P.Ng;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (Ng + FC - 1) / FC, pt = (per + FT - 1) / FT;
+    const int c0 = (int)cr * per, c1 = min(Ng, c0 + per), j0 = c0 + t * pt;
+    cluster_arrive();                      // this block runs (before others write to its shared memory)
+    // U sin(2 pi f t) at t^{n+1} (end of step) or t^n (after a load), evaluated
+    // on the host in FP64 and staged in a ring indexed by the step; D0 needs it
+    // in one lane per warp
+    unsigned long long fstep = 0ull;
+    double V0 = 0.0;
+    if (lane == 0) fstep = C->field_step;
+    // Q = (this step's deposit Qf, or the kept Q of a species not pushed) + the
+    // births' deposit Qb, and the cycle moments Qacc += Q
+    long long r[FN], net[FN];
+#pragma unroll
+    for (int i = 0; i < FN; ++i) {
         const int j = j0 + i;
-        if (j < n) { const long long r = a[j]; ra += r; a[j] = ra; rb += (long long)j * r; }
+        r[i] = 0;
+        net[i] = 0;
+        if (i >= pt || j >= c1) continue;
+        unsigned long long q[NSP], qa[NSP];
+#pragma unroll
+        for (int s = 0; s < NSP; ++s) {
+            qa[s] = (mode == 0) ? P.Qacc[s][j] : 0ull;
+            unsigned long long v = P.Qb[s][j];
+            if ((mode == 1) || ((pushed_mask >> s) & 1)) {
+#pragma unroll
+                for (int k = 0; k < QCOPIES; ++k) v += P.Qf[s][(size_t)k * Ng + j];
+            } else {
+                v += P.Q[s][j];
+            }
+            q[s] = v;
+        }
+#pragma unroll
+        for (int s = 0; s < NSP; ++s) {
+            P.Q[s][j] = q[s];
+            if (mode == 0) P.Qacc[s][j] = qa[s] + q[s];
+            P.Qf[s][j] = 0ull;
+            if ((mode == 1) || ((pushed_mask >> s) & 1)) {   // only pushes fill copies 1..
+#pragma unroll
+                for (int k = 1; k < QCOPIES; ++k) P.Qf[s][(size_t)k * Ng + j] = 0ull;
+            }
+            P.Qb[s][j] = 0ull;
+            net[i] += (s == SP_OP) ? (long long)q[s] : -(long long)q[s];
+        }
+        if (j >= 1 && j < N) r[i] = net[i];
     }
-    const int lane = t & 31, warp = t >> 5;
-    long long xa = ra, xb = rb;
+    // the scans of R_j and j R_j (j = 1 .. N - 1) over the cluster
+    long long a = 0, b = 0;
+#pragma unroll
+    for (int i = 0; i < FN; ++i) { a += r[i]; b += (long long)(j0 + i) * r[i]; }
+    long long xa = a, xb = b;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const long long ya = __shfl_up_sync(0xffffffffu, xa, o);
         const long long yb = __shfl_up_sync(0xffffffffu, xb, o);
         if (lane >= o) { xa += ya; xb += yb; }
     }
-    if (lane == 31) { ws[warp] = xa; ws[32 + warp] = xb; }
+    if (lane == 31) { ws[warp] = xa; ws[FW + warp] = xb; }
+    if (lane == 0) V0 = P.vring[(mode == 0 ? fstep + 1 : fstep) & P.vring_mask];
     __syncthreads();
-    if (warp == 0) {
-        long long va = (lane < GA / 32) ? ws[lane] : 0, vb = (lane < GA / 32) ? ws[32 + lane] : 0;
+    long long sa = xa - a, sb = xb - b;    // exclusive, over the block
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long ya = __shfl_up_sync(0xffffffffu, va, o);
-            const long long yb = __shfl_up_sync(0xffffffffu, vb, o);
-            if (lane >= o) { va += ya; vb += yb; }
-        }
-        if (lane < GA / 32) { ws[lane] = va; ws[32 + lane] = vb; }
+    for (int k = 0; k < FW - 1; ++k)
+        if (k < warp) { sa += ws[k]; sb += ws[FW + k]; }
+    cluster_wait();
+    if (t < 2 * FC) {
+        const int h = t & 1;               // 0: S, 1: U
+        long long tot = 0;
+#pragma unroll
+        for (int k = 0; k < FW; ++k) tot += ws[h * FW + k];
+        store_remote(&part[h * FC + cr], (unsigned)t >> 1, tot);
     }
-    __syncthreads();
-    const long long offa = (warp == 0 ? 0 : ws[warp - 1]) + (xa - ra);
-    const long long offb = (warp == 0 ? 0 : ws[32 + warp - 1]) + (xb - rb);
-    long long prev = 0, ub = 0;
-    for (int i = 0; i < per; ++i) {
+    cluster_arrive();
+    cluster_wait();
+    long long ta = 0, tb = 0;              // over the cluster: S_{N-1}, U_{N-1}
+#pragma unroll
+    for (int k = 0; k < FC; ++k) {
+        const long long pa = part[k], pb = part[FC + k];
+        if (k < (int)cr) { sa += pa; sb += pb; }
+        ta += pa;
+        tb += pb;
+    }
+    // D0 in one lane per warp: FP64 throughput on this GPU is low
+    const double c = P.c_field;
+    double D0 = 0.0;
+    if (lane == 0) {
+        const long long TN = (long long)N * ta - tb;
+        // a power-of-two N divides exactly by its reciprocal (same IEEE
+        // result as the division, which is slow in FP64 here)
+        const double num = c * (double)TN - V0;
+        D0 = (P.inv_Nc64 != 0.0) ? num * P.inv_Nc64 : num / (double)N;
+        if (cr == 0 && warp == 0) {
+            P.fVD[0] = V0;
+            P.fVD[1] = D0;
+            if (mode == 0) C->field_step = fstep + 1;   // read by this cluster only, before its barrier
+        }
+    }
+    D0 = __shfl_sync(0xffffffffu, D0, 0);
+    // E on the nodes (what the next push gathers).  The potential needs as
+    // much FP64 work again and only diagnostics read it: S, U, V0 and D0
+    // are kept so that k_phi evaluates it with the same expressions.
+    const double D2 = 2.0 * D0;            // exact
+#pragma unroll
+    for (int i = 0; i < FN; ++i) {
         const int j = j0 + i;
-        if (j < n) {
-            const long long sl = a[j];          // thread-local inclusive S
-            ub += (long long)j * (sl - prev);
-            prev = sl;
-            a[j] = sl + offa;
-            U[j] = ub + offb;
-            if (j == n - 2) *u_last = ub + offb;
-        }
+        if (i >= pt || j >= c1) continue;
+        const long long below = sa;        // S_{j-1}
+        sa += r[i];
+        sb += (long long)j * r[i];
+        double E;
+        if (j == 0) E = (-D0 - c * (double)net[i]) * P.inv_dx64;
+        else if (j == N) E = (c * (double)ta - D0 + c * (double)net[i]) * P.inv_dx64;
+        else E = (c * (double)(sa + below) - D2) * P.inv_2dx64;
+        P.Ef[j] = (float)E;
+        P.fS[j] = sa;
+        P.fU[j] = sb;
     }
-    __syncthreads();
 }
 
-// mode 0: end of a step (pushed_mask = species pushed this step);
-// mode 1: after a load (all species freshly deposited into Qf).
-// Dynamic shared memory: S as int64 [Ng] (charge group), then three u32
-// [max warps + 1] (births group).
-__device__ __forceinline__ void field_body(const Params& P, int mode, int pushed_mask, int role) {
-    extern __shared__ long long fsm[];
-    __shared__ long long wsA[64];
-    __shared__ unsigned long long wsB[2 * (GB / 32)];
+// Births, (17) removals and the commit of the step, by one block (rank cr) of
+// the births cluster.  Dynamic shared memory: three u32 [units + 1].
+__device__ __forceinline__ void step_commit(const Params& P, int mode, int pushed_mask, unsigned cr) {
+    __shared__ unsigned long long ws[2 * FW];
     __shared__ CtrlSnap cs;
-    __shared__ long long sh_R0, sh_RN, sh_UN1;
-    __shared__ double sh_V0, sh_D0;
-    __shared__ unsigned long long sh_fstep;
+    extern __shared__ unsigned fsm[];
     DevCtrl* C = P.ctrl;
-    const int N = P.Nc, Ng = P.Ng;
-    const int t = threadIdx.x;
-
-    if (role == 0) {
-        // ================= charge commit, cycle moments, field solve
-        long long* Ss = fsm;          // S_j = sum_{k=1..j} R_k   (T_j = j S_{j-1} - U_{j-1})
-        if (t == 0) {
-            // U sin(2 pi f t) at t^{n+1} (end of step) or t^n (after a load),
-            // evaluated on the host in FP64 and staged in a ring indexed by
-            // the step
-            const unsigned long long fstep = C->field_step;
-            sh_fstep = fstep;
-            sh_V0 = P.vring[(mode == 0 ? fstep + 1 : fstep) & P.vring_mask];
-        }
-        // Q = (this step's deposit Qf, or the kept Q of a species not pushed)
-        // + the births' deposit Qb, and the cycle moments Qacc += Q; two
-        // nodes per thread with all their loads issued before any store
-        for (int j0 = t; j0 < Ng; j0 += 2 * GA) {
-            unsigned long long q[2][NSP], qa[2][NSP];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = j0 + h * GA;
-#pragma unroll
-                for (int s = 0; s < NSP; ++s) {
-                    q[h][s] = 0ull;
-                    qa[h][s] = 0ull;
-                    if (j < Ng) {
-                        if (mode == 0) qa[h][s] = P.Qacc[s][j];
-                        const bool fresh = (mode == 1) || ((pushed_mask >> s) & 1);
-                        unsigned long long v = P.Qb[s][j];
-                        if (fresh) {
-#pragma unroll
-                            for (int k = 0; k < QCOPIES; ++k) v += P.Qf[s][(size_t)k * Ng + j];
-                        } else {
-                            v += P.Q[s][j];
-                        }
-                        q[h][s] = v;
-                    }
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = j0 + h * GA;
-                if (j >= Ng) continue;
-                long long net = 0;
-#pragma unroll
-                for (int s = 0; s < NSP; ++s) {
-                    P.Q[s][j] = q[h][s];
-                    if (mode == 0) P.Qacc[s][j] = qa[h][s] + q[h][s];
-                    P.Qf[s][j] = 0ull;
-                    if ((mode == 1) || ((pushed_mask >> s) & 1)) {   // only pushes fill copies 1..
-#pragma unroll
-                        for (int k = 1; k < QCOPIES; ++k) P.Qf[s][(size_t)k * Ng + j] = 0ull;
-                    }
-                    P.Qb[s][j] = 0ull;
-                    net += (s == SP_OP) ? (long long)q[h][s] : -(long long)q[h][s];
-                }
-                Ss[j] = (j >= 1) ? net : 0;                    // scanned below
-                if (j == 0) sh_R0 = net;
-                if (j == N) sh_RN = net;
-            }
-        }
-        __syncthreads();
-        groupA_scan_SU(Ss, Ng, wsA, P.fU, &sh_UN1);
-        const double c = P.c_field;
-        // D0 once per block: FP64 throughput on this GPU is low
-        if (t == 0) {
-            const long long TN = (long long)N * Ss[N - 1] - sh_UN1;
-            // a power-of-two N divides exactly by its reciprocal (same IEEE
-            // result as the division, which is slow in FP64 here)
-            const double num = c * (double)TN - sh_V0;
-            const double D0 = (P.inv_Nc64 != 0.0) ? num * P.inv_Nc64 : num / (double)N;
-            sh_D0 = D0;
-            P.fVD[0] = sh_V0;
-            P.fVD[1] = D0;
-            if (mode == 0) C->field_step = sh_fstep + 1;   // only this block reads it
-        }
-        __syncthreads();
-        // E on the nodes (what the next push gathers).  The potential needs as
-        // much FP64 work again and only diagnostics read it: S, U, V0 and D0
-        // are kept so that k_phi evaluates it with the same expressions.
-        const double D0 = sh_D0, D2 = 2.0 * sh_D0;   // 2 D0 is exact
-        const long long R0 = sh_R0, RN = sh_RN;
-        for (int j = t; j < Ng; j += GA) {
-            double E;
-            if (j == 0) E = (-D0 - c * (double)R0) * P.inv_dx64;
-            else if (j == N) E = (c * (double)Ss[N - 1] - D0 + c * (double)RN) * P.inv_dx64;
-            else E = (c * (double)(Ss[j] + Ss[j - 1]) - D2) * P.inv_2dx64;
-            P.Ef[j] = (float)E;
-            P.fS[j] = Ss[j];
-        }
-        return;
-    }
-
-    // ===================== births, (17) removals and the commit of the step
-    const int tB = t;
-    unsigned* p1 = reinterpret_cast<unsigned*>(fsm + Ng);
-    unsigned* p2 = p1 + (P.max_push_warps + 1);
-    unsigned* p3 = p2 + (P.max_push_warps + 1);
+    const int N = P.Nc, t = threadIdx.x;
+    const unsigned ct = cr * FT + (unsigned)t;            // thread of the cluster
+    constexpr unsigned CT = FC * FT;
+    unsigned* p1 = fsm;
+    unsigned* p2 = p1 + (P.max_push_warps / PW + 1);
+    unsigned* p3 = p2 + (P.max_push_warps / PW + 1);
     const bool births_e = mode == 0 && P.births_possible[SP_E];
     const bool births_om = mode == 0 && ((pushed_mask >> SP_OM) & 1) && P.births_possible[SP_OM];
-    if (tB < NSP) {
-        cs.slots[tB] = C->slots[tB]; cs.live[tB] = C->live[tB]; cs.removed[tB] = C->removed[tB];
-        cs.next_id[tB] = C->next_id[tB]; cs.cur[tB] = C->cur[tB];
-    } else if (tB == 32) {
+    if (t < NSP) {
+        cs.slots[t] = C->slots[t]; cs.live[t] = C->live[t]; cs.removed[t] = C->removed[t];
+        cs.next_id[t] = C->next_id[t]; cs.cur[t] = C->cur[t];
+    } else if (t == 32) {
         cs.step = C->step;
         cs.epoch = C->epoch;
         cs.acc_steps = C->acc_steps;
         cs.removals = C->removals;
         cs.births22 = C->births22;
     }
-    prefetch_units(P.wcount[B_E_FROM_E], P.wcount[B_OM_FROM_E], births_e ? P.push_warps[SP_E] : 0u,
-                   P.wcount[B_E_FROM_OM], births_om ? P.push_warps[SP_OM] : 0u);
-    __syncthreads();
-
     // births of the step: n1 ionizations (e + O2+) and n2 attachments (O-)
     // staged by the electron kernel, n3 detachment electrons staged by the O-
     // kernel (ion steps), placed after the electrons' own, then n4 electrons
-    // of (22) staged in order by its apply kernel (ion steps)
-    unsigned long long btot[NB];
-    for (int k = 0; k < NB; ++k) btot[k] = 0;
-    const unsigned n4 = (mode == 0) ? cs.births22 : 0u;
-    if (births_e || births_om || n4) {
-        const unsigned ns1 = (unsigned)(cs.slots[SP_E] < P.sp[SP_E].cap ? cs.slots[SP_E] : P.sp[SP_E].cap);
-        const unsigned ns3 = (unsigned)(cs.slots[SP_OM] < P.sp[SP_OM].cap ? cs.slots[SP_OM] : P.sp[SP_OM].cap);
-        const unsigned nu1 = births_e ? P.push_warps[SP_E] : 0u, nu3 = births_om ? P.push_warps[SP_OM] : 0u;
-        const unsigned R1 = warp_range_len(ns1, nu1 ? nu1 : 1u), R3 = warp_range_len(ns3, nu3 ? nu3 : 1u);
-        unsigned long long t12, t3;
-        unit_offsets(P.wcount[B_E_FROM_E], P.wcount[B_OM_FROM_E], nu1, P.wcount[B_E_FROM_OM], nu3, p1, p2, p3, wsB,
-                     t12, t3);
-        const unsigned n1 = (unsigned)t12, n2 = (unsigned)(t12 >> 32), n3 = (unsigned)t3;
-        const unsigned ntot = n1 + n2 + n3 + n4;
-        // one birth per thread and pass: which list, its rank there, the warp
-        // that staged it (binary search over that list's offsets) and its
-        // staging slot; all loads of the birth before its stores
-        for (unsigned b = tB; b < ntot; b += GB) {
-            if (b >= n1 + n2 + n3) {   // (22): staged in place order
-                const unsigned r = b - n1 - n2 - n3;
-                place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + n1 + n3 + r,
-                            (unsigned long long)cs.next_id[SP_E] + n1 + n3 + r, P.stage22[r], cs.step);
-                continue;
-            }
-            const int kind = b < n1 ? 0 : (b < n1 + n2 ? 1 : 2);
-            const unsigned r = kind == 0 ? b : (kind == 1 ? b - n1 : b - n1 - n2);
-            const unsigned* p = kind == 0 ? p1 : (kind == 1 ? p2 : p3);
-            const unsigned nu = kind == 2 ? nu3 : nu1, R = kind == 2 ? R3 : R1, ns = kind == 2 ? ns3 : ns1;
-            const unsigned u = find_unit(p, nu, r);
-            const unsigned long long sb = ((unsigned long long)u * R < ns ? (unsigned long long)u * R : ns) + (r - p[u]);
-            if (kind == 0) {
-                const float4 be = P.stage[B_E_FROM_E][sb], bo = P.stage[B_OP_FROM_E][sb];
-                place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + r, (unsigned long long)cs.next_id[SP_E] + r, be,
-                            cs.step);
-                place_birth(P, C, cs.cur, SP_OP, cs.slots[SP_OP] + r, (unsigned long long)cs.next_id[SP_OP] + r, bo,
-                            cs.step);
-            } else if (kind == 1) {
-                place_birth(P, C, cs.cur, SP_OM, cs.slots[SP_OM] + r, (unsigned long long)cs.next_id[SP_OM] + r,
-                            P.stage[B_OM_FROM_E][sb], cs.step);
-            } else {
-                place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + n1 + r, (unsigned long long)cs.next_id[SP_E] + n1 + r,
-                            P.stage[B_E_FROM_OM][sb], cs.step);
-            }
+    // of (22) staged in order by its apply kernel (ion steps).  Offsets of the
+    // particle-kernel blocks' counts by one scan: a thread owns `ub`
+    // neighbouring blocks
+    const unsigned nu1 = births_e ? P.push_warps[SP_E] / PW : 0u, nu3 = births_om ? P.push_warps[SP_OM] / PW : 0u;
+    const unsigned nu = nu1 > nu3 ? nu1 : nu3, ub = (nu + FT - 1) / FT, u0 = (unsigned)t * ub;
+    unsigned long long m12 = 0, m3 = 0, t12 = 0, t3 = 0;
+    for (unsigned i = 0; i < ub; ++i) {
+        const unsigned u = u0 + i;
+        WarpCounts a, b, d;
+        if (u < nu1) { a.load(P.wcount[B_E_FROM_E], u); b.load(P.wcount[B_OM_FROM_E], u); }
+        if (u < nu3) d.load(P.wcount[B_E_FROM_OM], u);
+        if (u < nu1) {
+            const unsigned sa = a.sum(), sb = b.sum();
+            p1[u] = sa;
+            p2[u] = sb;
+            m12 += (unsigned long long)sa | ((unsigned long long)sb << 32);
         }
-        btot[B_E_FROM_E] = n1;
-        btot[B_OP_FROM_E] = n1;
-        btot[B_OM_FROM_E] = n2;
-        btot[B_E_FROM_OM] = n3 + n4;
+        if (u < nu3) { const unsigned sd = d.sum(); p3[u] = sd; m3 += sd; }
     }
-
-    if (mode == 0) {
-        // (17) removals: mark both ions of every reacted pair dead
-        const unsigned nrem = (cs.removals < P.max_removals) ? cs.removals : P.max_removals;
-        for (unsigned r = tB; r < nrem; r += GB) {
-            P.sp[SP_OM].x[cs.cur[SP_OM]][P.removal[2 * r]] = dead_marker();
-            P.sp[SP_OP].x[cs.cur[SP_OP]][P.removal[2 * r + 1]] = dead_marker();
+    unsigned long long e12, e3;
+    block_excl_scan_pair(m12, m3, ws, e12, e3, t12, t3);
+    cluster_arrive();                      // every block has its snapshot of the step state
+    {
+        unsigned r1 = (unsigned)e12, r2 = (unsigned)(e12 >> 32), r3 = (unsigned)e3;
+        for (unsigned i = 0; i < ub; ++i) {
+            const unsigned u = u0 + i;
+            if (u < nu1) { const unsigned x = p1[u], y = p2[u]; p1[u] = r1; p2[u] = r2; r1 += x; r2 += y; }
+            if (u < nu3) { const unsigned z = p3[u]; p3[u] = r3; r3 += z; }
         }
+    }
+    __syncthreads();
+    const unsigned n1 = (unsigned)t12, n2 = (unsigned)(t12 >> 32), n3 = (unsigned)t3;
+    const unsigned n4 = (mode == 0) ? cs.births22 : 0u;
+    const unsigned ntot = n1 + n2 + n3 + n4;
+    const unsigned ns1 = (unsigned)(cs.slots[SP_E] < P.sp[SP_E].cap ? cs.slots[SP_E] : P.sp[SP_E].cap);
+    const unsigned ns3 = (unsigned)(cs.slots[SP_OM] < P.sp[SP_OM].cap ? cs.slots[SP_OM] : P.sp[SP_OM].cap);
+    const unsigned R1 = warp_range_len(ns1, nu1 ? nu1 * PW : 1u), R3 = warp_range_len(ns3, nu3 ? nu3 * PW : 1u);
+    // one birth per thread and pass: which list, its rank there, the warp that
+    // staged it and its staging slot; all loads of the birth before its stores
+    for (unsigned b = ct; b < ntot; b += CT) {
+        if (b >= n1 + n2 + n3) {   // (22): staged in place order
+            const unsigned r = b - n1 - n2 - n3;
+            place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + n1 + n3 + r,
+                        (unsigned long long)cs.next_id[SP_E] + n1 + n3 + r, P.stage22[r], cs.step);
+            continue;
+        }
+        const int kind = b < n1 ? 0 : (b < n1 + n2 ? 1 : 2);
+        const unsigned r = kind == 0 ? b : (kind == 1 ? b - n1 : b - n1 - n2);
+        const unsigned* p = kind == 0 ? p1 : (kind == 1 ? p2 : p3);
+        const unsigned R = kind == 2 ? R3 : R1, ns = kind == 2 ? ns3 : ns1;
+        const unsigned blk = find_unit(p, kind == 2 ? nu3 : nu1, r);
+        WarpCounts wc;
+        wc.load(P.wcount[kind == 0 ? B_E_FROM_E : (kind == 1 ? B_OM_FROM_E : B_E_FROM_OM)], blk);
+        unsigned rank = r - p[blk];
+        const unsigned long long u = (unsigned long long)blk * PW + wc.warp_of(rank);
+        const unsigned long long sb = (u * R < ns ? u * R : ns) + rank;
+        if (kind == 0) {
+            const float4 be = P.stage[B_E_FROM_E][sb], bo = P.stage[B_OP_FROM_E][sb];
+            place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + r, (unsigned long long)cs.next_id[SP_E] + r, be,
+                        cs.step);
+            place_birth(P, C, cs.cur, SP_OP, cs.slots[SP_OP] + r, (unsigned long long)cs.next_id[SP_OP] + r, bo,
+                        cs.step);
+        } else if (kind == 1) {
+            place_birth(P, C, cs.cur, SP_OM, cs.slots[SP_OM] + r, (unsigned long long)cs.next_id[SP_OM] + r,
+                        P.stage[B_OM_FROM_E][sb], cs.step);
+        } else {
+            place_birth(P, C, cs.cur, SP_E, cs.slots[SP_E] + n1 + r, (unsigned long long)cs.next_id[SP_E] + n1 + r,
+                        P.stage[B_E_FROM_OM][sb], cs.step);
+        }
+    }
+    const unsigned long long btot[NB] = {n1, n1, n2, n3 + n4};   // by BirthSlot
+    // (17) removals: mark both ions of every reacted pair dead
+    const unsigned nrem = (mode != 0) ? 0u : (cs.removals < P.max_removals) ? cs.removals : P.max_removals;
+    for (unsigned r = ct; r < nrem; r += CT) {
+        P.sp[SP_OM].x[cs.cur[SP_OM]][P.removal[2 * r]] = dead_marker();
+        P.sp[SP_OP].x[cs.cur[SP_OP]][P.removal[2 * r + 1]] = dead_marker();
+    }
+    // per-cell totals of the pair processes: zero for the next ion step
+    if (mode != 0 || pushed_mask != 1)
+        for (unsigned k = ct; k < 2u * N; k += CT) { P.ptot[k] = 0u; P.rtot[k] = 0u; P.dtot[k] = 0u; }
+    if (mode != 0)   // the ring of conduction-current sums restarts
+        for (unsigned k = ct; k < JRING * NSP; k += CT) P.jring[k] = 0ull;
+    cluster_wait();
+    if (cr != 0) return;
+    const int tB = t;
+    if (mode == 0) {
         // commit of the step: one thread per species, then the step counters
         if (tB < NSP) {
             const int s = tB;
@@ -478,13 +438,10 @@ __device__ __forceinline__ void field_body(const Params& P, int mode, int pushed
             C->ticket[tB - 64] = 0u;
         }
     }
-    // per-cell ion totals of (17): zero for the next ion step
-    for (int k = tB; k < 2 * N; k += GB) { P.ptot[k] = 0u; P.rtot[k] = 0u; P.dtot[k] = 0u; }
-    // conduction-current sums: after a load the ring restarts; at the end of
-    // step n the ions' entries of a step without an ion push repeat those of
-    // step n-1, and the slot of step n+1 is cleared for its pushes
+    // conduction-current sums: at the end of step n the ions' entries of a step
+    // without an ion push repeat those of step n-1, and the slot of step n+1 is
+    // cleared for its pushes
     if (mode != 0) {
-        for (int k = tB; k < JRING * NSP; k += GB) P.jring[k] = 0ull;
         if (tB < NKK + NSP) C->ticket[tB] = 0u;
     } else if (tB >= 96 && tB < 96 + NSP) {
         const int sp = tB - 96;
@@ -532,19 +489,25 @@ __device__ __forceinline__ void compact_body(const Params& P, int S, CompactShar
         });
 }
 
-__global__ void __launch_bounds__(FT) k_field(Params P, int mode, int pushed_mask) {
-    pdl_wait();
-    pdl_trigger();   // two blocks on two SMs: the next step's push may take the others
-    field_body(P, mode, pushed_mask, (int)blockIdx.x);
+__device__ __forceinline__ void field_body(const Params& P, int mode, int pushed_mask, unsigned cluster) {
+    if (cluster == 0) field_solve(P, mode, pushed_mask, cluster_rank());
+    else step_commit(P, mode, pushed_mask, cluster_rank());
 }
 
-// batched: blocks 2d and 2d + 1 are the end-of-step kernel of discharge d
-__global__ void __launch_bounds__(FT) k_field_b(const Params* __restrict__ all, int mode, int pushed_mask) {
+__global__ void __cluster_dims__(FC, 1, 1) __launch_bounds__(FT) k_field(Params P, int mode, int pushed_mask) {
+    pdl_wait();
+    pdl_trigger();   // a few SMs: the next step's push may take the others
+    field_body(P, mode, pushed_mask, blockIdx.x / FC);
+}
+
+// batched: clusters 2d and 2d + 1 are the end-of-step kernel of discharge d
+__global__ void __cluster_dims__(FC, 1, 1) __launch_bounds__(FT) k_field_b(const Params* __restrict__ all, int mode,
+                                                                           int pushed_mask) {
     __shared__ Params sP;
+    load_params(sP, all + blockIdx.x / (2 * FC));
     pdl_wait();
     pdl_trigger();
-    load_params(sP, all + (blockIdx.x >> 1));
-    field_body(sP, mode, pushed_mask, (int)(blockIdx.x & 1u));
+    field_body(sP, mode, pushed_mask, (blockIdx.x / FC) & 1u);
 }
 
 // The compaction check of all species: blockIdx.y is the species.
@@ -640,7 +603,7 @@ __global__ void k_ln(const float* x, float* out, unsigned long long n) {
 }  // namespace
 
 size_t field_smem_bytes(const Params& P) {
-    return sizeof(long long) * (size_t)P.Ng + 3 * sizeof(unsigned) * ((size_t)P.max_push_warps + 1);
+    return 3 * sizeof(unsigned) * ((size_t)P.max_push_warps / PW + 1);
 }
 
 // The potential of the last field solve: phi_0 = V0, phi_N = 0,
@@ -660,7 +623,7 @@ void launch_phi(const Params& P, cudaStream_t s) {
 }
 
 void launch_field_batched(const Params* all, int n, size_t smem, int mode, int pushed_mask, cudaStream_t s) {
-    launch_pdl(k_field_b, 2 * n, FT, smem, s, all, mode, pushed_mask);
+    launch_pdl(k_field_b, 2 * FC * n, FT, smem, s, all, mode, pushed_mask);
 }
 
 void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
@@ -668,7 +631,7 @@ void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cu
 }
 
 void launch_field(const Params& P, int mode, int pushed_mask, cudaStream_t s) {
-    launch_pdl(k_field, 2, FT, field_smem_bytes(P), s, P, mode, pushed_mask);
+    launch_pdl(k_field, 2 * FC, FT, field_smem_bytes(P), s, P, mode, pushed_mask);
 }
 
 cudaError_t configure_field_smem(size_t bytes) {
