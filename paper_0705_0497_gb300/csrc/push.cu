@@ -81,7 +81,7 @@ struct PushShared {
     unsigned wtries;
     unsigned events[MAXPROC];    // electrons: real collisions per process
     // electrons: the block's pool of collisions (see push_body)
-    unsigned first[WARPS], start[WARPS + 1];   // first pooled record of each warp, its place in the pool
+    unsigned start[WARPS + 1];                 // place of each warp's first record in the pool
     unsigned nb1[WARPS], nb2[WARPS];           // births of each warp's own passes (ionizations, attachments)
     unsigned m1[WARPS], m2[WARPS];             // births of the pool, by thread
 };
@@ -167,29 +167,36 @@ __device__ __forceinline__ int collide_electron(const Params& P, const float* __
     if (E < thr) return -1;
     const int kind = P.kind[SP_E][k];
     const bool ionize = kind == K_IONIZE, attach = kind == K_ATTACH;
-    uint4 buf = w0;
+    // words come from a window of one block (w0) or two (the next ones, drawn
+    // together so that their rounds overlap); pos: the next word in it
+    uint4 lo = w0, hi = w0;
     uint32_t block = 0;
-    int pos = 2;
+    int pos = 2, words = 4;
     float u = 0.0f;
-    if (ionize) { u = uniform(buf.z); pos = 3; }
+    if (ionize) { u = uniform(lo.z); pos = 3; }
     float a0 = 0.0f, c0 = 0.0f, s0 = 0.0f, a1 = 0.0f, c1 = 0.0f, s1 = 0.0f, a2 = 0.0f, c2 = 0.0f, s2 = 0.5f,
           a3 = 0.0f, s3 = 0.5f;
     const int last_task = (ionize || attach) ? 4 : 1;
     int task = attach ? 2 : 0, tries = 0;
+    auto word = [&](int i) {
+        const uint4 q = i < 4 ? lo : hi;
+        const uint32_t e = (i & 1) ? q.y : q.x, f = (i & 1) ? q.w : q.z;
+        return (i & 2) ? f : e;
+    };
     while (task < last_task) {
-        // the next two words
-        const uint32_t held = pos == 2 ? buf.z : (pos == 3 ? buf.w : (pos == 0 ? buf.x : buf.y));
-        uint32_t wa = held, wb;
-        if (pos <= 2) {
-            wb = pos == 2 ? buf.w : (pos == 1 ? buf.z : buf.y);
+        // the next two words (the second may be the first of the next window)
+        uint32_t wa = word(pos), wb;
+        if (pos + 1 < words) {
+            wb = word(pos + 1);
             pos += 2;
         } else {
-            ++block;
-            buf = philox4x32_10(make_uint4((uint32_t)step, SpeciesTraits<SP_E>::tag, block, (uint32_t)(step >> 32)),
-                                make_uint2(id, P.seed));
-            wa = pos == 3 ? held : buf.x;
-            wb = pos == 3 ? buf.x : buf.y;
-            pos = pos == 3 ? 1 : 2;
+            const uint4 ctr = make_uint4((uint32_t)step, SpeciesTraits<SP_E>::tag, block + 1, (uint32_t)(step >> 32));
+            lo = philox4x32_10(ctr, make_uint2(id, P.seed));
+            hi = philox4x32_10(make_uint4(ctr.x, ctr.y, block + 2, ctr.w), make_uint2(id, P.seed));
+            block += 2;
+            if (pos < words) { wb = lo.x; pos = 1; }
+            else { wa = lo.x; wb = lo.y; pos = 2; }
+            words = 8;
         }
         float a = 2.0f * uniform(wa) - 1.0f;
         float b = 2.0f * uniform(wb) - 1.0f;
@@ -343,7 +350,18 @@ __device__ __forceinline__ bool electron_is_real(const Params& P, const float* t
 // Total-rate column (the last cumulative column) of species S into shared memory.
 __device__ __forceinline__ void stage_total(const Params& P, int S, float* tot) {
     const float* __restrict__ g = P.tot[S];
-    for (int i = threadIdx.x; i < NGRID; i += blockDim.x) tot[i] = g[i];
+    constexpr int K = (NGRID + BLOCK - 1) / BLOCK;
+    float v[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int i = (int)threadIdx.x + k * BLOCK;
+        v[k] = i < NGRID ? g[i] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int i = (int)threadIdx.x + k * BLOCK;
+        if (i < NGRID) tot[i] = v[k];
+    }
 }
 
 // (long long)v for |v| >= 2^31 (and infinities, NaN) in integer arithmetic: a
@@ -450,6 +468,11 @@ constexpr int QN = 32 + ROUND;
 struct PushQueue {
     unsigned slot[WARPS][QN];
 };
+// Electrons: the last records of each warp, record i of a warp at place i mod 32
+// (what is pooled is read from here, without a trip to the list in memory).
+struct PushPool {
+    uint4 a[WARPS][32], b[WARPS][32];
+};
 
 // Body of the particle kernel for block blk of nblk blocks (the launch's own
 // block, or a block a batched launch maps to this discharge).
@@ -458,7 +481,9 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     extern __shared__ __align__(16) unsigned char smem[];
     const int np = P.nproc[S];
     PushShared& sh = *reinterpret_cast<PushShared*>(smem);
-    float* Es = reinterpret_cast<float*>(smem + align16(sizeof(PushShared)));
+    PushPool& pool = *reinterpret_cast<PushPool*>(smem + align16(sizeof(PushShared)));   // electrons only
+    unsigned char* rest = smem + align16(sizeof(PushShared)) + (S == SP_E ? sizeof(PushPool) : 0);
+    float* Es = reinterpret_cast<float*>(rest);
     unsigned* cnt = reinterpret_cast<unsigned*>(Es + P.Ng);
     unsigned* rsum = cnt + P.Ng;
     PushQueue& Q = *reinterpret_cast<PushQueue*>(rsum + P.Ng);
@@ -467,6 +492,17 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned* qs = Q.slot[warp];
+    const int Nc = P.Nc, Ng = P.Ng;
+
+    // what no earlier kernel writes, before waiting for the one before
+    for (int j = tid; j < Ng; j += BLOCK) { cnt[j] = 0u; rsum[j] = 0u; }
+    if (electrons) stage_total(P, S, Tt);
+    if (tid == 0) {
+        sh.absorbed[0] = sh.absorbed[1] = 0u; sh.removed = 0u; sh.psteps = 0u; sh.nonfinite = 0u; sh.wtries = 0u;
+        sh.jsum = 0ull;
+    }
+    if (electrons && tid < MAXPROC) sh.events[tid] = 0u;
+    pdl_wait();
 
     DevCtrl* C = P.ctrl;
     const unsigned long long step = C->step;
@@ -483,7 +519,6 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const float qmdt = P.qmdt[S], dts = P.dt_s[S], inv_dx = P.inv_dx, Lf = P.Lf;
     const float inv_lnq = P.inv_lnq[S], kcap = P.kcap[S];
     const unsigned sub = P.sub[S];
-    const int Nc = P.Nc, Ng = P.Ng;
     const float jmax = cell_limit(Nc);
     unsigned long long* __restrict__ Qcopy = P.Qf[S] + (size_t)(blk & (QCOPIES - 1)) * Ng;
     const PhiloxPre pre = philox_pre(step_lo, SpeciesTraits<S>::tag, (uint32_t)(step >> 32), P.seed);
@@ -529,16 +564,17 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     };
     if (ga < gz) load_round(ga, xs, vxs, tcs);
 
-    for (int j = tid; j < Ng; j += BLOCK) { Es[j] = P.Ef[j]; cnt[j] = 0u; rsum[j] = 0u; }
-    if (electrons) stage_total(P, S, Tt);
-    if (tid == 0) {
-        sh.absorbed[0] = sh.absorbed[1] = 0u; sh.removed = 0u; sh.psteps = 0u; sh.nonfinite = 0u; sh.wtries = 0u;
-        sh.jsum = 0ull;
+    for (int j0 = tid; j0 < Ng; j0 += 4 * BLOCK) {       // four loads in flight
+        float e[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = j0 + k * BLOCK < Ng ? P.Ef[j0 + k * BLOCK] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (j0 + k * BLOCK < Ng) Es[j0 + k * BLOCK] = e[k];
     }
-    if (electrons && tid < MAXPROC) sh.events[tid] = 0u;
     __syncthreads();
 
-    unsigned psteps = 0, nabs0 = 0, nabs1 = 0, nnf = 0, wemax = 0, wtries = 0, wnumax = 0;
+    unsigned nabs0 = 0, nabs1 = 0, nnf = 0, wemax = 0, wtries = 0, wnumax = 0;
     long long jacc = 0;   // conduction current: sum of trunc(256 v_x^{n+1/2}) (exact)
     unsigned nrec = 0;    // warp-uniform: records of this warp so far
     unsigned qn = 0;      // warp-uniform: queued candidates
@@ -546,18 +582,15 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     // m (<= 32) queued candidates from entry h on, one per lane: the candidate's
     // stream at this step (block 0) draws its next free flight (word 0) and
     // the electrons' real/null test (word 1 against the total rate at the
-    // particle's energy); records go to the warp's list in slot order, two uint4 each: electrons {slot, id,
-    // x, vx}{vy, vz, -, -} per real collision, ions {slot, id, vx, vy}{vz, w1,
-    // w2, w3} per candidate.
+    // particle's energy); records go to the warp's list in slot order, two uint4
+    // each: {slot, id, vx, vy}{vz, w1, w2, w3}, electrons per real collision,
+    // ions per candidate.
     auto flush = [&](unsigned h, unsigned m) {
         const bool has = (unsigned)lane < m;
         const unsigned slot = has ? qs[h + lane] : 0u;
         uint32_t id = 0u;
-        float cx = 0.0f, cvx = 0.0f, cvy = 0.0f, cvz = 0.0f;
-        if (has) {
-            id = ID[slot]; cvx = VX[slot]; cvy = VY[slot]; cvz = VZ[slot];   // (x, v_x: as this warp just stored them)
-            if (S == SP_E) cx = X[slot];
-        }
+        float cvx = 0.0f, cvy = 0.0f, cvz = 0.0f;
+        if (has) { id = ID[slot]; cvx = VX[slot]; cvy = VY[slot]; cvz = VZ[slot]; }   // (v_x: as this warp stored it)
         bool rec = false;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         if (has) {
@@ -567,14 +600,13 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         }
         const unsigned cm = __ballot_sync(0xffffffffu, rec);
         if (rec) {
-            const size_t q = rec0 + nrec + __popc(cm & lt_mask);
-            if (S == SP_E) {
-                CAND[2 * q] = make_uint4(slot, id, __float_as_uint(cx), __float_as_uint(cvx));
-                CAND[2 * q + 1] = make_uint4(__float_as_uint(cvy), __float_as_uint(cvz), 0u, 0u);
-            } else {
-                CAND[2 * q] = make_uint4(slot, id, __float_as_uint(cvx), __float_as_uint(cvy));
-                CAND[2 * q + 1] = make_uint4(__float_as_uint(cvz), w.y, w.z, w.w);
-            }
+            const unsigned i = nrec + __popc(cm & lt_mask);
+            const size_t q = rec0 + i;
+            const uint4 a = make_uint4(slot, id, __float_as_uint(cvx), __float_as_uint(cvy));
+            const uint4 b = make_uint4(__float_as_uint(cvz), w.y, w.z, w.w);
+            CAND[2 * q] = a;
+            CAND[2 * q + 1] = b;
+            if (electrons) { pool.a[warp][i & 31u] = a; pool.b[warp][i & 31u] = b; }
         }
         nrec += __popc(cm);
     };
@@ -587,9 +619,10 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         // the four slots without branches (a dead slot's NaN falls through the
         // arithmetic and takes part in nothing); what is rare is flagged and
         // handled once per round: bit k of `out`: the particle left the gap,
-        // `wide`: its current term does not fit 32 bits, `wrap`: its weight
-        // sum wrapped, `cand`: its free flight ends at this step
-        unsigned cand = 0u, out = 0u, wide = 0u, wrap = 0u;
+        // `wrap`: its weight sum wrapped, `cand`: its free flight ends at this
+        // step; vmax: a current term may not fit 32 bits
+        unsigned cand = 0u, out = 0u, wrap = 0u;
+        float vmax = 0.0f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             float x = xs[k], vx = vxs[k];
@@ -601,11 +634,8 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
             x = fmaf(vx, dts, x);
             // exact scaling by 2^8, then truncation
             const float jv = vx * 256.0f;
-            if (live) {
-                ++psteps;
-                jacc += (long long)__float2int_rz(jv);
-                if (!(fabsf(jv) < 2147483648.0f)) wide |= 1u << k;
-            }
+            jacc += (long long)__float2int_rz(jv);       // 0 for a dead slot's NaN
+            vmax = fmaxf(vmax, fabsf(jv));               // (leaves a NaN out)
             if (x >= 0.0f && x < Lf) {
                 // (a finite x here has a finite v_x.)  CIC deposit as (count,
                 // sum of r) per cell: node c gets 2^16 count_c - rsum_c, node
@@ -623,13 +653,13 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
             xs[k] = x;
             vxs[k] = vx;
         }
-        if (out | wide | wrap) {
+        if ((out | wrap) || !(vmax < 2147483648.0f)) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                if ((wide >> k) & 1u) {
-                    const float jv = vxs[k] * 256.0f;
+                // (a NaN here is a particle's, not a dead slot's, if it is in `out`)
+                const float jv = vxs[k] * 256.0f;
+                if (fabsf(jv) >= 2147483648.0f || (((out >> k) & 1u) && is_dead(jv)))
                     jacc += trunc_s64_large(jv) - (long long)__float2int_rz(jv);
-                }
                 if ((wrap >> k) & 1u) {
                     int j2; float f2;
                     cell_of_inside(xs[k], inv_dx, jmax, j2, f2);
@@ -701,7 +731,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         // its own passes, then those of its pooled records.
         const unsigned own = nrec & ~31u;
         unsigned nb1 = 0, nb2 = 0;   // warp-uniform: births of its own passes
-        if (lane == 0) { sh.first[warp] = rec0 + own; sh.start[warp + 1] = nrec - own; }
+        if (lane == 0) sh.start[warp + 1] = nrec - own;
         __syncthreads();
         if (warp == 0) {
             unsigned v = lane < WARPS ? sh.start[lane + 1] : 0u;
@@ -720,23 +750,23 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = b1;
         unsigned u = (unsigned)warp;              // the warp whose record this is
         for (unsigned c = 0;; c += 32u) {
-            const bool pool = c >= own;
+            const bool last = c >= own;           // the pool
             bool has = true;
-            unsigned rec = rec0 + c + lane;
-            if (pool) {
+            if (last) {
                 has = (unsigned)tid < pooled;
                 for (u = 0; u < WARPS - 1 && (unsigned)tid >= sh.start[u + 1]; ++u) {}
-                rec = sh.first[u] + ((unsigned)tid - sh.start[u]);
             }
             bkind = 0;
             if (has) {
-                const uint4 a = CAND[2 * (size_t)rec], b = CAND[2 * (size_t)rec + 1];
+                const unsigned i = (unsigned)tid - sh.start[u];   // (pool)
+                const uint4 a = last ? pool.a[u][i] : CAND[2 * (size_t)(rec0 + c + lane)];
+                const uint4 b = last ? pool.b[u][i] : CAND[2 * (size_t)(rec0 + c + lane) + 1];
                 const unsigned slot = a.x;
-                const float x = __uint_as_float(a.z);
-                float vx = __uint_as_float(a.w), vy = __uint_as_float(b.x), vz = __uint_as_float(b.y);
+                const float x = X[slot];                          // needed late: births, removals
+                float vx = __uint_as_float(a.z), vy = __uint_as_float(a.w), vz = __uint_as_float(b.x);
                 bool alive;
-                const int k = collide_electron(P, P.cum[S], np, step, a.y, philox_id(pre, a.y), x, vx, vy, vz, alive,
-                                               bkind, b1, b2, wtries);
+                const int k = collide_electron(P, P.cum[S], np, step, a.y, b, x, vx, vy, vz, alive, bkind, b1, b2,
+                                               wtries);
                 if (k >= 0) {
                     atomicAdd(&sh.events[k], 1u);
                     if (alive) {
@@ -752,7 +782,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
             }
             const unsigned m1 = __ballot_sync(0xffffffffu, bkind == 1), m2 = __ballot_sync(0xffffffffu, bkind == 2);
             unsigned rank1 = nb1 + __popc(m1 & lt_mask), rank2 = nb2 + __popc(m2 & lt_mask), s0 = r0;
-            if (pool) {
+            if (last) {
                 if (lane == 0) { sh.nb1[warp] = nb1; sh.nb2[warp] = nb2; sh.m1[warp] = m1; sh.m2[warp] = m2; }
                 __syncthreads();
                 if (bkind) {
@@ -772,7 +802,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
                 P.stage[B_OM_FROM_E][s0 + rank2] = b1;
                 deposit_add_global(P.Qb[SP_OM], b1.x, inv_dx, Nc);
             }
-            if (pool) break;
+            if (last) break;
             nb1 += __popc(m1);
             nb2 += __popc(m2);
         }
@@ -787,7 +817,6 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) jacc += __shfl_down_sync(0xffffffffu, jacc, o);
     if (lane == 0 && jacc) atomicAdd(&sh.jsum, (unsigned long long)jacc);
-    if (psteps) atomicAdd(&sh.psteps, psteps);
     if (nabs0) atomicAdd(&sh.absorbed[0], nabs0);
     if (nabs1) atomicAdd(&sh.absorbed[1], nabs1);
     if (nabs0 + nabs1 + nnf + nrm) atomicAdd(&sh.removed, nabs0 + nabs1 + nnf + nrm);
@@ -798,12 +827,19 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     __syncthreads();
     if (electrons && tid < np && sh.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)sh.events[tid]);
     // one 64-bit add per node: what its two cells give it
+    unsigned kept = 0;
     for (int j = tid; j < Ng; j += BLOCK) {
         unsigned long long v = 0ull;
-        if (j < Nc) v = ((unsigned long long)cnt[j] << 16) - rsum[j];
+        if (j < Nc) { v = ((unsigned long long)cnt[j] << 16) - rsum[j]; kept += cnt[j]; }
         if (j > 0) v += rsum[j - 1];
         if (v) atomicAdd(&Qcopy[j], v);
     }
+    // pushed: those still in the deposit and those removed since
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) kept += __shfl_down_sync(0xffffffffu, kept, o);
+    if (lane == 0 && kept) atomicAdd(&sh.psteps, kept);
+    __syncthreads();
+    if (tid == 0) sh.psteps += sh.removed;
     if (tid == 0) {
         if (sh.absorbed[0]) atomicAdd(&C->cnt.absorbed[S][0], (unsigned long long)sh.absorbed[0]);
         if (sh.absorbed[1]) atomicAdd(&C->cnt.absorbed[S][1], (unsigned long long)sh.absorbed[1]);
@@ -980,7 +1016,6 @@ constexpr int push_min_blocks() { return S == SP_E ? O2PIC_PUSH_E_MIN_BLOCKS : O
 
 template <int S>
 __global__ void __launch_bounds__(BLOCK, push_min_blocks<S>()) k_push(Params P) {
-    pdl_wait();
     push_body<S>(P, blockIdx.x, gridDim.x);
 }
 
@@ -1007,7 +1042,6 @@ template <int S>
 __global__ void __launch_bounds__(BLOCK, push_min_blocks<S>()) k_push_b(const Params* __restrict__ all,
                                                                         const uint4* __restrict__ map) {
     __shared__ Params sP;
-    pdl_wait();
     const uint4 m = map[blockIdx.x];
     load_params(sP, all + m.x);
     push_body<S>(sP, m.y, m.z);
@@ -1072,7 +1106,7 @@ __global__ void __launch_bounds__(BLOCK) k_deposit(Params P) {
 
 size_t push_smem_bytes(int species, const Params& P) {
     const size_t base = align16(sizeof(PushShared)) + (sizeof(float) + 2 * sizeof(unsigned)) * P.Ng + sizeof(PushQueue);
-    return base + (species == SP_E ? sizeof(float) * NGRID : 0);
+    return base + (species == SP_E ? sizeof(float) * NGRID + sizeof(PushPool) : 0);
 }
 
 void launch_flight_init(int species, const Params& P, cudaStream_t s) {

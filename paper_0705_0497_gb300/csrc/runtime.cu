@@ -24,16 +24,11 @@ namespace o2 {
 thread_local bool pdl_enabled = true;
 
 // Ion chains on their own streams on ion steps (1), or all on the step's
-// stream (0); programmatic dependent launches inside the graph of a batch of
-// one discharge (1), or only outside graphs (0).  Both keep the results.  On
-// the 512-cell, 1.6e7-particle discharge at its periodic state the fork took
-// the RF cycle from 46.2 to 44.3 ms; the programmatic launches inside the
-// one-discharge graph gained nothing (46.7 ms without the fork, 44.1 with).
+// stream (0).  Both keep the results.  On the 512-cell, 1.6e7-particle
+// discharge at its periodic state the fork took the RF cycle from 46.2 to 44.3
+// ms.
 #ifndef O2PIC_ION_FORK
 #define O2PIC_ION_FORK 1
-#endif
-#ifndef O2PIC_GRAPH_PDL_SINGLE
-#define O2PIC_GRAPH_PDL_SINGLE 0
 #endif
 constexpr bool ION_FORK = O2PIC_ION_FORK != 0;
 }
@@ -1370,8 +1365,10 @@ int batch_capture(o2pic_batch* b) {
         enqueue_fused(b, b->stream);
     } else {
         // several branches: no early-launched blocks that could crowd out
-        // the single-block kernels of other branches
-        pdl_enabled = O2PIC_GRAPH_PDL_SINGLE && n == 1;
+        // the small kernels of other branches (one discharge: the set-up of a
+        // kernel overlaps the end of the one before, 38.2 -> 37.0 ms per RF
+        // cycle of 512 cells)
+        pdl_enabled = n == 1;
         cudaEventRecord(b->fork, b->stream);
         for (size_t i = 0; i < n; ++i) {
             cudaStreamWaitEvent(b->branch[i], b->fork, 0);
