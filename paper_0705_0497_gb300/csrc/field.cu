@@ -431,6 +431,7 @@ __device__ __forceinline__ void step_commit(const Params& P, int mode, int pushe
             C->rremovals = 0u;
             C->dremovals = 0u;
             C->births22 = 0u;
+            C->pcand[0] = C->pcand[1] = C->pcand[2] = 0u;
             C->acc_steps = cs.acc_steps + 1;
             C->step = cs.step + 1;
             C->epoch = cs.epoch + 1;

@@ -111,6 +111,8 @@ struct DevCtrl {
     unsigned int rremovals;                // (16) pairs to remove
     unsigned int dremovals;                // (22) pairs listed
     unsigned int births22;                 // (22) electron births staged this step
+    unsigned int pcand[3];                 // pair candidates of this step: (22), (16), (17)
+    unsigned int pad;
     DevCounters cnt;
 };
 
@@ -195,6 +197,7 @@ struct Params {
     float Kmax_r_hi, kappa_r;
     int have_recomb;
     unsigned int* rhist[2];      // 0: e, 1: O2+
+    uint2* rcand;                // candidates of (16), [capacity of e]
     unsigned int* rtot;          // [2][Nc] (cleared by the end-of-step kernel)
     unsigned int* rremoval;      // [2 * max_rremovals]: e slot, O2+ slot
     unsigned int max_rremovals;
@@ -233,6 +236,8 @@ struct PairSpec {
     const float* K;              // [NGRID] sigma g
     float Kmax_hi, kappa;
     uint32_t tag_pair, tag_shift;
+    uint2* cand;                 // candidates (A slot, word of the acceptance draw), and their number
+    unsigned int* ncand;
     unsigned int* removal;
     unsigned int* nremovals;     // device counter of listed pairs
     unsigned int max_removals;
@@ -260,8 +265,10 @@ void launch_push(int species, const Params& P, int grid, cudaStream_t s);
 void launch_cand(int species, const Params& P, int grid, cudaStream_t s);   // ion species
 void launch_filter(int species, const Params& P, int grid, cudaStream_t s);
 void launch_filter_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
-void launch_pair_hist(const Params& P, const PairSpec& S, int grid, cudaStream_t s);
-cudaError_t configure_pair_hist_smem(int Nc);
+// na blocks for species A (counts and draws), nb for B (counts); either may be 0
+void launch_pair_count(const Params& P, const PairSpec& S, int na, int nb, cudaStream_t s);
+cudaError_t configure_pair_count_smem(int Nc);
+size_t pair_count_smem_bytes(int Nc);
 void launch_pair(const Params& P, const PairSpec& S, int grid, cudaStream_t s);
 void launch_pair_apply(const Params& P, const PairSpec& S, cudaStream_t s);
 void launch_edet_apply(const Params& P, const PairSpec& S, cudaStream_t s);
@@ -273,8 +280,8 @@ void launch_push_batched(int species, const Params* all, const uint4* map, int n
 void launch_cand_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_field_batched(const Params* all, int n, size_t smem, int mode, int pushed_mask, cudaStream_t s);
 void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cudaStream_t s);
-void launch_pair_hist_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,
-                              cudaStream_t s);
+void launch_pair_count_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,
+                               cudaStream_t s);
 void launch_pair_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, cudaStream_t s);
 void launch_pair_apply_batched(const Params* all, const PairSpec* specs, int n, cudaStream_t s);
 void launch_field(const Params& P, int mode, int pushed_mask, cudaStream_t s);

@@ -11,16 +11,21 @@
 // P <= K_max M pf (pf = w dt_ion / (A dx)), so an O- can react only if
 // u < K_max M pf; at the method's weights and time steps that bound is
 // ~1e-6 and only a handful of O- per step pass it.  So:
-//   * k_pair_hist counts, per 8192-slot tile of each ion species, the live
-//     ions per cell, and adds them into per-cell totals n-, n+;
-//   * k_pair streams x and id of the O- once, draws u and flags the O- below
-//     the bound (M from the totals);
-//   * for a flagged O- the whole block finds its rank k in the cell list
-//     (counts of the earlier tiles + same-cell slots before it in its tile),
-//     the partner rank q, the O2+ tile holding rank q (block scan of that
-//     cell's per-tile counts) and the partner's slot there (block scan of the
-//     hits in slot order), each step with all of the block's loads in flight;
-//     one thread then does the reaction test with the exact P.
+//   * k_pair_count, O- part: streams x and id of the O- once; per tile of 8192
+//     slots the live O- per cell (and their totals n-), and u against the
+//     bound with M replaced by the number of slots in use: the ~1e-3 that pass
+//     go to a candidate list.  O2+ part: the same counts of the O2+.  Neither
+//     part needs the other, so each runs behind its own species' chain and the
+//     draws (ALU) beside the O2+ push (HBM), off the step's critical path;
+//   * k_pair, once both are there: the candidates against the bound with the
+//     cell's M, one per thread; for each one left the whole block finds its
+//     rank k in the cell list (counts of the earlier tiles + same-cell slots
+//     before it in its tile), the partner rank q, the O2+ tile holding rank q
+//     (block scan of that cell's per-tile counts) and the partner's slot there
+//     (block scan of the hits in slot order), each step with all of the
+//     block's loads in flight; one thread then does the reaction test with the
+//     exact P.
+// Both streams are bound by HBM on large arrays and by latency on small ones.
 // Reactions only append (O- slot, O2+ slot) to the removal list and take the
 // pair out of the fresh deposit; both are order-independent, so flagged ions
 // may be resolved in any order.
@@ -36,62 +41,110 @@ namespace o2 {
 
 namespace {
 
-constexpr int HIST_T = 512;                  // threads of k_pair_hist
-constexpr int HIST_PER = TILE / HIST_T;      // 16 slots per thread
+constexpr int HIST_T = 512;                  // threads of k_pair_count
+constexpr int HIST_V = TILE / HIST_T / 4;    // 16-byte loads of an array per thread and tile
 constexpr int PAIR_T = 256;                  // threads of k_pair
 constexpr int PER_T = TILE / PAIR_T;         // 32 slots of a tile per thread
-constexpr int LCAP = 256;                    // flagged O- listed per tile before the slow path
-constexpr unsigned short CELL_DEAD = 0x7FFFu, CELL_FLAG = 0x8000u;
 static_assert(PER_T == 32, "one 32-bit hit mask per thread");
-static_assert(MAX_NODES - 1 < CELL_DEAD, "cell index fits 15 bits");
 
-// Per tile of each ion species, the live ions per cell (post-push
-// positions): hist[sp][tile][cell]; and the per-cell totals ptot[sp][cell]
-// (zero on entry; the end-of-step kernel clears them).  Blocks take tiles of
-// O- first, then of O2+, and add their totals once at the end.
-__device__ __forceinline__ void pair_hist_body(const Params& P, const PairSpec& Sp, unsigned blk, unsigned nblk) {
-    extern __shared__ unsigned hsm[];   // [Nc] tile counts, [2][Nc] block totals
+// Four slots from p on of an array of n (p a multiple of 4); `fill` beyond n.
+template <class V, class T>
+__device__ __forceinline__ V load4(const T* __restrict__ A, unsigned long long p, unsigned long long n, T fill) {
+    V v;
+    if (p + 4 <= n) {
+        v = *reinterpret_cast<const V*>(A + p);
+    } else {
+        v.x = p < n ? A[p] : fill;
+        v.y = p + 1 < n ? A[p + 1] : fill;
+        v.z = p + 2 < n ? A[p + 2] : fill;
+        v.w = fill;
+    }
+    return v;
+}
+
+// Live particles per cell (post-push positions) of each tile of one of the two
+// species (`first`: A): hist[tile][cell], and the totals per cell (zero on
+// entry; the end-of-step kernel clears them), added once per block at the end.
+// A also draws: the particles whose acceptance number is below the bound for
+// as many partners as there are slots go to the candidate list.
+template <bool FIRST>
+__device__ __forceinline__ void pair_count_body(const Params& P, const PairSpec& Sp, unsigned blk, unsigned nblk) {
+    extern __shared__ unsigned hsm[];   // [Nc] tile counts, [Nc] block totals
     DevCtrl* C = P.ctrl;
     const int Nc = P.Nc;
+    const float inv_dx = P.inv_dx, limit = cell_limit(P.Nc);
     unsigned* bt = hsm + Nc;
-    for (int c = threadIdx.x; c < 2 * Nc; c += HIST_T) bt[c] = 0u;
-    const unsigned long long nsa = C->slots[Sp.A], nsb = C->slots[Sp.B];
-    const unsigned nta = (unsigned)ceil_div(nsa, TILE), ntb = (unsigned)ceil_div(nsb, TILE);
-    for (unsigned g = blk; g < nta + ntb; g += nblk) {
-        const int sp = (g < nta) ? 0 : 1;
-        const unsigned tile = (g < nta) ? g : g - nta;
-        const int S = sp == 0 ? Sp.A : Sp.B;
-        const unsigned long long n = sp == 0 ? nsa : nsb;
-        const float* __restrict__ X = P.sp[S].x[C->cur[S]];
-        for (int c = threadIdx.x; c < Nc; c += HIST_T) hsm[c] = 0u;
-        const unsigned long long base = (unsigned long long)tile * TILE;
-        float xs[HIST_PER];
+    for (int c = threadIdx.x; c < Nc; c += HIST_T) { hsm[c] = 0u; bt[c] = 0u; }
+    pdl_wait();
+    const int S = FIRST ? Sp.A : Sp.B;
+    const unsigned long long n = C->slots[S];
+    const unsigned ntiles = (unsigned)ceil_div(n, TILE);
+    if (blk >= ntiles) return;          // block-uniform
+    const unsigned cb = C->cur[S];
+    const float* __restrict__ X = P.sp[S].x[cb];
+    const uint32_t* __restrict__ ID = P.sp[S].id[cb];
+    const unsigned long long step = C->step;
+    const PhiloxPre pre = philox_pre((uint32_t)step, Sp.tag_pair, (uint32_t)(step >> 32), P.seed);
+    // P <= K_max M pf with M at most the slots in use of either species
+    const unsigned long long mb = C->slots[Sp.A] > C->slots[Sp.B] ? C->slots[Sp.A] : C->slots[Sp.B];
+    const float bound = Sp.Kmax_hi * (P.pair_factor * (float)mb);
+    __syncthreads();
+    for (unsigned tile = blk; tile < ntiles; tile += nblk) {
+        const unsigned long long base = (unsigned long long)tile * TILE + 4u * threadIdx.x;
+        float4 x[HIST_V];
+        uint4 id[FIRST ? HIST_V : 1];
 #pragma unroll
-        for (int i = 0; i < HIST_PER; ++i) {
-            const unsigned long long p = base + (unsigned long long)i * HIST_T + threadIdx.x;
-            xs[i] = (p < n) ? X[p] : dead_marker();
+        for (int i = 0; i < HIST_V; ++i) x[i] = load4<float4>(X, base + 4ull * HIST_T * i, n, dead_marker());
+        if (FIRST) {
+#pragma unroll
+            for (int i = 0; i < HIST_V; ++i) id[i] = load4<uint4>(ID, base + 4ull * HIST_T * i, n, 0u);
         }
-        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < HIST_PER; ++i) {
-            if (!is_dead(xs[i])) {
+        for (int i = 0; i < HIST_V; ++i) {
+            const float xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (is_dead(xs[k])) continue;
                 int c; float fr;
-                cell_of(xs[i], P.inv_dx, Nc, c, fr);
+                cell_of_inside(xs[k], inv_dx, limit, c, fr);
                 atomicAdd(&hsm[c], 1u);
             }
         }
+        if (FIRST) {
+#pragma unroll
+            for (int i = 0; i < HIST_V; ++i) {
+                const float xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+                const uint32_t ids[4] = {id[i].x, id[i].y, id[i].z, id[i].w};
+                uint32_t w[4];
+                bool any = false;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    w[k] = philox_id(pre, ids[k]).x;
+                    any |= uniform(w[k]) < bound;
+                }
+                if (any) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (uniform(w[k]) < bound && !is_dead(xs[k])) {
+                            const unsigned q = atomicAdd(Sp.ncand, 1u);   // at most the slots of A
+                            Sp.cand[q] = make_uint2((unsigned)(base + 4ull * HIST_T * i) + k, w[k]);
+                        }
+                }
+            }
+        }
         __syncthreads();
-        unsigned* H = (sp == 0 ? Sp.histA : Sp.histB) + (size_t)tile * Nc;
+        unsigned* H = (FIRST ? Sp.histA : Sp.histB) + (size_t)tile * Nc;
         for (int c = threadIdx.x; c < Nc; c += HIST_T) {
             const unsigned v = hsm[c];
             H[c] = v;
-            bt[sp * Nc + c] += v;
+            bt[c] += v;
+            hsm[c] = 0u;
         }
         __syncthreads();
     }
     pdl_trigger();
-    for (int c = threadIdx.x; c < 2 * Nc; c += HIST_T)
-        if (bt[c]) atomicAdd(&Sp.tot[c], bt[c]);
+    for (int c = threadIdx.x; c < Nc; c += HIST_T)
+        if (bt[c]) atomicAdd(&Sp.tot[FIRST ? c : Nc + c], bt[c]);
 }
 
 __device__ __forceinline__ unsigned block_sum(unsigned v, unsigned* ws) {
@@ -100,24 +153,34 @@ __device__ __forceinline__ unsigned block_sum(unsigned v, unsigned* ws) {
     return total;
 }
 
-// Resolve one flagged O- (tile position pos, cell in cell16[pos]).  Every
+// Resolve one flagged O- (slot p, acceptance number u, in cell c).  Every
 // thread of the block calls it; all return at the same point except at the
 // very end.  sh = 2 words of shared memory for the partner tile search.
-__device__ void resolve_one(const Params& P, const PairSpec& Sp, unsigned pos, unsigned tile, unsigned long long base,
-                            const unsigned short* cell16, unsigned* ws, unsigned* sh, unsigned long long step,
-                            unsigned long long nsp, unsigned ntp, unsigned cm, unsigned cp, unsigned& gt1) {
+__device__ void resolve_one(const Params& P, const PairSpec& Sp, unsigned p, float u, unsigned c, unsigned* ws,
+                            unsigned* sh, unsigned long long step, unsigned long long nsp, unsigned ntp, unsigned cm,
+                            unsigned cp, unsigned& gt1) {
     DevCtrl* C = P.ctrl;
     const int Nc = P.Nc;
     const int tid = threadIdx.x;
-    const unsigned c = cell16[pos] & CELL_DEAD;
     // rank k of the O- in its cell list
+    const unsigned tile = p / TILE;
     unsigned cnt = 0;
     const unsigned* H0 = Sp.histA;
     for (unsigned t = tid; t < tile; t += PAIR_T) cnt += H0[(size_t)t * Nc + c];
-#pragma unroll 8
+    const float* XM = P.sp[Sp.A].x[cm];
+    float xa[PER_T];
+#pragma unroll
     for (int i = 0; i < PER_T; ++i) {
-        const unsigned q = (unsigned)i * PAIR_T + tid;
-        if (q < pos && (cell16[q] & CELL_DEAD) == c) ++cnt;
+        const unsigned q = tile * TILE + (unsigned)i * PAIR_T + tid;
+        xa[i] = q < p ? XM[q] : dead_marker();
+    }
+#pragma unroll
+    for (int i = 0; i < PER_T; ++i) {
+        if (!is_dead(xa[i])) {
+            int j; float fr;
+            cell_of(xa[i], P.inv_dx, Nc, j, fr);
+            cnt += (unsigned)j == c ? 1u : 0u;
+        }
     }
     const unsigned k = block_sum(cnt, ws);
     const unsigned nm = Sp.tot[c], npl = Sp.tot[Nc + c];
@@ -179,12 +242,8 @@ __device__ void resolve_one(const Params& P, const PairSpec& Sp, unsigned pos, u
     for (unsigned t = 0; t < want - excl; ++t) bits &= bits - 1u;
     const unsigned b_slot = (unsigned)(bb + (unsigned)(__ffs(bits) - 1));
     // reaction test with the exact probability
-    const unsigned long long p = base + pos;
     const SpeciesBuf& SM = P.sp[Sp.A];
     const SpeciesBuf& SPp = P.sp[Sp.B];
-    const uint4 w = philox4x32_10(make_uint4((uint32_t)step, Sp.tag_pair, 0u, (uint32_t)(step >> 32)),
-                                  make_uint2(SM.id[cm][p], P.seed));
-    const float u = uniform(w.x);
     const float gx = SM.vx[cm][p] - SPp.vx[cp][b_slot];
     const float gy = SM.vy[cm][p] - SPp.vy[cp][b_slot];
     const float gz = SM.vz[cm][p] - SPp.vz[cp][b_slot];
@@ -198,7 +257,7 @@ __device__ void resolve_one(const Params& P, const PairSpec& Sp, unsigned pos, u
     if (u < Pp && E >= Sp.thr) {
         const unsigned idx = atomicAdd(Sp.nremovals, 1u);
         if (idx < Sp.max_removals) {
-            Sp.removal[2 * idx] = (unsigned)p;
+            Sp.removal[2 * idx] = p;
             Sp.removal[2 * idx + 1] = b_slot;
         }
         // take both out of the fresh deposit
@@ -216,11 +275,12 @@ __device__ void resolve_one(const Params& P, const PairSpec& Sp, unsigned pos, u
     }
 }
 
-// One block per O- tile (grid-stride): the streaming pass, then the flagged
-// O- of the tile.  Block 0 also adds sum_c min(n-, n+) to the pair counter.
+// The candidates, one per thread, against the bound with their cell's M; those
+// left are resolved one after another by the block.  Block 0 also adds
+// sum_c min(n-, n+) to the pair counter.
 __device__ __forceinline__ void pair_body(const Params& P, const PairSpec& Sp, unsigned blk, unsigned nblk) {
-    __shared__ unsigned short cell16[TILE];
-    __shared__ unsigned short list[LCAP];
+    __shared__ unsigned list[PAIR_T], cell[PAIR_T];
+    __shared__ float draw[PAIR_T];
     __shared__ unsigned ws[32];
     __shared__ unsigned sh[2];
     __shared__ unsigned nflag;
@@ -229,14 +289,11 @@ __device__ __forceinline__ void pair_body(const Params& P, const PairSpec& Sp, u
     const int tid = threadIdx.x;
     const unsigned long long step = C->step;
     const unsigned long long nsm = C->slots[Sp.A], nsp = C->slots[Sp.B];
-    const unsigned ntm = (unsigned)ceil_div(nsm, TILE), ntp = (unsigned)ceil_div(nsp, TILE);
+    const unsigned ntp = (unsigned)ceil_div(nsp, TILE);
     const unsigned cm = C->cur[Sp.A], cp = C->cur[Sp.B];
     const float* __restrict__ XM = P.sp[Sp.A].x[cm];
-    const uint32_t* __restrict__ IDM = P.sp[Sp.A].id[cm];
     const unsigned* __restrict__ tot = Sp.tot;
-    // the acceptance draw's Philox block (counter (step, tag, 0), key (id,
-    // seed)) with its id-free first-round products computed once
-    const PhiloxPre pre = philox_pre((uint32_t)step, Sp.tag_pair, (uint32_t)(step >> 32), P.seed);
+    const unsigned n = *Sp.ncand < nsm ? *Sp.ncand : (unsigned)nsm;
     unsigned gt1 = 0;
 
     if (blk == 0) {
@@ -248,61 +305,28 @@ __device__ __forceinline__ void pair_body(const Params& P, const PairSpec& Sp, u
         const unsigned s = block_sum(pairs, ws);
         if (tid == 0 && s) atomicAdd(Sp.tested, (unsigned long long)s);
     }
-
-    for (unsigned tile = blk; tile < ntm; tile += nblk) {
-        const unsigned long long base = (unsigned long long)tile * TILE;
+    for (unsigned e0 = 0; e0 < n; e0 += nblk * PAIR_T) {
         if (tid == 0) nflag = 0u;
         __syncthreads();
-#pragma unroll
-        for (int h = 0; h < PER_T; h += 16) {
-            float xs[16];
-            uint32_t ids[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const unsigned long long p = base + (unsigned long long)(h + i) * PAIR_T + tid;
-                const bool in = p < nsm;
-                xs[i] = in ? XM[p] : dead_marker();
-                ids[i] = in ? IDM[p] : 0u;
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const unsigned pos = (unsigned)(h + i) * PAIR_T + tid;
-                unsigned short cc = CELL_DEAD;
-                if (!is_dead(xs[i])) {
-                    int c; float fr;
-                    cell_of(xs[i], P.inv_dx, Nc, c, fr);
-                    const unsigned a = __ldg(&tot[c]), b = __ldg(&tot[Nc + c]);
-                    const unsigned M = a < b ? b : a;
-                    const float u = uniform(philox_id(pre, ids[i]).x);
-                    cc = (unsigned short)c;
-                    if (u < Sp.Kmax_hi * (P.pair_factor * (float)M)) {
-                        cc |= CELL_FLAG;
-                        const unsigned idx = atomicAdd(&nflag, 1u);
-                        if (idx < LCAP) list[idx] = (unsigned short)pos;
-                    }
-                }
-                cell16[pos] = cc;
+        const unsigned e = e0 + (unsigned)tid * nblk + blk;
+        if (e < n) {
+            const uint2 r = Sp.cand[e];
+            int c; float fr;
+            cell_of(XM[r.x], P.inv_dx, Nc, c, fr);
+            const unsigned a = tot[c], b = tot[Nc + c];
+            const unsigned M = a < b ? b : a;
+            const float u = uniform(r.y);
+            if (u < Sp.Kmax_hi * (P.pair_factor * (float)M)) {
+                const unsigned i = atomicAdd(&nflag, 1u);
+                list[i] = r.x;
+                cell[i] = (unsigned)c;
+                draw[i] = u;
             }
         }
         __syncthreads();
         const unsigned nf = nflag;
-        if (nf > 0 && nf <= LCAP) {
-            for (unsigned j = 0; j < nf; ++j)
-                resolve_one(P, Sp, list[j], tile, base, cell16, ws, sh, step, nsp, ntp, cm, cp, gt1);
-        } else if (nf > LCAP) {
-            // many flagged ions: list them segment by segment from the flags
-            for (int seg = 0; seg < PER_T; ++seg) {
-                const unsigned pos = (unsigned)seg * PAIR_T + tid;
-                const bool f = (cell16[pos] & CELL_FLAG) != 0;
-                unsigned ns;
-                const unsigned idx = block_excl_scan<PAIR_T>(f ? 1u : 0u, ws, &ns);
-                if (f) list[idx] = (unsigned short)pos;
-                __syncthreads();
-                for (unsigned j = 0; j < ns; ++j)
-                    resolve_one(P, Sp, list[j], tile, base, cell16, ws, sh, step, nsp, ntp, cm, cp, gt1);
-                __syncthreads();
-            }
-        }
+        for (unsigned j = 0; j < nf; ++j)
+            resolve_one(P, Sp, list[j], draw[j], cell[j], ws, sh, step, nsp, ntp, cm, cp, gt1);
         __syncthreads();
     }
     pdl_trigger();
@@ -393,9 +417,10 @@ __device__ __forceinline__ void edet_apply_body(const Params& P, const PairSpec&
     }
 }
 
-__global__ void __launch_bounds__(HIST_T) k_pair_hist(Params P, PairSpec Sp) {
-    pdl_wait();
-    pair_hist_body(P, Sp, blockIdx.x, gridDim.x);
+// Blocks [0, na) count A, the others B.
+__global__ void __launch_bounds__(HIST_T, 2) k_pair_count(Params P, PairSpec Sp, unsigned na) {
+    if (blockIdx.x < na) pair_count_body<true>(P, Sp, blockIdx.x, na);
+    else pair_count_body<false>(P, Sp, blockIdx.x - na, gridDim.x - na);
 }
 
 __global__ void __launch_bounds__(PAIR_T) k_pair(Params P, PairSpec Sp) {
@@ -410,16 +435,17 @@ __global__ void k_pair_apply(Params P, PairSpec Sp) {
 }
 
 // batched: block b works for discharge map[b].x (block map[b].y of map[b].z)
-__global__ void __launch_bounds__(HIST_T) k_pair_hist_b(const Params* __restrict__ all,
-                                                         const PairSpec* __restrict__ specs,
-                                                         const uint4* __restrict__ map) {
+// batched: map[b].w = 0 counts A, 1 B
+__global__ void __launch_bounds__(HIST_T, 2) k_pair_count_b(const Params* __restrict__ all,
+                                                            const PairSpec* __restrict__ specs,
+                                                            const uint4* __restrict__ map) {
     __shared__ Params sP;
-    pdl_wait();
     const uint4 m = map[blockIdx.x];
     const PairSpec Sp = specs[m.x];
     if (!Sp.active) return;   // block-uniform
     load_params(sP, all + m.x);
-    pair_hist_body(sP, Sp, m.y, m.z);
+    if (m.w == 0u) pair_count_body<true>(sP, Sp, m.y, m.z);
+    else pair_count_body<false>(sP, Sp, m.y, m.z);
 }
 
 __global__ void __launch_bounds__(PAIR_T) k_pair_b(const Params* __restrict__ all, const PairSpec* __restrict__ specs,
@@ -460,19 +486,19 @@ __global__ void k_pair_apply_b(const Params* __restrict__ all, const PairSpec* _
 
 }  // namespace
 
-size_t pair_hist_smem_bytes(int Nc) { return 3 * sizeof(unsigned) * (size_t)Nc; }
+size_t pair_count_smem_bytes(int Nc) { return 2 * sizeof(unsigned) * (size_t)Nc; }
 
-cudaError_t configure_pair_hist_smem(int Nc) {
-    cudaError_t e = cudaFuncSetAttribute(k_pair_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)pair_hist_smem_bytes(Nc));
+cudaError_t configure_pair_count_smem(int Nc) {
+    cudaError_t e = cudaFuncSetAttribute(k_pair_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)pair_count_smem_bytes(Nc));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pair_hist_b, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pair_hist_smem_bytes(Nc));
+        e = cudaFuncSetAttribute(k_pair_count_b, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)pair_count_smem_bytes(Nc));
     return e;
 }
 
-void launch_pair_hist(const Params& P, const PairSpec& S, int grid, cudaStream_t s) {
-    launch_pdl(k_pair_hist, grid, HIST_T, pair_hist_smem_bytes(P.Nc), s, P, S);
+void launch_pair_count(const Params& P, const PairSpec& S, int na, int nb, cudaStream_t s) {
+    launch_pdl(k_pair_count, na + nb, HIST_T, pair_count_smem_bytes(P.Nc), s, P, S, (unsigned)na);
 }
 
 void launch_pair(const Params& P, const PairSpec& S, int grid, cudaStream_t s) {
@@ -492,9 +518,9 @@ void launch_edet_apply_batched(const Params* all, const PairSpec* specs, int n, 
     launch_pdl(k_edet_apply_b, n, 256, 0, s, all, specs);
 }
 
-void launch_pair_hist_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,
-                              cudaStream_t s) {
-    launch_pdl(k_pair_hist_b, nblocks, HIST_T, smem, s, all, specs, map);
+void launch_pair_count_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,
+                               cudaStream_t s) {
+    launch_pdl(k_pair_count_b, nblocks, HIST_T, smem, s, all, specs, map);
 }
 
 void launch_pair_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, cudaStream_t s) {

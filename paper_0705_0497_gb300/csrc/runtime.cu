@@ -108,7 +108,8 @@ struct o2pic_ctx {
     bool coul_alloc = false;                       // Coulomb cell-sort buffers allocated
     int latched = 0;
     int grid_push[NSP] = {0, 0, 0};
-    int grid_pair = 0, grid_pair_e = 0, grid_compact = 0, grid_deposit = 0;
+    int grid_count[NSP] = {0, 0, 0};   // blocks of the pair counts: two per SM, or one per tile
+    int grid_compact = 0, grid_deposit = 0;
     unsigned long long launches = 0;
     unsigned long long gen = 0;        // bumped by every call that invalidates a captured graph
     unsigned long long ring_start = 0; // first step recorded in the current-sum ring
@@ -309,24 +310,25 @@ int prepare(o2pic_ctx* c, cudaStream_t s) {
     return cuda_fail(c, cudaGetLastError());
 }
 
-// The cell-binned binary processes of a context: (22) e + O- -> O + 2e
+// The cell-binned binary processes of a context (the O- candidate records of
+// the step are done with when (22) and (17) list theirs in their place): (22) e + O- -> O + 2e
 // (A = O-, only A removed), (16) e + O2+ -> O + O, (17) O- + O2+ -> O + O2.
 PairSpec spec_edet(o2pic_ctx* c) {
     const Params& P = c->P;
     return PairSpec{SP_OM, SP_E, P.dhist[0], P.dhist[1], P.dtot, P.Ktab_d, P.Kmax_d_hi, P.kappa_d, TAG_EDET,
-                    TAG_SHIFT_EDET, P.dremoval, &c->d_ctrl->dremovals, P.max_dremovals,
+                    TAG_SHIFT_EDET, (uint2*)P.cand[SP_OM], &c->d_ctrl->pcand[0], P.dremoval, &c->d_ctrl->dremovals, P.max_dremovals,
                     &c->d_ctrl->cnt.edet_candidates, &c->d_ctrl->cnt.edetached, P.have_edet, P.thr_d, 1};
 }
 PairSpec spec_rec(o2pic_ctx* c) {
     const Params& P = c->P;
     return PairSpec{SP_E, SP_OP, P.rhist[0], P.rhist[1], P.rtot, P.Ktab_r, P.Kmax_r_hi, P.kappa_r, TAG_REC,
-                    TAG_SHIFT_REC, P.rremoval, &c->d_ctrl->rremovals, P.max_rremovals,
+                    TAG_SHIFT_REC, P.rcand, &c->d_ctrl->pcand[1], P.rremoval, &c->d_ctrl->rremovals, P.max_rremovals,
                     &c->d_ctrl->cnt.rec_candidates, &c->d_ctrl->cnt.recombined, P.have_recomb, 0.0f, 0};
 }
 PairSpec spec_neu(o2pic_ctx* c) {
     const Params& P = c->P;
     return PairSpec{SP_OM, SP_OP, P.hist[0], P.hist[1], P.ptot, P.Ktab, P.Kmax_hi, P.kappa_n, TAG_PAIR,
-                    TAG_SHIFT, P.removal, &c->d_ctrl->removals, P.max_removals,
+                    TAG_SHIFT, (uint2*)P.cand[SP_OM], &c->d_ctrl->pcand[2], P.removal, &c->d_ctrl->removals, P.max_removals,
                     &c->d_ctrl->cnt.pair_candidates, &c->d_ctrl->cnt.neutralized, P.have_neutral, 0.0f, 0};
 }
 
@@ -361,6 +363,14 @@ void enqueue_steps(o2pic_ctx* c, uint64_t nsteps, cudaStream_t s) {
                 launch(c, KK_FILT_OP, sp2, [&] { launch_filter(SP_OP, P, c->grid_push[SP_OP], sp2); });
                 launch(c, KK_CAND_OP, sp2, [&] { launch_cand(SP_OP, P, c->grid_push[SP_OP], sp2); });
             }
+            // (17): each species is counted behind its own chain, where no other
+            // pair process removes particles in between
+            const bool early = fork && P.have_neutral && !P.have_edet && !P.have_recomb;
+            if (early) {
+                const PairSpec N = spec_neu(c);
+                launch(c, KK_PAIR_HIST, so, [&] { launch_pair_count(P, N, c->grid_count[SP_OM], 0, so); });
+                launch(c, KK_PAIR_HIST, sp2, [&] { launch_pair_count(P, N, 0, c->grid_count[SP_OP], sp2); });
+            }
             if (fork) {
                 cudaEventRecord(c->ev_join[0], so);
                 cudaEventRecord(c->ev_join[1], sp2);
@@ -374,20 +384,22 @@ void enqueue_steps(o2pic_ctx* c, uint64_t nsteps, cudaStream_t s) {
             }
             if (P.have_edet) {
                 const PairSpec D = spec_edet(c);
-                launch(c, KK_REC, s, [&] { launch_pair_hist(P, D, c->grid_compact, s); });
-                launch(c, KK_REC, s, [&] { launch_pair(P, D, c->grid_pair, s); });
+                launch(c, KK_REC, s, [&] { launch_pair_count(P, D, c->grid_count[SP_OM], c->grid_count[SP_E], s); });
+                launch(c, KK_REC, s, [&] { launch_pair(P, D, c->num_sms, s); });
                 launch(c, KK_REC, s, [&] { launch_edet_apply(P, D, s); });
             }
             if (P.have_recomb) {
                 const PairSpec R = spec_rec(c);
-                launch(c, KK_REC, s, [&] { launch_pair_hist(P, R, c->grid_compact, s); });
-                launch(c, KK_REC, s, [&] { launch_pair(P, R, c->grid_pair_e, s); });
+                launch(c, KK_REC, s, [&] { launch_pair_count(P, R, c->grid_count[SP_E], c->grid_count[SP_OP], s); });
+                launch(c, KK_REC, s, [&] { launch_pair(P, R, c->num_sms, s); });
                 launch(c, KK_REC, s, [&] { launch_pair_apply(P, R, s); });
             }
             if (P.have_neutral) {
                 const PairSpec N = spec_neu(c);
-                launch(c, KK_PAIR_HIST, s, [&] { launch_pair_hist(P, N, c->grid_compact, s); });
-                launch(c, KK_PAIR, s, [&] { launch_pair(P, N, c->grid_pair, s); });
+                if (!early)
+                    launch(c, KK_PAIR_HIST, s,
+                           [&] { launch_pair_count(P, N, c->grid_count[SP_OM], c->grid_count[SP_OP], s); });
+                launch(c, KK_PAIR, s, [&] { launch_pair(P, N, c->num_sms, s); });
             }
         }
         launch(c, KK_FIELD, s, [&] { launch_field(P, 0, ion ? 7 : 1, s); });
@@ -537,6 +549,7 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     // (16): e and O2+ tiles, totals, pair list
     TRY(ctx_alloc(c, &P.rhist[0], (ceil_div(cfg->capacity[SP_E], TILE) + 1) * Nc));
     TRY(ctx_alloc(c, &P.rhist[1], (ceil_div(cfg->capacity[SP_OP], TILE) + 1) * Nc));
+    TRY(ctx_alloc(c, &P.rcand, (size_t)cfg->capacity[SP_E]));
     TRY(ctx_alloc(c, &P.rtot, 2 * (size_t)Nc));
     P.max_rremovals = (unsigned)std::max<unsigned long long>(1, std::min(cfg->capacity[SP_E], cfg->capacity[SP_OP]));
     TRY(ctx_alloc(c, &P.rremoval, 2 * (size_t)P.max_rremovals));
@@ -563,10 +576,10 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     smax = std::max(smax, sizeof(unsigned) * (size_t)Ng);
     TRY(configure_push_smem(smax));
     TRY(configure_field_smem(field_smem_bytes(P)));
-    TRY(configure_pair_hist_smem(Nc));
-    c->grid_pair = (int)std::max<unsigned long long>(1, std::min<unsigned long long>(tiles_ion, 8ull * c->num_sms));
-    c->grid_pair_e = (int)std::max<unsigned long long>(
-        1, std::min<unsigned long long>(ceil_div(cfg->capacity[SP_E], TILE) + 1, 8ull * c->num_sms));
+    TRY(configure_pair_count_smem(Nc));
+    for (int s = 0; s < NSP; ++s)
+        c->grid_count[s] = (int)std::max<unsigned long long>(
+            1, std::min<unsigned long long>(ceil_div(cfg->capacity[s], TILE), 2ull * c->num_sms));
     c->grid_compact = 4 * c->num_sms;
     c->grid_deposit = 4 * c->num_sms;
     // steady initial control state
@@ -1205,10 +1218,8 @@ struct o2pic_batch {
     PairSpec* dD = nullptr;               // [n] (22)
     PairSpec* dN = nullptr;               // [n] (17)
     uint4* dmap = nullptr;                // block maps, concatenated
-    size_t map_push[NSP] = {0, 0, 0}, map_comp = 0, map_rh = 0, map_rp = 0, map_nh = 0, map_np = 0;
-    size_t map_dh = 0, map_dp = 0;
-    int nb_push[NSP] = {0, 0, 0}, nb_comp = 0, nb_rh = 0, nb_rp = 0, nb_nh = 0, nb_np = 0;
-    int nb_dh = 0, nb_dp = 0;
+    size_t map_push[NSP] = {0, 0, 0}, map_comp = 0, map_rh = 0, map_nh = 0, map_dh = 0, map_pair = 0;
+    int nb_push[NSP] = {0, 0, 0}, nb_comp = 0, nb_rh = 0, nb_nh = 0, nb_dh = 0, nb_pair = 0;
     bool any_recomb = false, any_neutral = false, any_edet = false;
     size_t smem_push = 0, smem_field = 0, smem_hist = 0;
 };
@@ -1252,7 +1263,7 @@ int fused_tables(o2pic_batch* b) {
         b->any_neutral |= P.have_neutral != 0;
         for (int sp = 0; sp < NSP; ++sp) b->smem_push = std::max(b->smem_push, push_smem_bytes(sp, P));
         b->smem_field = std::max(b->smem_field, field_smem_bytes(P));
-        b->smem_hist = std::max(b->smem_hist, 3 * sizeof(unsigned) * (size_t)P.Nc);
+        b->smem_hist = std::max(b->smem_hist, pair_count_smem_bytes(P.Nc));
     }
     for (int sp = 0; sp < NSP; ++sp)
         add_map(b->map_push[sp], b->nb_push[sp], [&](o2pic_ctx* c) { return c->grid_push[sp]; });
@@ -1263,15 +1274,20 @@ int fused_tables(o2pic_batch* b) {
             for (unsigned j = 0; j < k; ++j) map.push_back(make_uint4((unsigned)i, j, k, sp));
         }
     b->nb_comp = (int)(map.size() - b->map_comp);
-    add_map(b->map_dh, b->nb_dh, [&](o2pic_ctx* c) {
-        return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap) + tiles(c->P.sp[SP_E].cap), 32); });
-    add_map(b->map_dp, b->nb_dp, [&](o2pic_ctx* c) { return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap), 64); });
-    add_map(b->map_rh, b->nb_rh, [&](o2pic_ctx* c) {
-        return std::min<unsigned long long>(tiles(c->P.sp[SP_E].cap) + tiles(c->P.sp[SP_OP].cap), 32); });
-    add_map(b->map_rp, b->nb_rp, [&](o2pic_ctx* c) { return std::min<unsigned long long>(tiles(c->P.sp[SP_E].cap), 64); });
-    add_map(b->map_nh, b->nb_nh, [&](o2pic_ctx* c) {
-        return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap) + tiles(c->P.sp[SP_OP].cap), 32); });
-    add_map(b->map_np, b->nb_np, [&](o2pic_ctx* c) { return std::min<unsigned long long>(tiles(c->P.sp[SP_OM].cap), 64); });
+    // pair counts: blocks of A and of B (.w), then the candidates' blocks
+    auto add_count = [&](size_t& off, int& nb, int A, int B) {
+        off = map.size();
+        for (size_t i = 0; i < n; ++i)
+            for (unsigned w = 0; w < 2; ++w) {
+                const unsigned k = (unsigned)std::min<unsigned long long>(tiles(b->ctx[i]->P.sp[w ? B : A].cap), 32);
+                for (unsigned j = 0; j < k; ++j) map.push_back(make_uint4((unsigned)i, j, k, w));
+            }
+        nb = (int)(map.size() - off);
+    };
+    add_count(b->map_dh, b->nb_dh, SP_OM, SP_E);
+    add_count(b->map_rh, b->nb_rh, SP_E, SP_OP);
+    add_count(b->map_nh, b->nb_nh, SP_OM, SP_OP);
+    add_map(b->map_pair, b->nb_pair, [&](o2pic_ctx*) { return 16; });
     if (b->dP) cudaFree(b->dP);
     if (b->dR) cudaFree(b->dR);
     if (b->dD) cudaFree(b->dD);
@@ -1315,20 +1331,20 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
                 launches += 2;
             }
             if (b->any_edet) {
-                launch_pair_hist_batched(b->dP, b->dD, b->dmap + b->map_dh, b->nb_dh, b->smem_hist, s);
-                launch_pair_batched(b->dP, b->dD, b->dmap + b->map_dp, b->nb_dp, s);
+                launch_pair_count_batched(b->dP, b->dD, b->dmap + b->map_dh, b->nb_dh, b->smem_hist, s);
+                launch_pair_batched(b->dP, b->dD, b->dmap + b->map_pair, b->nb_pair, s);
                 launch_edet_apply_batched(b->dP, b->dD, n, s);
                 launches += 3;
             }
             if (b->any_recomb) {
-                launch_pair_hist_batched(b->dP, b->dR, b->dmap + b->map_rh, b->nb_rh, b->smem_hist, s);
-                launch_pair_batched(b->dP, b->dR, b->dmap + b->map_rp, b->nb_rp, s);
+                launch_pair_count_batched(b->dP, b->dR, b->dmap + b->map_rh, b->nb_rh, b->smem_hist, s);
+                launch_pair_batched(b->dP, b->dR, b->dmap + b->map_pair, b->nb_pair, s);
                 launch_pair_apply_batched(b->dP, b->dR, n, s);
                 launches += 3;
             }
             if (b->any_neutral) {
-                launch_pair_hist_batched(b->dP, b->dN, b->dmap + b->map_nh, b->nb_nh, b->smem_hist, s);
-                launch_pair_batched(b->dP, b->dN, b->dmap + b->map_np, b->nb_np, s);
+                launch_pair_count_batched(b->dP, b->dN, b->dmap + b->map_nh, b->nb_nh, b->smem_hist, s);
+                launch_pair_batched(b->dP, b->dN, b->dmap + b->map_pair, b->nb_pair, s);
                 launches += 2;
             }
         }
