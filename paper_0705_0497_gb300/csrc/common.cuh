@@ -262,7 +262,9 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* ws, un
 // kernel may be scheduled while its predecessor in the stream still runs.
 // pdl_wait() returns once the predecessor has completed and its writes are
 // visible (immediately for a normal launch), so every such kernel calls it
-// before it reads anything a predecessor wrote.  pdl_trigger() lets the
+// before it reads anything a predecessor wrote, in every block (a grid that
+// ended before its predecessor would let its successor run too early).
+// pdl_trigger() lets the
 // successor be scheduled once every block of this grid has issued it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

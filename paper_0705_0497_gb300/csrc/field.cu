@@ -51,8 +51,16 @@ __device__ __forceinline__ unsigned cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Cluster barrier (not the .aligned form, which needs a converged warp: the
+// loops before a barrier diverge).
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
 // v into the same shared-memory word of block `rank` of the cluster
 __device__ __forceinline__ void store_remote(long long* p, unsigned rank, long long v) {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
@@ -457,14 +465,26 @@ __device__ __forceinline__ void step_commit(const Params& P, int mode, int pushe
 // when more than a fraction of the slots is dead.
 __device__ __forceinline__ void compact_body(const Params& P, int S, CompactShared& sh) {
     DevCtrl* C = P.ctrl;
-    const unsigned long long nslots = C->slots[S];
-    const unsigned long long live = C->live[S];
-    const unsigned long long dead = nslots - live;
-    const bool many_dead = (double)dead > (double)P.compact_dead_frac * (double)nslots;
-    const bool near_full = dead > 0 && 4 * nslots > 3 * P.sp[S].cap;
-    if (!many_dead && !near_full) return;
+    // One thread decides for the block: the block of the last tile writes the
+    // new counts while blocks may still be starting, and the threads of one of
+    // those must not differ.  (Such a block claims no tile, whatever mixture of
+    // counts it sees: all tiles are claimed by then.)
+    if (threadIdx.x == 0) {
+        const unsigned long long n = C->slots[S];
+        const unsigned long long dead = n - C->live[S];
+        const bool many_dead = (double)dead > (double)P.compact_dead_frac * (double)n;
+        const bool near_full = dead > 0 && 4 * n > 3 * P.sp[S].cap;
+        sh.excl = n;
+        sh.tile = C->cur[S];
+        sh.ok = (many_dead || near_full) ? 1 : 0;
+    }
+    __syncthreads();
+    const unsigned long long nslots = sh.excl;
+    const unsigned cb = sh.tile, nb = cb ^ 1u;
+    const bool go = sh.ok != 0;
+    __syncthreads();
+    if (!go) return;
     const SpeciesBuf& B = P.sp[S];
-    const unsigned cb = C->cur[S], nb = cb ^ 1u;
     const unsigned long long cap = B.cap;
     compact_tiles(
         sh, B.x[cb], nslots, &C->ticket[NKK + S], P.lb_flag[S], P.lb_val[S], C->epoch, &C->error_flags,

@@ -442,7 +442,10 @@ __global__ void __launch_bounds__(HIST_T, 2) k_pair_count_b(const Params* __rest
     __shared__ Params sP;
     const uint4 m = map[blockIdx.x];
     const PairSpec Sp = specs[m.x];
-    if (!Sp.active) return;   // block-uniform
+    if (!Sp.active) {         // block-uniform; no block may end before the predecessor has
+        pdl_wait();
+        return;
+    }
     load_params(sP, all + m.x);
     if (m.w == 0u) pair_count_body<true>(sP, Sp, m.y, m.z);
     else pair_count_body<false>(sP, Sp, m.y, m.z);
