@@ -262,9 +262,7 @@ __host__ __device__ inline unsigned warp_range_len(unsigned n, unsigned W) {
 // ---------------------------------------------------------------- launchers
 // (defined in the kernel translation units, called by the runtime)
 void launch_push(int species, const Params& P, int grid, cudaStream_t s);
-void launch_cand(int species, const Params& P, int grid, cudaStream_t s);   // ion species
-void launch_filter(int species, const Params& P, int grid, cudaStream_t s);
-void launch_filter_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
+void launch_ion(int species, const Params& P, int grid, cudaStream_t s);   // collisions of an ion species
 // na blocks for species A (counts and draws), nb for B (counts); either may be 0
 void launch_pair_count(const Params& P, const PairSpec& S, int na, int nb, cudaStream_t s);
 cudaError_t configure_pair_count_smem(int Nc);
@@ -277,7 +275,7 @@ cudaError_t configure_coulomb_smem(int Nc);
 void launch_edet_apply_batched(const Params* all, const PairSpec* specs, int n, cudaStream_t s);
 // batched launches (one grid for many discharges; map[b] = discharge, block, blocks)
 void launch_push_batched(int species, const Params* all, const uint4* map, int nblocks, size_t smem, cudaStream_t s);
-void launch_cand_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
+void launch_ion_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_field_batched(const Params* all, int n, size_t smem, int mode, int pushed_mask, cudaStream_t s);
 void launch_compact_batched(const Params* all, const uint4* map, int nblocks, cudaStream_t s);
 void launch_pair_count_batched(const Params* all, const PairSpec* specs, const uint4* map, int nblocks, size_t smem,

@@ -35,10 +35,10 @@
 //     collisions are recorded (32 B each: slot, id, x, v), and the warp runs
 //     their kinematics itself once its range is pushed, while other warps
 //     are still pushing (no second kernel on electron steps);
-//   * ions: candidates are recorded (slot and the rest of the Philox block),
-//     a lean filter kernel (target sampled from the gas Maxwellian, energy
-//     against the total rate) keeps the real ones, and the kinematics kernel
-//     handles those, 32 at a time;
+//   * ions: candidates are recorded (slot and the rest of the Philox block) and
+//     a second kernel filters them (target sampled from the gas Maxwellian,
+//     energy against the total rate) and runs the kinematics of the real ones
+//     (inside the particle kernel the target draws cost registers and time);
 //   * births are ranked with warp ballots and staged at the warp's range;
 //     the end-of-step kernel places them in parent order.
 #include "common.cuh"
@@ -54,10 +54,10 @@
 #ifndef O2PIC_PUSH_E_MIN_BLOCKS
 #define O2PIC_PUSH_E_MIN_BLOCKS 3
 #endif
-// Minimum resident blocks per SM of the kinematics kernel (caps its registers
-// at 85, no spills; 3 timed fastest of 2, 3, 4 on the same workload).
-#ifndef O2PIC_CAND_MIN_BLOCKS
-#define O2PIC_CAND_MIN_BLOCKS 3
+// Minimum resident blocks per SM of the ion collision kernel (caps its
+// registers; the particle kernel's grid then runs in one wave).
+#ifndef O2PIC_ION_MIN_BLOCKS
+#define O2PIC_ION_MIN_BLOCKS 3
 #endif
 
 namespace o2 {
@@ -79,11 +79,20 @@ struct PushShared {
     unsigned psteps;
     unsigned nonfinite;
     unsigned wtries;
-    unsigned events[MAXPROC];    // electrons: real collisions per process
-    // electrons: the block's pool of collisions (see push_body)
+};
+
+// A block's real collisions and their births (see collide_tail).
+struct CollideShared {
+    unsigned events[MAXPROC];                  // per process
     unsigned start[WARPS + 1];                 // place of each warp's first record in the pool
-    unsigned nb1[WARPS], nb2[WARPS];           // births of each warp's own passes (ionizations, attachments)
+    unsigned nb1[WARPS], nb2[WARPS];           // births of each warp's own passes, by bkind
     unsigned m1[WARPS], m2[WARPS];             // births of the pool, by thread
+};
+
+// The last records of each warp, record i of a warp at place i mod 32 (what is
+// pooled is read from here, without a trip to the list in memory).
+struct PushPool {
+    uint4 a[WARPS][32], b[WARPS][32];
 };
 
 // First record of particle-kernel warp gw (of W) in its species' candidate list:
@@ -249,6 +258,53 @@ __device__ __forceinline__ int collide_electron(const Params& P, const float* __
     return k;
 }
 
+// An ion's random words after u1: pairs of words, (2, 3) of block 0 (w0), then
+// (0, 1), (2, 3) of block 1, and so on; try t takes pair t.  All that an ion
+// draws is drawn in pairs (normals, directions), so the lanes of a warp need a
+// new block at the same tries.
+struct IonPairs {
+    uint4 buf;
+    uint32_t id, t;
+    template <int S>
+    __device__ __forceinline__ void next(const Params& P, unsigned long long step, float& a, float& b) {
+        uint32_t wa = buf.z, wb = buf.w;
+        if (t & 1u) {
+            buf = philox4x32_10(make_uint4((uint32_t)step, SpeciesTraits<S>::tag, (t + 1u) >> 1, (uint32_t)(step >> 32)),
+                                make_uint2(id, P.seed));
+            wa = buf.x;
+            wb = buf.y;
+        }
+        ++t;
+        a = 2.0f * uniform(wa) - 1.0f;
+        b = 2.0f * uniform(wb) - 1.0f;
+    }
+};
+
+// The gas molecule an ion meets: maxwellian() with both pairs of normals drawn
+// by one rejection loop, transformed once at its end.
+template <int S>
+__device__ __forceinline__ void gas_target(const Params& P, unsigned long long step, IonPairs& r, float& vx, float& vy,
+                                           float& vz, unsigned& warn) {
+    float a0 = 0.0f, b0 = 0.0f, s0 = 0.5f, a1 = 0.0f, s1 = 0.5f;
+    int task = 0, tries = 0;
+    while (task < 2) {
+        float a, b;
+        r.next<S>(P, step, a, b);
+        float s = fmaf(a, a, b * b);
+        if (!(s > 0.0f && s < 1.0f)) {
+            if (++tries < MAX_TRIES) continue;
+            ++warn;                    // gives up: normals 0
+            a = 0.0f; b = 0.0f; s = 0.5f;
+        }
+        if (task == 0) { a0 = a; b0 = b; s0 = s; }
+        else { a1 = a; s1 = s; }
+        ++task;
+        tries = 0;
+    }
+    const float f0 = sqrtf((-2.0f * ln_series(s0)) / s0), f1 = sqrtf((-2.0f * ln_series(s1)) / s1);
+    vx = P.sig_gas * (a0 * f0); vy = P.sig_gas * (b0 * f0); vz = P.sig_gas * (a1 * f1);
+}
+
 // One real collision of an ion, exactly in the order of the oracle (its filter
 // already counted the warnings of the target sample and the energy).  Returns
 // as collide_electron; bkind 2: detachment (the electron in b1).
@@ -259,17 +315,15 @@ __device__ __forceinline__ int collide_ion(const Params& P, const float* __restr
                                            unsigned& warn_tries) {
     alive = true;
     bkind = 0;
-    Stream st;
-    st.resume(id, P.seed, step, SpeciesTraits<S>::tag, w0, 1);
-    const float u1 = uniform(st.next());
+    IonPairs r = {w0, id, 0u};
     float vtx, vty, vtz;
     unsigned counted_by_filter = 0;
-    maxwellian(st, P.sig_gas, vtx, vty, vtz, counted_by_filter);
+    gas_target<S>(P, step, r, vtx, vty, vtz, counted_by_filter);
     const float gx = vx - vtx, gy = vy - vty, gz = vz - vtz;
     const float E = P.kappa[S] * dot3(gx, gy, gz, gx, gy, gz);
     int i; float w; bool above;
     grid_locate(E, i, w, above);
-    const int k = select_process(cum, np, u1 * P.numax[S], i, w);
+    const int k = select_process(cum, np, uniform(w0.y) * P.numax[S], i, w);
     if (k < 0) return -1;
     const float thr = P.thr[S][k];
     if (E < thr) return -1;
@@ -278,8 +332,19 @@ __device__ __forceinline__ int collide_ion(const Params& P, const float* __restr
         vx = vtx; vy = vty; vz = vtz;
         return k;
     }
-    float nx, ny, nz;
-    isotropic(st, nx, ny, nz, warn_tries);
+    float nx = 0.0f, ny = 0.0f, nz = 1.0f;     // isotropic()
+    int t = 0;
+    for (; t < MAX_TRIES; ++t) {
+        float a, b;
+        r.next<S>(P, step, a, b);
+        const float s = fmaf(a, a, b * b);
+        if (s < 1.0f) {
+            const float h = 2.0f * sqrtf(1.0f - s);
+            nx = a * h; ny = b * h; nz = 1.0f - 2.0f * s;
+            break;
+        }
+    }
+    if (t == MAX_TRIES) ++warn_tries;
     if (kind == K_ELASTIC) {
         const float gm = sqrtf(dot3(gx, gy, gz, gx, gy, gz));
         const float cmx = fmaf(P.a_m[S], vx, P.a_M[S] * vtx);
@@ -391,68 +456,6 @@ __device__ __forceinline__ void cell_sub(unsigned* cnt, unsigned* rsum, int c, u
     if (old < r) weight_wrapped(Q, c, -1);
 }
 
-// Real collisions of the list of one ion-push warp (records r0 .. r0 + n - 1, in
-// slot order), taken SEGW records per pass by the SEGW lanes of one segment of
-// the calling warp (seg_mask: its lanes; sl: this lane's index in it; lt_mask:
-// the segment's lanes below this one; nmax: the longest list among the warp's
-// segments, so that every lane makes the same passes).  Records carry the
-// slot, id, v and block 0 of the Philox stream (its first word, the candidate
-// draw, is spent); x is read from the array.  A removed particle's charge
-// comes off the step's deposit.  Births are ranked with ballots within the
-// segment and staged at the push warp's slot range; nb counts them.
-template <int S, int SEGW>
-__device__ __forceinline__ void collide_list(const Params& P, unsigned long long step, unsigned r0, unsigned n,
-                                             unsigned nmax, unsigned sl, unsigned seg_mask, unsigned lt_mask,
-                                             unsigned* events, unsigned& nb, unsigned& nremoved, unsigned& wtries) {
-    const int np = P.nproc[S];
-    const float* __restrict__ cum = P.cum[S];
-    const unsigned cb = P.ctrl->cur[S];
-    float* __restrict__ X = P.sp[S].x[cb];
-    float* __restrict__ VX = P.sp[S].vx[cb];
-    float* __restrict__ VY = P.sp[S].vy[cb];
-    float* __restrict__ VZ = P.sp[S].vz[cb];
-    const uint4* __restrict__ CAND = P.cand[S];
-    const float inv_dx = P.inv_dx;
-    const int Nc = P.Nc;
-    const bool births = S == SP_OM && P.births_possible[S] != 0;
-    for (unsigned c0 = 0; c0 < nmax; c0 += SEGW) {
-        const unsigned ci = c0 + sl;
-        const bool has = ci < n;
-        int bkind = 0;
-        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (has) {
-            const uint4 a = CAND[2 * (size_t)(r0 + ci)], b = CAND[2 * (size_t)(r0 + ci) + 1];
-            const unsigned slot = a.x;
-            const float x = X[slot];
-            float vx = __uint_as_float(a.z), vy = __uint_as_float(a.w), vz = __uint_as_float(b.x);
-            bool alive;
-            const int k = collide_ion<S>(P, cum, np, step, a.y, make_uint4(a.y, b.y, b.z, b.w), x, vx, vy, vz, alive,
-                                         bkind, b1, wtries);
-            if (k >= 0) {
-                atomicAdd(&events[k], 1u);
-                if (alive) {
-                    VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
-                } else {
-                    X[slot] = dead_marker();
-                    deposit_sub_global(P.Qf[S], x, inv_dx, Nc);
-                    ++nremoved;
-                }
-            }
-        }
-        if (births) {
-            // staged for the end-of-step kernel, which places them; their
-            // charge goes to Qb now
-            const unsigned m = __ballot_sync(0xffffffffu, bkind == 2) & seg_mask;
-            if (bkind == 2) {
-                P.stage[B_E_FROM_OM][r0 + nb + __popc(m & lt_mask)] = b1;
-                deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
-            }
-            nb += __popc(m);
-        }
-        __syncwarp();
-    }
-}
-
 // Set bits [a, b) of the 32-bit words in m (b - a <= 32).
 __device__ __forceinline__ unsigned bits_between(const unsigned* m, unsigned a, unsigned b) {
     if (a >= b) return 0u;
@@ -461,17 +464,131 @@ __device__ __forceinline__ unsigned bits_between(const unsigned* m, unsigned a, 
     return wa == wb ? __popc(m[wa] & lo & hi) : __popc(m[wa] & lo) + __popc(m[wb] & hi);
 }
 
+// The kinematics of a block's real collisions: nrec records of this warp
+// {slot, id, vx, vy}{vz, w1, w2, w3} from CAND[2 rec0] on, in slot order, the
+// last ones also in `pool`.  Each warp takes its own records 32 at a time, and
+// what is left (fewer than 32 per warp) is pooled over the block, in warp
+// order, one record per thread, so that short lists still fill their warps
+// (1.5e6 electrons: 14 records per warp).  A removed particle's charge comes
+// off the block's deposit when `cnt` is given (the particle kernel), else off
+// the step's deposit in memory.  The filter counted the warnings of the part
+// it shares with the kinematics.  Births are staged at their warp's slot range
+// [gw R, ...) in slot order (those of its own passes, then those of its pooled
+// records), with their number per warp, for the end-of-step kernel, which
+// places them; their charge goes to Qb now.
+template <int S>
+__device__ __forceinline__ void collide_tail(const Params& P, CollideShared& sh, PushPool& pool, unsigned blk,
+                                             unsigned long long step, unsigned cb, unsigned R, unsigned rec0,
+                                             unsigned nrec, unsigned* cnt, unsigned* rsum, unsigned long long* Qcopy,
+                                             unsigned& nrm, unsigned& wtries) {
+    const int np = P.nproc[S];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    float* __restrict__ X = P.sp[S].x[cb];
+    float* __restrict__ VX = P.sp[S].vx[cb];
+    float* __restrict__ VY = P.sp[S].vy[cb];
+    float* __restrict__ VZ = P.sp[S].vz[cb];
+    const uint4* CAND = P.cand[S];             // written by this warp just now
+    const float inv_dx = P.inv_dx;
+    const int Nc = P.Nc;
+    const unsigned own = nrec & ~31u;
+    unsigned nb1 = 0, nb2 = 0;   // warp-uniform: births of its own passes
+    if (lane == 0) sh.start[warp + 1] = nrec - own;
+    __syncthreads();
+    if (warp == 0) {
+        unsigned v = lane < WARPS ? sh.start[lane + 1] : 0u;
+#pragma unroll
+        for (int o = 1; o < WARPS; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane < WARPS) sh.start[lane + 1] = v;
+        if (lane == 0) sh.start[0] = 0u;
+    }
+    __syncthreads();
+    const unsigned pooled = sh.start[WARPS];
+    const bool births = S != SP_OP && P.births_possible[S] != 0;
+    unsigned u = (unsigned)warp;              // the warp whose record this is
+    for (unsigned c = 0;; c += 32u) {
+        const bool last = c >= own;           // the pool
+        bool has = true;
+        if (last) {
+            has = (unsigned)tid < pooled;
+            for (u = 0; u < WARPS - 1 && (unsigned)tid >= sh.start[u + 1]; ++u) {}
+        }
+        int bkind = 0;
+        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = b1;
+        if (has) {
+            const unsigned i = (unsigned)tid - sh.start[u];   // (pool)
+            const uint4 a = last ? pool.a[u][i] : CAND[2 * (size_t)(rec0 + c + lane)];
+            const uint4 b = last ? pool.b[u][i] : CAND[2 * (size_t)(rec0 + c + lane) + 1];
+            const unsigned slot = a.x;
+            const float x = S != SP_OP ? X[slot] : 0.0f;      // needed late: births, removals
+            float vx = __uint_as_float(a.z), vy = __uint_as_float(a.w), vz = __uint_as_float(b.x);
+            bool alive;
+            const int k = S == SP_E ? collide_electron(P, P.cum[S], np, step, a.y, b, x, vx, vy, vz, alive, bkind, b1,
+                                                       b2, wtries)
+                                    : collide_ion<S>(P, P.cum[S], np, step, a.y, b, x, vx, vy, vz, alive, bkind, b1,
+                                                     wtries);
+            if (k >= 0) {
+                atomicAdd(&sh.events[k], 1u);
+                if (S == SP_OP || alive) {
+                    VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
+                } else {
+                    X[slot] = dead_marker();
+                    if (S == SP_E) {
+                        int j; float f;
+                        cell_of(x, inv_dx, Nc, j, f);
+                        cell_sub(cnt, rsum, j, cic_r(f), Qcopy);
+                    } else {
+                        deposit_sub_global(P.Qf[S], x, inv_dx, Nc);
+                    }
+                    ++nrm;
+                }
+            }
+        }
+        if (S == SP_OP) {
+            if (last) break;
+            continue;
+        }
+        const unsigned m1 = __ballot_sync(0xffffffffu, bkind == 1), m2 = __ballot_sync(0xffffffffu, bkind == 2);
+        unsigned rank1 = nb1 + __popc(m1 & lt_mask), rank2 = nb2 + __popc(m2 & lt_mask), w = blk * WARPS + warp;
+        if (last) {
+            if (lane == 0) { sh.nb1[warp] = nb1; sh.nb2[warp] = nb2; sh.m1[warp] = m1; sh.m2[warp] = m2; }
+            __syncthreads();
+            if (bkind) {
+                rank1 = sh.nb1[u] + bits_between(sh.m1, sh.start[u], (unsigned)tid);
+                rank2 = sh.nb2[u] + bits_between(sh.m2, sh.start[u], (unsigned)tid);
+                w = blk * WARPS + u;
+            }
+        }
+        const unsigned s0 = w * R;
+        if (bkind == 1) {
+            P.stage[B_E_FROM_E][s0 + rank1] = b1;
+            P.stage[B_OP_FROM_E][s0 + rank1] = b2;
+            deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
+            deposit_add_global(P.Qb[SP_OP], b2.x, inv_dx, Nc);
+        } else if (bkind == 2) {
+            P.stage[S == SP_E ? B_OM_FROM_E : B_E_FROM_OM][s0 + rank2] = b1;
+            deposit_add_global(P.Qb[S == SP_E ? SP_OM : SP_E], b1.x, inv_dx, Nc);
+        }
+        if (last) break;
+        nb1 += __popc(m1);
+        nb2 += __popc(m2);
+    }
+    if (births && tid < WARPS) {
+        const unsigned w = blk * WARPS + tid, a = sh.start[tid], b = sh.start[tid + 1];
+        if (S == SP_E) P.wcount[B_E_FROM_E][w] = sh.nb1[tid] + bits_between(sh.m1, a, b);
+        P.wcount[S == SP_E ? B_OM_FROM_E : B_E_FROM_OM][w] = sh.nb2[tid] + bits_between(sh.m2, a, b);
+    }
+}
+
 // Candidate queue of one warp of the particle kernel (shared memory): the slots
 // of its candidates in slot order.  Fewer than 32 stay from one round to the
 // next and a round adds at most ROUND.
 constexpr int QN = 32 + ROUND;
 struct PushQueue {
     unsigned slot[WARPS][QN];
-};
-// Electrons: the last records of each warp, record i of a warp at place i mod 32
-// (what is pooled is read from here, without a trip to the list in memory).
-struct PushPool {
-    uint4 a[WARPS][32], b[WARPS][32];
 };
 
 // Body of the particle kernel for block blk of nblk blocks (the launch's own
@@ -482,7 +599,9 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     const int np = P.nproc[S];
     PushShared& sh = *reinterpret_cast<PushShared*>(smem);
     PushPool& pool = *reinterpret_cast<PushPool*>(smem + align16(sizeof(PushShared)));   // electrons only
-    unsigned char* rest = smem + align16(sizeof(PushShared)) + (S == SP_E ? sizeof(PushPool) : 0);
+    CollideShared& ch = *reinterpret_cast<CollideShared*>(&pool + 1);                    // electrons only
+    unsigned char* rest = smem + align16(sizeof(PushShared)) +
+                          (S == SP_E ? sizeof(PushPool) + align16(sizeof(CollideShared)) : 0);
     float* Es = reinterpret_cast<float*>(rest);
     unsigned* cnt = reinterpret_cast<unsigned*>(Es + P.Ng);
     unsigned* rsum = cnt + P.Ng;
@@ -501,7 +620,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
         sh.absorbed[0] = sh.absorbed[1] = 0u; sh.removed = 0u; sh.psteps = 0u; sh.nonfinite = 0u; sh.wtries = 0u;
         sh.jsum = 0ull;
     }
-    if (electrons && tid < MAXPROC) sh.events[tid] = 0u;
+    if (electrons && tid < MAXPROC) ch.events[tid] = 0u;
     pdl_wait();
 
     DevCtrl* C = P.ctrl;
@@ -515,7 +634,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     float* __restrict__ VZ = P.sp[S].vz[cb];
     const uint32_t* __restrict__ ID = P.sp[S].id[cb];
     uint32_t* __restrict__ TC = P.sp[S].tc[cb];
-    uint4* CAND = P.cand[S];          // written by one warp, read by others of the block
+    uint4* CAND = P.cand[S];
     const float qmdt = P.qmdt[S], dts = P.dt_s[S], inv_dx = P.inv_dx, Lf = P.Lf;
     const float inv_lnq = P.inv_lnq[S], kcap = P.kcap[S];
     const unsigned sub = P.sub[S];
@@ -721,95 +840,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     if (qn > 0u) flush(0u, qn);
     unsigned nrm = 0;
     if (electrons) {
-        // The real collisions: each warp takes its own records 32 at a time,
-        // and what is left (fewer than 32 per warp) is pooled over the block,
-        // in warp order, one record per thread, so that short lists still fill
-        // their warps (1.5e6 electrons: 11 records per warp).  A removed
-        // particle's charge comes off this block's deposit.  The filter
-        // counted the warnings of the part it shares with the kinematics.
-        // Births are staged at their warp's slot range in slot order: those of
-        // its own passes, then those of its pooled records.
-        const unsigned own = nrec & ~31u;
-        unsigned nb1 = 0, nb2 = 0;   // warp-uniform: births of its own passes
-        if (lane == 0) sh.start[warp + 1] = nrec - own;
-        __syncthreads();
-        if (warp == 0) {
-            unsigned v = lane < WARPS ? sh.start[lane + 1] : 0u;
-#pragma unroll
-            for (int o = 1; o < WARPS; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            if (lane < WARPS) sh.start[lane + 1] = v;
-            if (lane == 0) sh.start[0] = 0u;
-        }
-        __syncthreads();
-        const unsigned pooled = sh.start[WARPS];
-        const bool births = P.births_possible[S] != 0;
-        int bkind = 0;
-        float4 b1 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = b1;
-        unsigned u = (unsigned)warp;              // the warp whose record this is
-        for (unsigned c = 0;; c += 32u) {
-            const bool last = c >= own;           // the pool
-            bool has = true;
-            if (last) {
-                has = (unsigned)tid < pooled;
-                for (u = 0; u < WARPS - 1 && (unsigned)tid >= sh.start[u + 1]; ++u) {}
-            }
-            bkind = 0;
-            if (has) {
-                const unsigned i = (unsigned)tid - sh.start[u];   // (pool)
-                const uint4 a = last ? pool.a[u][i] : CAND[2 * (size_t)(rec0 + c + lane)];
-                const uint4 b = last ? pool.b[u][i] : CAND[2 * (size_t)(rec0 + c + lane) + 1];
-                const unsigned slot = a.x;
-                const float x = X[slot];                          // needed late: births, removals
-                float vx = __uint_as_float(a.z), vy = __uint_as_float(a.w), vz = __uint_as_float(b.x);
-                bool alive;
-                const int k = collide_electron(P, P.cum[S], np, step, a.y, b, x, vx, vy, vz, alive, bkind, b1, b2,
-                                               wtries);
-                if (k >= 0) {
-                    atomicAdd(&sh.events[k], 1u);
-                    if (alive) {
-                        VX[slot] = vx; VY[slot] = vy; VZ[slot] = vz;
-                    } else {
-                        X[slot] = dead_marker();
-                        int j; float f;
-                        cell_of(x, inv_dx, Nc, j, f);
-                        cell_sub(cnt, rsum, j, cic_r(f), Qcopy);
-                        ++nrm;
-                    }
-                }
-            }
-            const unsigned m1 = __ballot_sync(0xffffffffu, bkind == 1), m2 = __ballot_sync(0xffffffffu, bkind == 2);
-            unsigned rank1 = nb1 + __popc(m1 & lt_mask), rank2 = nb2 + __popc(m2 & lt_mask), s0 = r0;
-            if (last) {
-                if (lane == 0) { sh.nb1[warp] = nb1; sh.nb2[warp] = nb2; sh.m1[warp] = m1; sh.m2[warp] = m2; }
-                __syncthreads();
-                if (bkind) {
-                    rank1 = sh.nb1[u] + bits_between(sh.m1, sh.start[u], (unsigned)tid);
-                    rank2 = sh.nb2[u] + bits_between(sh.m2, sh.start[u], (unsigned)tid);
-                    s0 = (blk * WARPS + u) * R;
-                }
-            }
-            // staged for the end-of-step kernel, which places them; their
-            // charge goes to Qb now
-            if (bkind == 1) {
-                P.stage[B_E_FROM_E][s0 + rank1] = b1;
-                P.stage[B_OP_FROM_E][s0 + rank1] = b2;
-                deposit_add_global(P.Qb[SP_E], b1.x, inv_dx, Nc);
-                deposit_add_global(P.Qb[SP_OP], b2.x, inv_dx, Nc);
-            } else if (bkind == 2) {
-                P.stage[B_OM_FROM_E][s0 + rank2] = b1;
-                deposit_add_global(P.Qb[SP_OM], b1.x, inv_dx, Nc);
-            }
-            if (last) break;
-            nb1 += __popc(m1);
-            nb2 += __popc(m2);
-        }
-        if (births && tid < WARPS) {
-            P.wcount[B_E_FROM_E][blk * WARPS + tid] = sh.nb1[tid] + bits_between(sh.m1, sh.start[tid], sh.start[tid + 1]);
-            P.wcount[B_OM_FROM_E][blk * WARPS + tid] = sh.nb2[tid] + bits_between(sh.m2, sh.start[tid], sh.start[tid + 1]);
-        }
+        collide_tail<S>(P, ch, pool, blk, step, cb, R, rec0, nrec, cnt, rsum, Qcopy, nrm, wtries);
     } else if (lane == 0) {
         P.ccount[S][gw] = nrec;
     }
@@ -825,7 +856,7 @@ __device__ __forceinline__ void push_body(const Params& P, unsigned blk, unsigne
     if (wemax) atomicAdd(&C->cnt.warn_emax, (unsigned long long)wemax);
     if (wnumax) atomicAdd(&C->cnt.warn_numax, (unsigned long long)wnumax);
     __syncthreads();
-    if (electrons && tid < np && sh.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)sh.events[tid]);
+    if (electrons && tid < np && ch.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)ch.events[tid]);
     // one 64-bit add per node: what its two cells give it
     unsigned kept = 0;
     for (int j = tid; j < Ng; j += BLOCK) {
@@ -878,136 +909,91 @@ __global__ void k_flight_init(Params P) {
     }
 }
 
-// Filter of the ion candidates of one species (one warp per warp of the
-// particle kernel, walking its candidate list in slot order): the target
-// sampled from the gas Maxwellian, the relative energy and the total rate
-// against u1 nu_max, the same arithmetic as the start of collide().  It reads
-// the records only (they carry the velocities and the Philox words).  The
-// real collisions keep their records, compacted in place at the start of the
-// list (a record is written only over one already read), and the list length
-// becomes their number.  This kernel carries no kinematics, so it runs at a
-// far higher occupancy than the kinematics kernel, which then sees only the
-// real collisions.
+// Collisions of one ion species: block b of the particle kernel's grid takes the
+// candidate lists of that kernel's block b, a warp each.  The filter: target
+// sampled from the gas Maxwellian, relative energy and total rate against u1
+// nu_max, the same arithmetic as the start of collide_ion(); it reads the
+// records only (they carry the velocities and the Philox words).  The real
+// collisions (some in ten) keep their records, compacted in place at the start
+// of the list (a record is written only over one already read), then run
+// through the kinematics, pooled over the block.
 template <int S>
-__device__ __forceinline__ void filter_body(const Params& P, unsigned blk, unsigned nblk) {
+__device__ __forceinline__ void ion_body(const Params& P, unsigned blk) {
     __shared__ float tot[NGRID];
-    __shared__ unsigned sh_wtries, sh_wemax;
+    __shared__ PushPool pool;
+    __shared__ CollideShared ch;
+    __shared__ unsigned sh_wtries, sh_wemax, sh_removed;
+    const int np = P.nproc[S];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
-    if (tid == 0) { sh_wtries = 0u; sh_wemax = 0u; }
+    if (tid == 0) { sh_wtries = 0u; sh_wemax = 0u; sh_removed = 0u; }
+    if (tid < MAXPROC) ch.events[tid] = 0u;
     stage_total(P, S, tot);
     __syncthreads();
+    pdl_wait();
     DevCtrl* C = P.ctrl;
     const unsigned long long step = C->step;
+    const unsigned cb = C->cur[S];
     const unsigned nslots = (unsigned)((C->slots[S] < P.sp[S].cap) ? C->slots[S] : P.sp[S].cap);
     uint4* CAND = P.cand[S];
-    const unsigned W = P.push_warps[S];
-    const float numax = P.numax[S], kap = P.kappa[S], sig = P.sig_gas;
-    unsigned wtries = 0, wemax = 0, wnumax = 0;
-    for (unsigned gw = blk * WARPS + warp; gw < W; gw += nblk * WARPS) {
-        const unsigned r0 = list_start<S>(gw, W, nslots);
-        const unsigned n = P.ccount[S][gw];
-        unsigned nreal = 0;   // warp-uniform
-        for (unsigned c0 = 0; c0 < n; c0 += 64) {
-            uint4 a[2], b[2];
+    const unsigned W = P.push_warps[S], gw = blk * WARPS + (unsigned)warp;
+    const float numax = P.numax[S], kap = P.kappa[S];
+    unsigned wtries = 0, wemax = 0, wnumax = 0, nremoved = 0;
+    const unsigned r0 = list_start<S>(gw, W, nslots);
+    const unsigned n = P.ccount[S][gw];
+    unsigned nreal = 0;   // warp-uniform
+    for (unsigned c0 = 0; c0 < n; c0 += 64) {
+        uint4 a[2], b[2];
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const unsigned ci = c0 + 32u * k + lane;
-                const bool in = ci < n;
-                a[k] = in ? CAND[2 * (size_t)(r0 + ci)] : make_uint4(0u, 0u, 0u, 0u);
-                b[k] = in ? CAND[2 * (size_t)(r0 + ci) + 1] : make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (c0 + 32u * k >= n) break;   // warp-uniform
-                const bool in = c0 + 32u * k + lane < n;
-                bool real = false;
-                if (in) {
-                    Stream st;
-                    st.resume(a[k].y, P.seed, step, SpeciesTraits<S>::tag, make_uint4(a[k].y, b[k].y, b[k].z, b[k].w), 1);
-                    const float u1 = uniform(st.next());
-                    float vtx, vty, vtz;
-                    maxwellian(st, sig, vtx, vty, vtz, wtries);
-                    const float gx = __uint_as_float(a[k].z) - vtx, gy = __uint_as_float(a[k].w) - vty,
-                                gz = __uint_as_float(b[k].x) - vtz;
-                    const float E = kap * dot3(gx, gy, gz, gx, gy, gz);
-                    int i; float w; bool above;
-                    grid_locate(E, i, w, above);
-                    if (above) ++wemax;
-                    const float total = grid_interp(tot, 1, 0, i, w);
-                    if (total > numax) ++wnumax;   // above a capped majorant
-                    real = (u1 * numax) < total;
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, real);
-                if (real) {
-                    const size_t q = r0 + nreal + __popc(m & lt_mask);
-                    CAND[2 * q] = a[k];
-                    CAND[2 * q + 1] = b[k];
-                }
-                nreal += __popc(m);
-            }
+        for (int k = 0; k < 2; ++k) {
+            const unsigned ci = c0 + 32u * k + lane;
+            const bool in = ci < n;
+            a[k] = in ? CAND[2 * (size_t)(r0 + ci)] : make_uint4(0u, 0u, 0u, 0u);
+            b[k] = in ? CAND[2 * (size_t)(r0 + ci) + 1] : make_uint4(0u, 0u, 0u, 0u);
         }
-        if (lane == 0) P.ccount[S][gw] = nreal;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (c0 + 32u * k >= n) break;   // warp-uniform
+            bool real = false;
+            if (c0 + 32u * k + lane < n) {
+                IonPairs r = {b[k], a[k].y, 0u};
+                float vtx, vty, vtz;
+                gas_target<S>(P, step, r, vtx, vty, vtz, wtries);
+                const float gx = __uint_as_float(a[k].z) - vtx, gy = __uint_as_float(a[k].w) - vty,
+                            gz = __uint_as_float(b[k].x) - vtz;
+                const float E = kap * dot3(gx, gy, gz, gx, gy, gz);
+                int i; float w; bool above;
+                grid_locate(E, i, w, above);
+                if (above) ++wemax;
+                const float total = grid_interp(tot, 1, 0, i, w);
+                if (total > numax) ++wnumax;   // above a capped majorant
+                real = (uniform(b[k].y) * numax) < total;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, real);
+            if (real) {
+                const unsigned i = nreal + __popc(m & lt_mask);
+                CAND[2 * (size_t)(r0 + i)] = a[k];
+                CAND[2 * (size_t)(r0 + i) + 1] = b[k];
+                pool.a[warp][i & 31u] = a[k];
+                pool.b[warp][i & 31u] = b[k];
+            }
+            nreal += __popc(m);
+        }
+        __syncwarp();
     }
+    collide_tail<S>(P, ch, pool, blk, step, cb, warp_range_len(nslots, W), r0, nreal, nullptr, nullptr, nullptr,
+                    nremoved, wtries);
     pdl_trigger();
     if (wtries) atomicAdd(&sh_wtries, wtries);
     if (wemax) atomicAdd(&sh_wemax, wemax);
+    if (nremoved) atomicAdd(&sh_removed, nremoved);
     if (wnumax) atomicAdd(&C->cnt.warn_numax, (unsigned long long)wnumax);
     __syncthreads();
-    if (tid == 0) {
-        if (sh_wtries) atomicAdd(&C->cnt.warn_tries, (unsigned long long)sh_wtries);
-        if (sh_wemax) atomicAdd(&C->cnt.warn_emax, (unsigned long long)sh_wemax);
-    }
-}
-
-// Real collisions of one ion species for this step (the electrons' run at
-// the end of their particle kernel).  Each warp takes two lists of the
-// particle kernel's warps at once, one per half-warp (16 lanes; a list holds
-// a few records at the method's rates), and walks them in slot order, 16
-// records per pass through the kinematics, so the lists of a step run in one
-// wave of resident warps.  Births are ranked with ballots within the
-// half-warp and staged at the particle warp's slot range with their count.
-constexpr int SEG = 16;
-constexpr int SEGS = 32 / SEG;
-
-template <int S>
-__device__ __forceinline__ void cand_body(const Params& P, unsigned blk, unsigned nblk) {
-    __shared__ unsigned events[MAXPROC];
-    __shared__ unsigned sh_removed, sh_wtries;
-    const int np = P.nproc[S];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned seg = (unsigned)lane / SEG, sl = (unsigned)lane % SEG;
-    const unsigned seg_mask = ((1u << SEG) - 1u) << (seg * SEG);
-    const unsigned lt_mask = ((1u << lane) - 1u) & seg_mask;   // lanes below, same half-warp
-    if (tid < MAXPROC) events[tid] = 0u;
-    if (tid == 0) { sh_removed = 0u; sh_wtries = 0u; }
-    __syncthreads();
-
-    DevCtrl* C = P.ctrl;
-    const unsigned long long step = C->step;
-    const unsigned nslots = (unsigned)((C->slots[S] < P.sp[S].cap) ? C->slots[S] : P.sp[S].cap);
-    const bool births = S == SP_OM && P.births_possible[S] != 0;
-    const unsigned W = P.push_warps[S];
-    unsigned wtries = 0, nremoved = 0;
-
-    for (unsigned gb = (blk * WARPS + warp) * SEGS; gb < W; gb += nblk * WARPS * SEGS) {
-        const unsigned gw = gb + seg;                  // this half-warp's list
-        const bool valid = gw < W;
-        const unsigned r0 = valid ? list_start<S>(gw, W, nslots) : 0u;
-        const unsigned n = valid ? P.ccount[S][gw] : 0u;
-        const unsigned nmax = max(n, __shfl_xor_sync(0xffffffffu, n, SEG));
-        unsigned nb = 0;   // half-warp-uniform
-        collide_list<S, SEG>(P, step, r0, n, nmax, sl, seg_mask, lt_mask, events, nb, nremoved, wtries);
-        if (births && valid && sl == 0) P.wcount[B_E_FROM_OM][gw] = nb;
-    }
-    pdl_trigger();
-    if (nremoved) atomicAdd(&sh_removed, nremoved);
-    if (wtries) atomicAdd(&sh_wtries, wtries);
-    __syncthreads();
-    if (tid < np && events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)events[tid]);
+    if (tid < np && ch.events[tid]) atomicAdd(&C->cnt.events[S][tid], (unsigned long long)ch.events[tid]);
     if (tid == 0) {
         if (sh_removed) atomicAdd(&C->removed[S], (unsigned long long)sh_removed);
         if (sh_wtries) atomicAdd(&C->cnt.warn_tries, (unsigned long long)sh_wtries);
+        if (sh_wemax) atomicAdd(&C->cnt.warn_emax, (unsigned long long)sh_wemax);
     }
 }
 
@@ -1020,19 +1006,8 @@ __global__ void __launch_bounds__(BLOCK, push_min_blocks<S>()) k_push(Params P) 
 }
 
 template <int S>
-__global__ void __launch_bounds__(BLOCK, O2PIC_CAND_MIN_BLOCKS) k_cand(Params P) {
-    pdl_wait();
-    cand_body<S>(P, blockIdx.x, gridDim.x);
-}
-
-// The ion filter is light (no kinematics): more resident blocks per SM.
-#ifndef O2PIC_FILTER_MIN_BLOCKS
-#define O2PIC_FILTER_MIN_BLOCKS 3
-#endif
-template <int S>
-__global__ void __launch_bounds__(BLOCK, O2PIC_FILTER_MIN_BLOCKS) k_filter(Params P) {
-    pdl_wait();
-    filter_body<S>(P, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(BLOCK, O2PIC_ION_MIN_BLOCKS) k_ion(Params P) {
+    ion_body<S>(P, blockIdx.x);
 }
 
 // Batched launches: block b works for discharge map[b].x as its block
@@ -1048,25 +1023,16 @@ __global__ void __launch_bounds__(BLOCK, push_min_blocks<S>()) k_push_b(const Pa
 }
 
 template <int S>
-__global__ void __launch_bounds__(BLOCK, O2PIC_CAND_MIN_BLOCKS) k_cand_b(const Params* __restrict__ all,
-                                                                        const uint4* __restrict__ map) {
+__global__ void __launch_bounds__(BLOCK, O2PIC_ION_MIN_BLOCKS) k_ion_b(const Params* __restrict__ all,
+                                                                      const uint4* __restrict__ map) {
     __shared__ Params sP;
-    pdl_wait();
     const uint4 m = map[blockIdx.x];
     load_params(sP, all + m.x);
-    if (sP.nproc[S] == 0) return;   // block-uniform
-    cand_body<S>(sP, m.y, m.z);
-}
-
-template <int S>
-__global__ void __launch_bounds__(BLOCK, O2PIC_FILTER_MIN_BLOCKS) k_filter_b(const Params* __restrict__ all,
-                                                                            const uint4* __restrict__ map) {
-    __shared__ Params sP;
-    pdl_wait();
-    const uint4 m = map[blockIdx.x];
-    load_params(sP, all + m.x);
-    if (sP.nproc[S] == 0) return;   // block-uniform
-    filter_body<S>(sP, m.y, m.z);
+    if (sP.nproc[S] == 0) {   // block-uniform; no block may end before the predecessor has
+        pdl_wait();
+        return;
+    }
+    ion_body<S>(sP, m.y);
 }
 
 // Deposit of all live particles of one species into Qf (used after a load).
@@ -1106,7 +1072,7 @@ __global__ void __launch_bounds__(BLOCK) k_deposit(Params P) {
 
 size_t push_smem_bytes(int species, const Params& P) {
     const size_t base = align16(sizeof(PushShared)) + (sizeof(float) + 2 * sizeof(unsigned)) * P.Ng + sizeof(PushQueue);
-    return base + (species == SP_E ? sizeof(float) * NGRID + sizeof(PushPool) : 0);
+    return base + (species == SP_E ? sizeof(float) * NGRID + sizeof(PushPool) + align16(sizeof(CollideShared)) : 0);
 }
 
 void launch_flight_init(int species, const Params& P, cudaStream_t s) {
@@ -1130,24 +1096,15 @@ void launch_push_batched(int species, const Params* all, const uint4* map, int n
     else launch_pdl(k_push_b<SP_OP>, nblocks, BLOCK, smem, s, all, map);
 }
 
-void launch_cand_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
-    if (species == SP_OM) launch_pdl(k_cand_b<SP_OM>, nblocks, BLOCK, 0, s, all, map);
-    else if (species == SP_OP) launch_pdl(k_cand_b<SP_OP>, nblocks, BLOCK, 0, s, all, map);
+// one block per block of the species' particle kernel
+void launch_ion(int species, const Params& P, int grid, cudaStream_t s) {
+    if (species == SP_OM) launch_pdl(k_ion<SP_OM>, grid, BLOCK, 0, s, P);
+    else if (species == SP_OP) launch_pdl(k_ion<SP_OP>, grid, BLOCK, 0, s, P);
 }
 
-void launch_filter(int species, const Params& P, int grid, cudaStream_t s) {
-    if (species == SP_OM) launch_pdl(k_filter<SP_OM>, grid, BLOCK, 0, s, P);
-    else if (species == SP_OP) launch_pdl(k_filter<SP_OP>, grid, BLOCK, 0, s, P);
-}
-
-void launch_filter_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
-    if (species == SP_OM) launch_pdl(k_filter_b<SP_OM>, nblocks, BLOCK, 0, s, all, map);
-    else if (species == SP_OP) launch_pdl(k_filter_b<SP_OP>, nblocks, BLOCK, 0, s, all, map);
-}
-
-void launch_cand(int species, const Params& P, int grid, cudaStream_t s) {
-    if (species == SP_OM) launch_pdl(k_cand<SP_OM>, grid, BLOCK, 0, s, P);
-    else if (species == SP_OP) launch_pdl(k_cand<SP_OP>, grid, BLOCK, 0, s, P);
+void launch_ion_batched(int species, const Params* all, const uint4* map, int nblocks, cudaStream_t s) {
+    if (species == SP_OM) launch_pdl(k_ion_b<SP_OM>, nblocks, BLOCK, 0, s, all, map);
+    else if (species == SP_OP) launch_pdl(k_ion_b<SP_OP>, nblocks, BLOCK, 0, s, all, map);
 }
 
 void launch_deposit(int species, const Params& P, int grid, cudaStream_t s) {

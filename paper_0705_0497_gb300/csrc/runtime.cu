@@ -93,7 +93,7 @@ struct o2pic_ctx {
     // ion steps: the O- and O2+ chains on their own streams beside the
     // electron kernel (forked from and joined back into the step's stream)
     cudaStream_t aux[2] = {nullptr, nullptr};
-    cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
+    cudaEvent_t ev_fork = nullptr, ev_pushed = nullptr, ev_join[2] = {nullptr, nullptr};
     Params P;
     DevCtrl* d_ctrl = nullptr;
     std::vector<void*> allocs;
@@ -186,6 +186,13 @@ void launch(o2pic_ctx* c, int kind, cudaStream_t s, F&& f) {
     }
     c->nlaunch[kind] += 1;
     c->launches += 1;
+}
+
+void destroy_streams(o2pic_ctx* c) {
+    for (cudaEvent_t e : {c->ev_fork, c->ev_pushed, c->ev_join[0], c->ev_join[1]})
+        if (e) cudaEventDestroy(e);
+    for (cudaStream_t st : {c->aux[0], c->aux[1], c->stream})
+        if (st) cudaStreamDestroy(st);
 }
 
 int check_flags(o2pic_ctx* c) {
@@ -354,22 +361,19 @@ void enqueue_steps(o2pic_ctx* c, uint64_t nsteps, cudaStream_t s) {
         launch(c, KK_PUSH_E, s, [&] { launch_push(SP_E, P, c->grid_push[SP_E], s); });
         if (ion) {
             launch(c, KK_PUSH_OM, so, [&] { launch_push(SP_OM, P, c->grid_push[SP_OM], so); });
-            if (P.nproc[SP_OM]) {
-                launch(c, KK_FILT_OM, so, [&] { launch_filter(SP_OM, P, c->grid_push[SP_OM], so); });
-                launch(c, KK_CAND_OM, so, [&] { launch_cand(SP_OM, P, c->grid_push[SP_OM], so); });
-            }
             launch(c, KK_PUSH_OP, sp2, [&] { launch_push(SP_OP, P, c->grid_push[SP_OP], sp2); });
-            if (P.nproc[SP_OP]) {
-                launch(c, KK_FILT_OP, sp2, [&] { launch_filter(SP_OP, P, c->grid_push[SP_OP], sp2); });
-                launch(c, KK_CAND_OP, sp2, [&] { launch_cand(SP_OP, P, c->grid_push[SP_OP], sp2); });
-            }
-            // (17): each species is counted behind its own chain, where no other
-            // pair process removes particles in between
+            // (17), where no other pair process removes particles before it: the
+            // O- are counted behind their own chain, the O2+ (whose collisions
+            // leave them where they are) behind their push, on the step's stream
             const bool early = fork && P.have_neutral && !P.have_edet && !P.have_recomb;
+            if (early) cudaEventRecord(c->ev_pushed, sp2);
+            if (P.nproc[SP_OM]) launch(c, KK_CAND_OM, so, [&] { launch_ion(SP_OM, P, c->grid_push[SP_OM], so); });
+            if (P.nproc[SP_OP]) launch(c, KK_CAND_OP, sp2, [&] { launch_ion(SP_OP, P, c->grid_push[SP_OP], sp2); });
             if (early) {
                 const PairSpec N = spec_neu(c);
                 launch(c, KK_PAIR_HIST, so, [&] { launch_pair_count(P, N, c->grid_count[SP_OM], 0, so); });
-                launch(c, KK_PAIR_HIST, sp2, [&] { launch_pair_count(P, N, 0, c->grid_count[SP_OP], sp2); });
+                cudaStreamWaitEvent(s, c->ev_pushed, 0);
+                launch(c, KK_PAIR_HIST, s, [&] { launch_pair_count(P, N, 0, c->grid_count[SP_OP], s); });
             }
             if (fork) {
                 cudaEventRecord(c->ev_join[0], so);
@@ -459,19 +463,10 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_pushed, cudaEventDisableTiming);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming);
     if (e != cudaSuccess) {
-        for (int i = 0; i < 2; ++i) {
-            if (c->aux[i]) cudaStreamDestroy(c->aux[i]);
-            if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
-        }
-        if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-        for (int i = 0; i < 2; ++i) {
-        if (c->aux[i]) cudaStreamDestroy(c->aux[i]);
-        if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
-    }
-    if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-    if (c->stream) cudaStreamDestroy(c->stream);
+        destroy_streams(c);
         delete c;
         return O2PIC_E_CUDA;
     }
@@ -600,7 +595,7 @@ void o2pic_destroy(o2pic_ctx* c) {
     for (void* p : c->allocs) cudaFree(p);
     for (auto& ev : c->pending) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }
     for (auto e : c->pool) cudaEventDestroy(e);
-    if (c->stream) cudaStreamDestroy(c->stream);
+    destroy_streams(c);
     delete c;
 }
 
@@ -1326,9 +1321,8 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
             for (int sp = SP_OM; sp <= SP_OP; ++sp) {
                 launch_push_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], b->smem_push, s);
                 launches += 1;
-                launch_filter_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
-                launch_cand_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
-                launches += 2;
+                launch_ion_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
+                launches += 1;
             }
             if (b->any_edet) {
                 launch_pair_count_batched(b->dP, b->dD, b->dmap + b->map_dh, b->nb_dh, b->smem_hist, s);
