@@ -213,11 +213,12 @@ struct Params {
     float4* stage22;             // [max_dremovals]
     // Coulomb (1)-(6): enabled reactions (bit r-1), per reaction the sigma^2
     // factor K and the shares m_b/(m_a+m_b), m_a/(m_a+m_b) of the change of
-    // u; per species the cell sort of a Coulomb step: slots in cell order,
-    // per-tile cell offsets, cell totals and cell starts
+    // u; per species the cell sort of a Coulomb step: entries in cell order and
+    // where each slot's is, per-tile cell offsets, cell totals and cell starts
     unsigned int coul_mask;
     float coul_K[6], coul_fa[6], coul_fb[6];
-    unsigned int* csort[NSP];
+    float4* csort[NSP];          // {vx, vy, vz, id} in cell order
+    unsigned int* cplace[NSP];   // place of each slot there
     unsigned int* chist[NSP];
     unsigned int* ctot[NSP];
     unsigned int* cstart[NSP];

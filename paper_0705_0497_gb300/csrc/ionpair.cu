@@ -113,6 +113,7 @@ __device__ __forceinline__ void pair_count_body(const Params& P, const PairSpec&
         if (FIRST) {
 #pragma unroll
             for (int i = 0; i < HIST_V; ++i) {
+                if (base + 4ull * HIST_T * i >= n) break;
                 const float xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
                 const uint32_t ids[4] = {id[i].x, id[i].y, id[i].z, id[i].w};
                 uint32_t w[4];

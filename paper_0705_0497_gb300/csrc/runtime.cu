@@ -933,6 +933,7 @@ int o2pic_set_coulomb(o2pic_ctx* c, uint32_t mask, double ln_lambda) {
         for (int s = 0; s < NSP && e == cudaSuccess; ++s) {
             const unsigned long long cap = P.sp[s].cap;
             e = ctx_alloc(c, &P.csort[s], (size_t)cap);
+            if (e == cudaSuccess) e = ctx_alloc(c, &P.cplace[s], (size_t)cap);
             if (e == cudaSuccess) e = ctx_alloc(c, &P.chist[s], (size_t)(ceil_div(cap, TILE) + 1) * P.Nc);
             if (e == cudaSuccess) e = ctx_alloc(c, &P.ctot[s], (size_t)P.Nc);
             if (e == cudaSuccess) e = ctx_alloc(c, &P.cstart[s], (size_t)P.Nc);
