@@ -96,6 +96,8 @@ struct o2pic_ctx {
     cudaEvent_t ev_fork = nullptr, ev_pushed = nullptr, ev_join[2] = {nullptr, nullptr};
     Params P;
     DevCtrl* d_ctrl = nullptr;
+    // pinned: the control block as last read (fetch), and small results
+    DevCtrl* h_ctrl = nullptr;
     std::vector<void*> allocs;
     // host state
     unsigned long long host_step = 0;
@@ -195,10 +197,9 @@ void destroy_streams(o2pic_ctx* c) {
         if (st) cudaStreamDestroy(st);
 }
 
-int check_flags(o2pic_ctx* c) {
-    unsigned long long flags = 0;
-    cudaError_t e = cudaMemcpy(&flags, &c->d_ctrl->error_flags, sizeof(flags), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e);
+// The error latched in the control block that was read last.
+int latch_flags(o2pic_ctx* c) {
+    const unsigned long long flags = c->h_ctrl->error_flags;
     int code = O2PIC_OK;
     if (flags & ERR_CAPACITY) code = O2PIC_E_CAPACITY;
     else if (flags & ERR_ID) code = O2PIC_E_ID_OVERFLOW;
@@ -208,12 +209,29 @@ int check_flags(o2pic_ctx* c) {
     return c->latched;
 }
 
-int sync_all(o2pic_ctx* c) {
+// The control block into h_ctrl, after what the context's own stream holds: one
+// copy to pinned memory and one wait, with whatever copies the caller has
+// enqueued on that stream before.
+int fetch(o2pic_ctx* c) {
+    cudaError_t e = cudaMemcpyAsync(c->h_ctrl, c->d_ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e);
+    return latch_flags(c);
+}
+
+// Waits for the device; what follows on the context's own stream (which does
+// not wait for others) then sees all earlier work.
+int device_idle(o2pic_ctx* c) {
     cudaError_t e = cudaSetDevice(c->device);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(c, e);
     if (c->timing) harvest_timing(c);
-    return check_flags(c);
+    return O2PIC_OK;
+}
+
+int sync_all(o2pic_ctx* c) {
+    if (int rc = device_idle(c)) return rc;
+    return fetch(c);
 }
 
 int validate(const o2pic_config* g) {
@@ -470,6 +488,11 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
         delete c;
         return O2PIC_E_CUDA;
     }
+    if (cudaHostAlloc((void**)&c->h_ctrl, sizeof(DevCtrl), cudaHostAllocDefault) != cudaSuccess) {
+        o2pic_destroy(c);
+        return O2PIC_E_CUDA;
+    }
+    std::memset(c->h_ctrl, 0, sizeof(DevCtrl));
     c->last = c->stream;
     set_constants(c);
     Params& P = c->P;
@@ -498,11 +521,13 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
         float* tot;
         TRY(ctx_alloc(c, &tot, NGRID));
         P.tot[s] = tot;
-        TRY(ctx_alloc(c, &P.Q[s], Ng));
         TRY(ctx_alloc(c, &P.Qf[s], (size_t)QCOPIES * Ng));
         TRY(ctx_alloc(c, &P.Qb[s], Ng));
-        TRY(ctx_alloc(c, &P.Qacc[s], Ng));
     }
+    // one array of all species each, so that a read is one copy
+    TRY(ctx_alloc(c, &P.Q[0], (size_t)NSP * Ng));
+    TRY(ctx_alloc(c, &P.Qacc[0], (size_t)NSP * Ng));
+    for (int s = 1; s < NSP; ++s) { P.Q[s] = P.Q[0] + (size_t)s * Ng; P.Qacc[s] = P.Qacc[0] + (size_t)s * Ng; }
     float* K;
     TRY(ctx_alloc(c, &K, NGRID));
     P.Ktab = K;
@@ -593,6 +618,7 @@ void o2pic_destroy(o2pic_ctx* c) {
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     for (void* p : c->allocs) cudaFree(p);
+    if (c->h_ctrl) cudaFreeHost(c->h_ctrl);
     for (auto& ev : c->pending) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }
     for (auto e : c->pool) cudaEventDestroy(e);
     destroy_streams(c);
@@ -765,9 +791,8 @@ int o2pic_load_particles(o2pic_ctx* c, int species, const float* x, const float*
     if (rc == O2PIC_E_CUDA) return rc;
     c->latched = 0;
     cudaStream_t s = pick(c, stream);
-    DevCtrl h;
-    cudaError_t e = cudaMemcpy(&h, c->d_ctrl, sizeof(h), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e);
+    DevCtrl& h = *c->h_ctrl;   // copied back by the same stream's order
+    cudaError_t e = cudaSuccess;
     const unsigned b = h.cur[species];
     const SpeciesBuf& B = c->P.sp[species];
     const cudaMemcpyKind k = (mem_kind == O2PIC_HOST) ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
@@ -790,14 +815,14 @@ int o2pic_load_particles(o2pic_ctx* c, int species, const float* x, const float*
         // both memory kinds: the particles are checked (and max(id) found) on
         // the device once they are there
         launch_load_check(species, c->P, n, s);
-        e = cudaStreamSynchronize(s);
+        e = cudaMemcpyAsync(&h, c->d_ctrl, sizeof(h), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(c, e);
-        unsigned long long flags = 0;
-        e = cudaMemcpy(&flags, &c->d_ctrl->error_flags, sizeof(flags), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(c, e);
-        if (flags & ERR_NONFINITE) {
-            // leave the species empty (h.error_flags is 0)
+        if (h.error_flags & ERR_NONFINITE) {
+            // leave the species empty, without its error and ids
             h.slots[species] = 0; h.live[species] = 0;
+            h.error_flags = 0;
+            h.next_id[species] = next;
             e = cudaMemcpy(c->d_ctrl, &h, sizeof(h), cudaMemcpyHostToDevice);
             if (e != cudaSuccess) return cuda_fail(c, e);
             return O2PIC_E_INVALID_ARG;
@@ -876,43 +901,43 @@ int o2pic_read_particles(o2pic_ctx* c, int species, float* x, float* vx, float* 
                          uint64_t cap, uint64_t* n, int mem_kind) {
     if (!c || species < 0 || species >= NSP || !n) return O2PIC_E_INVALID_ARG;
     if (mem_kind != O2PIC_HOST && mem_kind != O2PIC_DEVICE) return O2PIC_E_INVALID_ARG;
+    const bool want = cap > 0 && x && vx && vy && vz && id;
+    cudaStream_t s = c->stream;
+    if (want && mem_kind == O2PIC_DEVICE) {
+        // gathered at once (up to cap); the count comes back with the flags
+        if (int rc = device_idle(c)) return rc;
+        c->gepoch += 1;
+        cudaMemsetAsync(c->d_gticket, 0, sizeof(unsigned), s);
+        launch_gather(species, c->P, 2 * c->num_sms, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval, x,
+                      vx, vy, vz, id, nullptr, cap, c->d_gcount, s);
+        c->launches += 1;
+        const int rc = fetch(c);
+        if (rc == O2PIC_E_CUDA) return rc;
+        *n = c->h_ctrl->live[species];
+        return rc;
+    }
     int rc = sync_all(c);
     if (rc == O2PIC_E_CUDA) return rc;
-    cudaStream_t s = c->stream;
-    DevCtrl h;
-    cudaError_t e = cudaMemcpy(&h, c->d_ctrl, sizeof(h), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e);
-    *n = h.live[species];
-    const uint64_t m = std::min<uint64_t>(cap, h.live[species]);
-    if (m == 0 || !x || !vx || !vy || !vz || !id) return rc;
-    float *dx_ = x, *dvx = vx, *dvy = vy, *dvz = vz;
-    uint32_t* did = id;
-    std::vector<void*> tmp;
-    if (mem_kind == O2PIC_HOST) {
-        void* p;
-        for (int k = 0; k < 5; ++k) {
-            e = cudaMalloc(&p, 4 * m);
-            if (e != cudaSuccess) { for (void* q : tmp) cudaFree(q); return cuda_fail(c, e); }
-            tmp.push_back(p);
-        }
-        dx_ = (float*)tmp[0]; dvx = (float*)tmp[1]; dvy = (float*)tmp[2]; dvz = (float*)tmp[3]; did = (uint32_t*)tmp[4];
-    }
+    const unsigned long long live = c->h_ctrl->live[species];
+    *n = live;
+    const uint64_t m = std::min<uint64_t>(cap, live);
+    if (m == 0 || !want) return rc;
+    // host arrays: gathered into the buffer set that the compaction would fill
+    // next (nothing else uses it), then copied
+    const SpeciesBuf& B = c->P.sp[species];
+    const unsigned nb = c->h_ctrl->cur[species] ^ 1u;
     c->gepoch += 1;
     cudaMemsetAsync(c->d_gticket, 0, sizeof(unsigned), s);
     launch_gather(species, c->P, 2 * c->num_sms, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
-                  dx_, dvx, dvy, dvz, did, nullptr, m, c->d_gcount, s);
+                  B.x[nb], B.vx[nb], B.vy[nb], B.vz[nb], B.id[nb], nullptr, m, c->d_gcount, s);
     c->launches += 1;
-    e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && mem_kind == O2PIC_HOST) {
-        e = cudaMemcpy(x, dx_, 4 * m, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(vx, dvx, 4 * m, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(vy, dvy, 4 * m, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(vz, dvz, 4 * m, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(id, did, 4 * m, cudaMemcpyDeviceToHost);
-    }
-    for (void* q : tmp) cudaFree(q);
+    cudaError_t e = cudaMemcpyAsync(x, B.x[nb], 4 * m, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(vx, B.vx[nb], 4 * m, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(vy, B.vy[nb], 4 * m, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(vz, B.vz[nb], 4 * m, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(id, B.id[nb], 4 * m, cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return cuda_fail(c, e);
-    return check_flags(c);
+    return fetch(c);
 }
 
 int o2pic_set_majorant_cap(o2pic_ctx* c, const double* cap_eV) {
@@ -995,29 +1020,21 @@ int o2pic_read_flight(o2pic_ctx* c, int species, uint32_t* tc, uint64_t cap, uin
     int rc = sync_all(c);
     if (rc == O2PIC_E_CUDA) return rc;
     cudaStream_t s = c->stream;
-    DevCtrl h;
-    cudaError_t e = cudaMemcpy(&h, c->d_ctrl, sizeof(h), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e);
-    *n = h.live[species];
-    const uint64_t m = std::min<uint64_t>(cap, h.live[species]);
+    *n = c->h_ctrl->live[species];
+    const uint64_t m = std::min<uint64_t>(cap, *n);
     if (m == 0 || !tc) return rc;
-    uint32_t* dtc = tc;
-    void* tmp = nullptr;
-    if (mem_kind == O2PIC_HOST) {
-        e = cudaMalloc(&tmp, 4 * m);
-        if (e != cudaSuccess) return cuda_fail(c, e);
-        dtc = (uint32_t*)tmp;
-    }
+    const SpeciesBuf& B = c->P.sp[species];
+    uint32_t* dtc = mem_kind == O2PIC_HOST ? B.tc[c->h_ctrl->cur[species] ^ 1u] : tc;
     c->gepoch += 1;
     cudaMemsetAsync(c->d_gticket, 0, sizeof(unsigned), s);
     launch_gather(species, c->P, 2 * c->num_sms, (1ull << 60) | c->gepoch, c->d_gticket, c->d_gflag, c->d_gval,
                   nullptr, nullptr, nullptr, nullptr, nullptr, dtc, m, c->d_gcount, s);
     c->launches += 1;
-    e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && mem_kind == O2PIC_HOST) e = cudaMemcpy(tc, dtc, 4 * m, cudaMemcpyDeviceToHost);
-    if (tmp) cudaFree(tmp);
-    if (e != cudaSuccess) return cuda_fail(c, e);
-    return check_flags(c);
+    if (mem_kind == O2PIC_HOST) {
+        cudaError_t e = cudaMemcpyAsync(tc, dtc, 4 * m, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return cuda_fail(c, e);
+    }
+    return fetch(c);
 }
 
 int o2pic_read_field(o2pic_ctx* c, double* phi, float* E) {
@@ -1027,18 +1044,18 @@ int o2pic_read_field(o2pic_ctx* c, double* phi, float* E) {
         int rc = prepare(c, c->stream);
         if (rc) return rc;
     }
+    if (int rc = device_idle(c)) return rc;
     cudaError_t e = cudaSuccess;
     if (phi) {
-        e = cudaSetDevice(c->device);
-        if (e == cudaSuccess) { launch_phi(c->P, c->last); e = cudaGetLastError(); }
-        if (e != cudaSuccess) return cuda_fail(c, e);
+        launch_phi(c->P, c->stream);
+        e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(phi, c->P.phi, sizeof(double) * c->P.Ng, cudaMemcpyDeviceToHost, c->stream);
     }
-    int rc = sync_all(c);
-    if (rc == O2PIC_E_CUDA) return rc;
-    if (phi) e = cudaMemcpy(phi, c->P.phi, sizeof(double) * c->P.Ng, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && E) e = cudaMemcpy(E, c->P.Ef, sizeof(float) * c->P.Ng, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && E)
+        e = cudaMemcpyAsync(E, c->P.Ef, sizeof(float) * c->P.Ng, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e);
-    return rc;
+    return fetch(c);
 }
 
 int o2pic_read_currents(o2pic_ctx* c, uint64_t first, uint64_t n, double* out) {
@@ -1080,16 +1097,14 @@ int o2pic_read_charge(o2pic_ctx* c, uint64_t* Q, uint64_t* Qacc, uint64_t* acc_s
         int rc = prepare(c, c->stream);
         if (rc) return rc;
     }
-    int rc = sync_all(c);
-    if (rc == O2PIC_E_CUDA) return rc;
-    const int Ng = c->P.Ng;
+    if (int rc = device_idle(c)) return rc;
+    const size_t bytes = 8 * (size_t)NSP * c->P.Ng;
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < NSP && e == cudaSuccess; ++s) {
-        if (Q) e = cudaMemcpy(Q + (size_t)s * Ng, c->P.Q[s], 8 * (size_t)Ng, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess && Qacc) e = cudaMemcpy(Qacc + (size_t)s * Ng, c->P.Qacc[s], 8 * (size_t)Ng, cudaMemcpyDeviceToHost);
-    }
-    if (e == cudaSuccess && acc_steps) e = cudaMemcpy(acc_steps, &c->d_ctrl->acc_steps, 8, cudaMemcpyDeviceToHost);
+    if (Q) e = cudaMemcpyAsync(Q, c->P.Q[0], bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess && Qacc) e = cudaMemcpyAsync(Qacc, c->P.Qacc[0], bytes, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e);
+    const int rc = fetch(c);
+    if (acc_steps && rc != O2PIC_E_CUDA) *acc_steps = c->h_ctrl->acc_steps;
     return rc;
 }
 
@@ -1111,10 +1126,10 @@ int o2pic_read_moments(o2pic_ctx* c, double* density, uint64_t* acc_steps, int r
     }
     if (acc_steps) *acc_steps = steps;
     if (reset) {
-        cudaError_t e = cudaSuccess;
-        for (int s = 0; s < NSP && e == cudaSuccess; ++s) e = cudaMemset(c->P.Qacc[s], 0, 8 * (size_t)Ng);
-        const unsigned long long zero = 0;
-        if (e == cudaSuccess) e = cudaMemcpy(&c->d_ctrl->acc_steps, &zero, 8, cudaMemcpyHostToDevice);
+        cudaError_t e = cudaMemsetAsync(c->P.Qacc[0], 0, 8 * (size_t)NSP * Ng, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(&c->d_ctrl->acc_steps, 0, sizeof(unsigned long long), c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e);
     }
     return rc;
@@ -1124,9 +1139,7 @@ int o2pic_get_stats(o2pic_ctx* c, o2pic_stats* out) {
     if (!c || !out) return O2PIC_E_INVALID_ARG;
     int rc = sync_all(c);
     if (rc == O2PIC_E_CUDA) return rc;
-    DevCtrl h;
-    cudaError_t e = cudaMemcpy(&h, c->d_ctrl, sizeof(h), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(c, e);
+    const DevCtrl& h = *c->h_ctrl;
     std::memset(out, 0, sizeof(*out));
     for (int s = 0; s < NSP; ++s) {
         for (int k = 0; k < MAXPROC; ++k) out->events[s][k] = h.cnt.events[s][k];
@@ -1541,8 +1554,13 @@ int o2pic_batch_synchronize(o2pic_batch* b) {
     if (cudaSetDevice(b->device) != cudaSuccess) return O2PIC_E_CUDA;
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return O2PIC_E_CUDA;
     int first = O2PIC_OK;
+    for (o2pic_ctx* c : b->ctx)   // all copies in flight, then the waits
+        if (cudaMemcpyAsync(&c->h_ctrl->error_flags, &c->d_ctrl->error_flags, sizeof(unsigned long long),
+                            cudaMemcpyDeviceToHost, b->stream) != cudaSuccess)
+            return O2PIC_E_CUDA;
+    if (cudaStreamSynchronize(b->stream) != cudaSuccess) return O2PIC_E_CUDA;
     for (o2pic_ctx* c : b->ctx) {
-        const int rc = check_flags(c);
+        const int rc = latch_flags(c);
         if (rc && !first) first = rc;
     }
     return first;
