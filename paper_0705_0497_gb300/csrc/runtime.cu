@@ -1228,7 +1228,7 @@ struct o2pic_batch {
     PairSpec* dN = nullptr;               // [n] (17)
     uint4* dmap = nullptr;                // block maps, concatenated
     size_t map_push[NSP] = {0, 0, 0}, map_comp = 0, map_rh = 0, map_nh = 0, map_dh = 0, map_pair = 0;
-    int nb_push[NSP] = {0, 0, 0}, nb_comp = 0, nb_rh = 0, nb_nh = 0, nb_dh = 0, nb_pair = 0;
+    int nb_push[NSP] = {0, 0, 0}, nb_comp = 0, nb_rh = 0, nb_nh = 0, nb_nha = 0, nb_dh = 0, nb_pair = 0;
     bool any_recomb = false, any_neutral = false, any_edet = false;
     size_t smem_push = 0, smem_field = 0, smem_hist = 0;
 };
@@ -1284,18 +1284,21 @@ int fused_tables(o2pic_batch* b) {
         }
     b->nb_comp = (int)(map.size() - b->map_comp);
     // pair counts: blocks of A and of B (.w), then the candidates' blocks
-    auto add_count = [&](size_t& off, int& nb, int A, int B) {
+    auto add_count = [&](size_t& off, int& nb, int& nba, int A, int B) {
         off = map.size();
-        for (size_t i = 0; i < n; ++i)
-            for (unsigned w = 0; w < 2; ++w) {
+        for (unsigned w = 0; w < 2; ++w) {
+            for (size_t i = 0; i < n; ++i) {
                 const unsigned k = (unsigned)std::min<unsigned long long>(tiles(b->ctx[i]->P.sp[w ? B : A].cap), 32);
                 for (unsigned j = 0; j < k; ++j) map.push_back(make_uint4((unsigned)i, j, k, w));
             }
+            if (w == 0) nba = (int)(map.size() - off);
+        }
         nb = (int)(map.size() - off);
     };
-    add_count(b->map_dh, b->nb_dh, SP_OM, SP_E);
-    add_count(b->map_rh, b->nb_rh, SP_E, SP_OP);
-    add_count(b->map_nh, b->nb_nh, SP_OM, SP_OP);
+    int unused = 0;
+    add_count(b->map_dh, b->nb_dh, unused, SP_OM, SP_E);
+    add_count(b->map_rh, b->nb_rh, unused, SP_E, SP_OP);
+    add_count(b->map_nh, b->nb_nh, b->nb_nha, SP_OM, SP_OP);
     add_map(b->map_pair, b->nb_pair, [&](o2pic_ctx*) { return 16; });
     if (b->dP) cudaFree(b->dP);
     if (b->dR) cudaFree(b->dR);
@@ -1327,16 +1330,41 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
     unsigned long long step = c0->host_step;
     unsigned since = c0->since_check;
     unsigned long long launches = 0;
+    // the ion chains beside the electron kernel, as for a context alone (the
+    // streams and events of the first context carry the branches).  A few small
+    // discharges leave most of the GPU idle in each kernel: two of the paper's
+    // 18.4 -> 17.5 ms per RF cycle; 32 and 24 discharges fill it either way (within 1 %)
+    const cudaStream_t so = ION_FORK ? c0->aux[0] : s, sp2 = ION_FORK ? c0->aux[1] : s;
+    const bool early = ION_FORK && b->any_neutral && !b->any_edet && !b->any_recomb;
     for (uint64_t k = 0; k < b->K; ++k) {
         const bool ion = (step % S) == 0;
+        if (ion && ION_FORK) {
+            cudaEventRecord(c0->ev_fork, s);
+            cudaStreamWaitEvent(so, c0->ev_fork, 0);
+            cudaStreamWaitEvent(sp2, c0->ev_fork, 0);
+        }
         launch_push_batched(SP_E, b->dP, b->dmap + b->map_push[SP_E], b->nb_push[SP_E], b->smem_push, s);
         launches += 1;
         if (ion) {
             for (int sp = SP_OM; sp <= SP_OP; ++sp) {
-                launch_push_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], b->smem_push, s);
-                launches += 1;
-                launch_ion_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], s);
-                launches += 1;
+                const cudaStream_t st = sp == SP_OM ? so : sp2;
+                launch_push_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], b->smem_push, st);
+                if (sp == SP_OP && early) cudaEventRecord(c0->ev_pushed, sp2);
+                launch_ion_batched(sp, b->dP, b->dmap + b->map_push[sp], b->nb_push[sp], st);
+                launches += 2;
+            }
+            if (early) {
+                launch_pair_count_batched(b->dP, b->dN, b->dmap + b->map_nh, b->nb_nha, b->smem_hist, so);
+                cudaStreamWaitEvent(s, c0->ev_pushed, 0);
+                launch_pair_count_batched(b->dP, b->dN, b->dmap + b->map_nh + b->nb_nha, b->nb_nh - b->nb_nha,
+                                          b->smem_hist, s);
+                launches += 2;
+            }
+            if (ION_FORK) {
+                cudaEventRecord(c0->ev_join[0], so);
+                cudaEventRecord(c0->ev_join[1], sp2);
+                cudaStreamWaitEvent(s, c0->ev_join[0], 0);
+                cudaStreamWaitEvent(s, c0->ev_join[1], 0);
             }
             if (b->any_edet) {
                 launch_pair_count_batched(b->dP, b->dD, b->dmap + b->map_dh, b->nb_dh, b->smem_hist, s);
@@ -1351,9 +1379,12 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
                 launches += 3;
             }
             if (b->any_neutral) {
-                launch_pair_count_batched(b->dP, b->dN, b->dmap + b->map_nh, b->nb_nh, b->smem_hist, s);
+                if (!early) {
+                    launch_pair_count_batched(b->dP, b->dN, b->dmap + b->map_nh, b->nb_nh, b->smem_hist, s);
+                    launches += 1;
+                }
                 launch_pair_batched(b->dP, b->dN, b->dmap + b->map_pair, b->nb_pair, s);
-                launches += 2;
+                launches += 1;
             }
         }
         launch_field_batched(b->dP, n, b->smem_field, 0, ion ? 7 : 1, s);
