@@ -590,13 +590,17 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     TRY(ctx_alloc(c, &c->d_gflag, max_tiles));
     TRY(ctx_alloc(c, &c->d_gval, 2 * max_tiles));
     TRY(ctx_alloc(c, &c->d_gcount, 1));
-    // kernel shared-memory opt-in and launch shapes
-    size_t smax = 0;
-    for (int s = 0; s < NSP; ++s) smax = std::max(smax, push_smem_bytes(s, P));
-    smax = std::max(smax, sizeof(unsigned) * (size_t)Ng);
+    // kernel shared-memory opt-in and launch shapes.  The limits belong to the
+    // kernels, not to a context, so each is set to what the largest grid needs:
+    // contexts of any cell counts then leave it alike.
+    Params largest = P;
+    largest.Nc = MAX_NODES - 1;
+    largest.Ng = MAX_NODES;
+    size_t smax = sizeof(unsigned) * (size_t)MAX_NODES;
+    for (int s = 0; s < NSP; ++s) smax = std::max(smax, push_smem_bytes(s, largest));
     TRY(configure_push_smem(smax));
-    TRY(configure_field_smem(field_smem_bytes(P)));
-    TRY(configure_pair_count_smem(Nc));
+    TRY(configure_field_smem(field_smem_bytes(largest)));
+    TRY(configure_pair_count_smem(largest.Nc));
     for (int s = 0; s < NSP; ++s)
         c->grid_count[s] = (int)std::max<unsigned long long>(
             1, std::min<unsigned long long>(ceil_div(cfg->capacity[s], TILE), 2ull * c->num_sms));
