@@ -197,7 +197,6 @@ struct Params {
     float Kmax_r_hi, kappa_r;
     int have_recomb;
     unsigned int* rhist[2];      // 0: e, 1: O2+
-    uint2* rcand;                // candidates of (16), [capacity of e]
     unsigned int* rtot;          // [2][Nc] (cleared by the end-of-step kernel)
     unsigned int* rremoval;      // [2 * max_rremovals]: e slot, O2+ slot
     unsigned int max_rremovals;

@@ -335,19 +335,21 @@ int prepare(o2pic_ctx* c, cudaStream_t s) {
     return cuda_fail(c, cudaGetLastError());
 }
 
-// The cell-binned binary processes of a context (the O- candidate records of
-// the step are done with when (22) and (17) list theirs in their place): (22) e + O- -> O + 2e
-// (A = O-, only A removed), (16) e + O2+ -> O + O, (17) O- + O2+ -> O + O2.
+// The cell-binned binary processes of a context: (22) e + O- -> O + 2e (A = O-,
+// only A removed), (16) e + O2+ -> O + O, (17) O- + O2+ -> O + O2.  Each lists
+// its candidates (8 B per slot of A at most) in the place of A's collision
+// records (32 B per slot), which the step is done with by then.
 PairSpec spec_edet(o2pic_ctx* c) {
     const Params& P = c->P;
     return PairSpec{SP_OM, SP_E, P.dhist[0], P.dhist[1], P.dtot, P.Ktab_d, P.Kmax_d_hi, P.kappa_d, TAG_EDET,
-                    TAG_SHIFT_EDET, (uint2*)P.cand[SP_OM], &c->d_ctrl->pcand[0], P.dremoval, &c->d_ctrl->dremovals, P.max_dremovals,
+                    TAG_SHIFT_EDET, (uint2*)P.cand[SP_OM], &c->d_ctrl->pcand[0], P.dremoval,
+                    &c->d_ctrl->dremovals, P.max_dremovals,
                     &c->d_ctrl->cnt.edet_candidates, &c->d_ctrl->cnt.edetached, P.have_edet, P.thr_d, 1};
 }
 PairSpec spec_rec(o2pic_ctx* c) {
     const Params& P = c->P;
     return PairSpec{SP_E, SP_OP, P.rhist[0], P.rhist[1], P.rtot, P.Ktab_r, P.Kmax_r_hi, P.kappa_r, TAG_REC,
-                    TAG_SHIFT_REC, P.rcand, &c->d_ctrl->pcand[1], P.rremoval, &c->d_ctrl->rremovals, P.max_rremovals,
+                    TAG_SHIFT_REC, (uint2*)P.cand[SP_E], &c->d_ctrl->pcand[1], P.rremoval, &c->d_ctrl->rremovals, P.max_rremovals,
                     &c->d_ctrl->cnt.rec_candidates, &c->d_ctrl->cnt.recombined, P.have_recomb, 0.0f, 0};
 }
 PairSpec spec_neu(o2pic_ctx* c) {
@@ -569,7 +571,6 @@ int o2pic_create(const o2pic_config* cfg, o2pic_ctx** out) {
     // (16): e and O2+ tiles, totals, pair list
     TRY(ctx_alloc(c, &P.rhist[0], (ceil_div(cfg->capacity[SP_E], TILE) + 1) * Nc));
     TRY(ctx_alloc(c, &P.rhist[1], (ceil_div(cfg->capacity[SP_OP], TILE) + 1) * Nc));
-    TRY(ctx_alloc(c, &P.rcand, (size_t)cfg->capacity[SP_E]));
     TRY(ctx_alloc(c, &P.rtot, 2 * (size_t)Nc));
     P.max_rremovals = (unsigned)std::max<unsigned long long>(1, std::min(cfg->capacity[SP_E], cfg->capacity[SP_OP]));
     TRY(ctx_alloc(c, &P.rremoval, 2 * (size_t)P.max_rremovals));
