@@ -216,8 +216,8 @@ struct Params {
     // where each slot's is, per-tile cell offsets, cell totals and cell starts
     unsigned int coul_mask;
     float coul_K[6], coul_fa[6], coul_fb[6];
-    float4* csort[NSP];          // {vx, vy, vz, id} in cell order
-    unsigned int* cplace[NSP];   // place of each slot there
+    float4* csort[NSP];          // {vx, vy, vz, id} in cell order (in cand[s])
+    unsigned int* cplace[NSP];   // place of each slot there (in cand[s])
     unsigned int* chist[NSP];
     unsigned int* ctot[NSP];
     unsigned int* cstart[NSP];

@@ -962,9 +962,14 @@ int o2pic_set_coulomb(o2pic_ctx* c, uint32_t mask, double ln_lambda) {
         cudaError_t e = cudaSuccess;
         for (int s = 0; s < NSP && e == cudaSuccess; ++s) {
             const unsigned long long cap = P.sp[s].cap;
-            e = ctx_alloc(c, &P.csort[s], (size_t)cap);
-            if (e == cudaSuccess) e = ctx_alloc(c, &P.cplace[s], (size_t)cap);
-            if (e == cudaSuccess) e = ctx_alloc(c, &P.chist[s], (size_t)(ceil_div(cap, TILE) + 1) * P.Nc);
+            // the sorted entries and their places lie in the species' collision
+            // records (32 B per slot), which the step is done with when the
+            // Coulomb collisions run; (17) may have listed its candidates in the
+            // first 8 B per slot by then, so the places come after those and
+            // the entries in the second half
+            P.cplace[s] = (unsigned int*)((uint2*)P.cand[s] + cap);
+            P.csort[s] = (float4*)(P.cand[s] + (cap + 128));
+            e = ctx_alloc(c, &P.chist[s], (size_t)(ceil_div(cap, TILE) + 1) * P.Nc);
             if (e == cudaSuccess) e = ctx_alloc(c, &P.ctot[s], (size_t)P.Nc);
             if (e == cudaSuccess) e = ctx_alloc(c, &P.cstart[s], (size_t)P.Nc);
         }

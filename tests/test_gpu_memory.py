@@ -33,3 +33,16 @@ def test_bytes_per_slot(torch_cuda, species, expected):
     per_slot = (_used(torch_cuda) - before) / CAP
     d.close()
     assert per_slot <= expected + SLACK
+
+
+# The cell sort of the Coulomb collisions: 4 B per cell and tile of 8192 slots.
+@pytest.mark.parametrize("species", [0, 1, 2])
+def test_bytes_per_slot_of_coulomb(torch_cuda, species):
+    cap = [64, 64, 64]
+    cap[species] = CAP
+    d = api.Discharge(_config(), cap)
+    before = _used(torch_cuda)
+    d.set_coulomb(63)
+    per_slot = (_used(torch_cuda) - before) / CAP
+    d.close()
+    assert per_slot <= 4 * 128 / 8192 + SLACK
