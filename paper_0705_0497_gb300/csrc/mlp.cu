@@ -462,9 +462,9 @@ struct o2pic_mlp {
     float *P = nullptr, *G = nullptr, *Mo = nullptr, *Ve = nullptr;
     __nv_bfloat16* Wb = nullptr;
     unsigned char* is_w = nullptr;
-    // for a batch of up to cap rows: activations H[l] (l = 1..L-1), output Y,
-    // gradients at the pre-activations dZ[l] (l = 1..L)
-    int cap = 0;
+    // for a batch of up to cap rows: activations H[l] (l = 1..L-1); of up to
+    // gcap rows: output Y, gradients at the pre-activations dZ[l] (l = 1..L)
+    int cap = 0, gcap = 0;
     std::vector<float*> H, dZ;
     float *Y = nullptr, *partial = nullptr;
     int sms = 0;
@@ -478,28 +478,48 @@ constexpr int CARVEOUT = 30;   // per cent shared memory (about two blocks of th
 
 int layers(const o2pic_mlp* m) { return (int)m->w.size() - 1; }
 
+void free_rows(std::vector<float*>& v) {
+    for (float* p : v) if (p) cudaFree(p);
+    v.clear();
+}
+
 void free_acts(o2pic_mlp* m) {
-    for (float* h : m->H) if (h) cudaFree(h);
-    for (float* d : m->dZ) if (d) cudaFree(d);
-    m->H.clear();
-    m->dZ.clear();
+    free_rows(m->H);
+    m->cap = 0;
+}
+
+void free_grads(o2pic_mlp* m) {
+    free_rows(m->dZ);
     if (m->Y) cudaFree(m->Y);
     m->Y = nullptr;
-    m->cap = 0;
+    m->gcap = 0;
+}
+
+// v[l] = B rows of layer l's width, l = 1..last.
+int alloc_rows(o2pic_mlp* m, std::vector<float*>& v, int last, int B) {
+    v.assign(last + 1, nullptr);
+    for (int l = 1; l <= last; ++l)
+        if (cudaMalloc((void**)&v[l], sizeof(float) * (size_t)B * m->w[l]) != cudaSuccess) return O2PIC_E_CUDA;
+    return O2PIC_OK;
 }
 
 int ensure_acts(o2pic_mlp* m, int B) {
     if (B <= m->cap) return O2PIC_OK;
     free_acts(m);
-    const int L = layers(m);
-    m->H.assign(L, nullptr);
-    m->dZ.assign(L + 1, nullptr);
-    for (int l = 1; l < L; ++l)
-        if (cudaMalloc((void**)&m->H[l], sizeof(float) * (size_t)B * m->w[l]) != cudaSuccess) return O2PIC_E_CUDA;
-    for (int l = 1; l <= L; ++l)
-        if (cudaMalloc((void**)&m->dZ[l], sizeof(float) * (size_t)B * m->w[l]) != cudaSuccess) return O2PIC_E_CUDA;
-    if (cudaMalloc((void**)&m->Y, sizeof(float) * (size_t)B * m->w[L]) != cudaSuccess) return O2PIC_E_CUDA;
+    if (int rc = alloc_rows(m, m->H, layers(m) - 1, B)) return rc;
     m->cap = B;
+    return O2PIC_OK;
+}
+
+// What a backward pass needs besides (a caller who only runs forward does not
+// hold it).
+int ensure_grads(o2pic_mlp* m, int B) {
+    if (B <= m->gcap) return O2PIC_OK;
+    free_grads(m);
+    const int L = layers(m);
+    if (int rc = alloc_rows(m, m->dZ, L, B)) return rc;
+    if (cudaMalloc((void**)&m->Y, sizeof(float) * (size_t)B * m->w[L]) != cudaSuccess) return O2PIC_E_CUDA;
+    m->gcap = B;
     return O2PIC_OK;
 }
 
@@ -672,6 +692,7 @@ int o2pic_mlp_gradients(o2pic_mlp* m, const float* X, const float* T, int32_t B,
     if (!m || B < 1 || !X || !T || !loss) return O2PIC_E_INVALID_ARG;
     if (cudaSetDevice(m->device) != cudaSuccess) return O2PIC_E_CUDA;
     if (int rc = ensure_acts(m, B)) return rc;
+    if (int rc = ensure_grads(m, B)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     forward(m, X, m->Y, B, s);
     backward(m, X, T, B, loss, grad ? grad : m->G, nullptr, s);
@@ -683,6 +704,7 @@ int o2pic_mlp_train_step(o2pic_mlp* m, const float* X, const float* T, int32_t B
     if (!m || B < 1 || !X || !T || !loss || !(lr >= 0.0f)) return O2PIC_E_INVALID_ARG;
     if (cudaSetDevice(m->device) != cudaSuccess) return O2PIC_E_CUDA;
     if (int rc = ensure_acts(m, B)) return rc;
+    if (int rc = ensure_grads(m, B)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned long long t = m->t + 1;
     const Adam ad = {m->P, m->Mo, m->Ve, m->Wb, lr, 0.9f, 0.999f, 1e-8f, (float)(1.0 - std::pow(0.9, (double)t)),
@@ -699,6 +721,7 @@ void o2pic_mlp_destroy(o2pic_mlp* m) {
     cudaSetDevice(m->device);
     cudaDeviceSynchronize();
     free_acts(m);
+    free_grads(m);
     for (void* p : {(void*)m->P, (void*)m->G, (void*)m->Mo, (void*)m->Ve, (void*)m->Wb, (void*)m->is_w,
                     (void*)m->partial})
         if (p) cudaFree(p);

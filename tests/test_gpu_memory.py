@@ -46,3 +46,22 @@ def test_bytes_per_slot_of_coulomb(torch_cuda, species):
     per_slot = (_used(torch_cuda) - before) / CAP
     d.close()
     assert per_slot <= 4 * 128 / 8192 + SLACK
+
+
+# A network that only runs forward holds its activations, no gradients.
+def test_bytes_per_row_of_forward(torch_cuda):
+    torch = torch_cuda
+    widths, rows = [4] + 14 * [512] + [8], 100_000
+    m = api.MLP(widths, seed=1)
+    X = torch.zeros(rows, 4, device="cuda")
+    torch.cuda.empty_cache()
+    before = _used(torch)
+    Y = m.forward(X)
+    torch.cuda.synchronize()
+    per_row = (_used(torch) - before) / rows
+    assert Y.shape == (rows, 8)
+    # 2 MB granularity of 14 arrays, and of the output's allocator
+    assert per_row <= 4 * (14 * 512 + 8) + 15 * 2 ** 21 / rows + 2 ** 21 / rows
+    g, _ = m.gradients(X, Y + 1.0)
+    assert torch.isfinite(g).all()
+    m.close()
