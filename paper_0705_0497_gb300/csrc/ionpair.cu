@@ -62,35 +62,6 @@ __device__ __forceinline__ V load4(const T* __restrict__ A, unsigned long long p
     return v;
 }
 
-// A warp's candidates of a tile (bit 4 i + k of `pass`: this lane's slot first +
-// 4 HIST_T i + k) to the list, with one atomic.  Added one by one, 4e6 O- that
-// all pass the bound took 76-90 us for the counts of both species, now 37-48
-// (27 where next to none passes).  A candidate's word is drawn again, so that
-// the common case, few candidates, keeps no words in registers.
-__device__ __forceinline__ void list_candidates(const PairSpec& Sp, const PhiloxPre& pre, unsigned pass,
-                                                const uint4 (&id)[HIST_V], unsigned first) {
-    const int lane = threadIdx.x & 31;
-    if (!__any_sync(0xffffffffu, pass != 0u)) return;
-    const unsigned mine = __popc(pass);
-    unsigned upto = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, upto, o);
-        if (lane >= o) upto += y;
-    }
-    unsigned q = 0u;
-    if (lane == 31) q = atomicAdd(Sp.ncand, upto);   // at most the slots of A
-    q = __shfl_sync(0xffffffffu, q, 31) + upto - mine;
-#pragma unroll
-    for (int i = 0; i < HIST_V; ++i) {
-        const uint32_t ids[4] = {id[i].x, id[i].y, id[i].z, id[i].w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if ((pass >> (4 * i + k)) & 1u)
-                Sp.cand[q++] = make_uint2(first + 4u * HIST_T * i + k, philox_id(pre, ids[k]).x);
-    }
-}
-
 // Live particles per cell (post-push positions) of each tile of one of the two
 // species (`first`: A): hist[tile][cell], and the totals per cell (zero on
 // entry; the end-of-step kernel clears them), added once per block at the end.
@@ -142,17 +113,41 @@ __device__ __forceinline__ void pair_count_body(const Params& P, const PairSpec&
             }
         }
         if constexpr (FIRST) {
-            unsigned pass = 0u;         // bit 4 i + k: the slot is a candidate
+            const int lane = threadIdx.x & 31;
 #pragma unroll
             for (int i = 0; i < HIST_V; ++i) {
                 if (base + 4ull * HIST_T * i >= n) break;
                 const float xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
                 const uint32_t ids[4] = {id[i].x, id[i].y, id[i].z, id[i].w};
+                uint32_t w[4];
+                bool any = false;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    w[k] = philox_id(pre, ids[k]).x;
+                    any |= uniform(w[k]) < bound;
+                }
+                if (!any) continue;
+                // the lanes that are here add their candidates with one atomic:
+                // one by one, 4e6 O- that all pass took 76-90 us for the counts
+                // of both species, now 35 (27 where next to none passes)
+                const unsigned act = __activemask();
+                unsigned in[4];                 // of them, those whose slot k is a candidate
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (uniform(philox_id(pre, ids[k]).x) < bound && !is_dead(xs[k])) pass |= 1u << (4 * i + k);
+                    in[k] = __ballot_sync(act, uniform(w[k]) < bound && !is_dead(xs[k]));
+                const int first = __ffs(act) - 1;
+                unsigned q = 0u;
+                if (lane == first)              // at most the slots of A
+                    q = atomicAdd(Sp.ncand, __popc(in[0]) + __popc(in[1]) + __popc(in[2]) + __popc(in[3]));
+                q = __shfl_sync(act, q, first);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if ((in[k] >> lane) & 1u)
+                        Sp.cand[q + __popc(in[k] & ((1u << lane) - 1u))] =
+                            make_uint2((unsigned)(base + 4ull * HIST_T * i) + k, w[k]);
+                    q += __popc(in[k]);
+                }
             }
-            list_candidates(Sp, pre, pass, id, (unsigned)base);
         }
         __syncthreads();
         unsigned* H = (FIRST ? Sp.histA : Sp.histB) + (size_t)tile * Nc;
