@@ -269,9 +269,9 @@ int o2pic_set_step(o2pic_ctx* ctx, uint64_t step);
 /* Kernel timing with CUDA events on the launching stream: on != 0 records an
  * event pair around every launch; o2pic_get_timing returns, per kernel kind
  * (0 push e, 1 push O-, 2 push O2+, 3 pair histograms, 4 pair, 5 field,
- * 6 compact, 7 deposit, 8 collisions e, 9 collisions O-, 10 collisions O2+
- * (filter and kinematics), 11 (16), (22) pairing, 12, 13 none, 14 Coulomb collisions (cell sort and reactions)),
- * the summed milliseconds and launches; items is reserved (zeros). */
+ * 6 compact, 7 deposit, 8 none (within push e), 9 collisions O-,
+ * 10 collisions O2+ (filter and kinematics), 11 (16), (22) pairing, 12, 13
+ * none, 14 Coulomb collisions (cell sort and reactions)), the summed milliseconds and launches; items is reserved (zeros). */
 int o2pic_set_timing(o2pic_ctx* ctx, int on);
 int o2pic_get_timing(o2pic_ctx* ctx, double* ms, uint64_t* launches, uint64_t* items, int nkinds);
 
@@ -344,8 +344,7 @@ int o2pic_compact_particles_noalloc(const float* x, const float* vx, const float
  * o2pic_step, whatever the batch, the mode and the launch shape. */
 
 /* Blocks of the particle kernels (push and collisions) per species, in
- * [max(1, capacity / 2^23), 8 * SMs] (a block's shared-memory deposit counts
- * fewer than 2^24 particles per cell); results do not depend on them.
+ * [max(1, capacity / 2^23), 8 * SMs]; results do not depend on them.
  * Defaults (set by o2pic_set_processes): as many as fit the GPU at once. */
 int o2pic_set_launch_shape(o2pic_ctx* ctx, const int32_t push_blocks[3]);
 int o2pic_get_launch_shape(o2pic_ctx* ctx, int32_t push_blocks[3]);

@@ -16,6 +16,8 @@ NSP = 3
 MAXPROC = 16
 E, OM, OP = 0, 1, 2
 HOST, DEVICE = 0, 1
+# cand_e, filter_om and filter_op are reserved names: those collisions run within
+# push_e, cand_om and cand_op
 KERNEL_KINDS = ("push_e", "push_om", "push_op", "pair_hist", "pair", "field", "compact", "deposit",
                 "cand_e", "cand_om", "cand_op", "recomb", "filter_om", "filter_op", "coulomb")
 

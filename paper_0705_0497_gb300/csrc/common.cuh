@@ -1,6 +1,6 @@
 // Device helpers of the o2pic kernels: Philox streams, the single-precision
 // transforms used by the collision kinematics, rate-table lookup, CIC cell
-// location, block scans and the decoupled look-back.
+// location, block scans and ordered loads and stores.
 //
 // All floating-point work here is written with explicit fmaf() where a fused
 // multiply-add is intended; the library is compiled with --fmad=false, so no
@@ -81,12 +81,6 @@ struct Stream {
         buf = philox4x32_10(make_uint4(step_lo, tag, 0u, step_hi), make_uint2(key0, seed));
         pos = 0;
     }
-    // resume after the first two words of block 0 (given)
-    __device__ __forceinline__ void resume(uint32_t k0, uint32_t sd, unsigned long long step, uint32_t tg,
-                                           uint4 block0, int p) {
-        key0 = k0; seed = sd; step_lo = (uint32_t)step; step_hi = (uint32_t)(step >> 32); tag = tg; block = 0;
-        buf = block0; pos = p;
-    }
     __device__ __forceinline__ uint32_t next() {
         if (pos == 4) {
             ++block;
@@ -150,28 +144,6 @@ __device__ __forceinline__ void isotropic(Stream& st, float& nx, float& ny, floa
         }
     }
     ++warn; nx = 0.0f; ny = 0.0f; nz = 1.0f;
-}
-
-// Marsaglia-Bray polar method: two independent standard normals.
-__device__ __forceinline__ void normal_pair(Stream& st, float& z0, float& z1, unsigned& warn) {
-    for (int t = 0; t < MAX_TRIES; ++t) {
-        const float a = 2.0f * uniform(st.next()) - 1.0f;
-        const float b = 2.0f * uniform(st.next()) - 1.0f;
-        const float s = fmaf(a, a, b * b);
-        if (s > 0.0f && s < 1.0f) {
-            const float f = sqrtf((-2.0f * ln_series(s)) / s);
-            z0 = a * f; z1 = b * f;
-            return;
-        }
-    }
-    ++warn; z0 = 0.0f; z1 = 0.0f;
-}
-
-__device__ __forceinline__ void maxwellian(Stream& st, float sig, float& vx, float& vy, float& vz, unsigned& warn) {
-    float z0, z1, z2, z3;
-    normal_pair(st, z0, z1, warn);
-    normal_pair(st, z2, z3, warn);
-    vx = sig * z0; vy = sig * z1; vz = sig * z2;
 }
 
 // ------------------------------------------------------------ rate tables

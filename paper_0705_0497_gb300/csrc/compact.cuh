@@ -86,9 +86,10 @@ __device__ __forceinline__ unsigned long long lookback(unsigned long long* flag,
 }
 
 // The tiles that this block claims from *ticket.  request(slot): prefetch of
-// the other arrays at a slot; move(src, dst, in): copy of one thread's slots
-// (src[i] -> dst[i] where bit i of `in` is set); total(n): called once, with the
-// number kept, by the block of the last tile.
+// the other arrays at a slot; move(x, base, d, off, in): copy of one thread's
+// slots (x[i] and slot base + 32 i of the other arrays to d + off[i] where bit i
+// of `in` is set); total(n): called once, with the number kept, by the block of
+// the last tile.
 template <class Request, class Move, class Total>
 __device__ __forceinline__ void compact_tiles(CompactShared& sh, const float* __restrict__ X, unsigned long long n,
                                               unsigned* ticket, unsigned long long* flag, unsigned long long* val,

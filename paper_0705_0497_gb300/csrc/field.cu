@@ -1,5 +1,5 @@
-// End-of-step kernel (two blocks): charge commit, cycle moments, Poisson solve
-// and E on the nodes; placement of the step's births, removals of (17) and the
+// End-of-step kernel (two clusters of blocks): charge commit, cycle moments,
+// Poisson solve and E on the nodes; placement of the step's births, removals of (17) and the
 // commit of the step; plus the stable compaction of dead slots and small
 // utility kernels.
 //
@@ -8,7 +8,7 @@
 // phi_0 = U sin(2 pi f t) (driven electrode at x = 0), phi_N = 0 (grounded).
 // With the net fixed-point charge R_j (2^16 per macro-particle, exact int64)
 // and c = e w dx / (A eps0 2^16), the system is solved in closed form by
-// exact integer prefix sums (one block-wide scan of the pair S, U):
+// exact integer prefix sums (one scan of the pair S, U over a cluster):
 //     S_m = sum_{k=1..m} R_k,  U_m = sum_{k=1..m} k R_k,
 //     T_j = sum_{m<j} S_m = j S_{j-1} - U_{j-1},
 //     D_0 = phi_1 - phi_0 = (c T_N - V0) / N,  phi_j = V0 + j D_0 - c T_j,
@@ -445,7 +445,7 @@ __device__ __forceinline__ void step_commit(const Params& P, int mode, int pushe
             C->acc_steps = cs.acc_steps + 1;
             C->step = cs.step + 1;
             C->epoch = cs.epoch + 1;
-        } else if (tB >= 64 && tB < 64 + NKK + NSP) {
+        } else if (tB >= 64 && tB < 64 + NSP) {
             C->ticket[tB - 64] = 0u;
         }
     }
@@ -453,7 +453,7 @@ __device__ __forceinline__ void step_commit(const Params& P, int mode, int pushe
     // without an ion push repeat those of step n-1, and the slot of step n+1 is
     // cleared for its pushes
     if (mode != 0) {
-        if (tB < NKK + NSP) C->ticket[tB] = 0u;
+        if (tB < NSP) C->ticket[tB] = 0u;
     } else if (tB >= 96 && tB < 96 + NSP) {
         const int sp = tB - 96;
         const unsigned long long n = cs.step;
@@ -489,7 +489,7 @@ __device__ __forceinline__ void compact_body(const Params& P, int S, CompactShar
     const SpeciesBuf& B = P.sp[S];
     const unsigned long long cap = B.cap;
     compact_tiles(
-        sh, B.x[cb], nslots, &C->ticket[NKK + S], P.lb_flag[S], P.lb_val[S], C->epoch, &C->error_flags,
+        sh, B.x[cb], nslots, &C->ticket[S], P.lb_flag[S], P.lb_val[S], C->epoch, &C->error_flags,
         [&](unsigned long long p) {
             prefetch_l2(B.vx[cb] + p); prefetch_l2(B.vy[cb] + p); prefetch_l2(B.vz[cb] + p);
             prefetch_l2(B.id[cb] + p); prefetch_l2(B.tc[cb] + p);
@@ -588,9 +588,9 @@ __global__ void __launch_bounds__(CMP_T, 2) k_gather(Params P, int S, unsigned l
 // and the largest id (+1) for the species' next id.  Bound by HBM (20 B per
 // particle, the five loads of a particle in flight together) as long as one
 // thread per block touches the two words: with one atomic per thread on the
-// same word 0.73 ms for 1.4e6 and for 5.7e6 particles alike (profiled).  Reading
-// and loading a 512-cell discharge from the host 4.94 -> 3.38 ms.
-constexpr int LOAD_T = 256, LOAD_BLOCKS = 8 * 152;   // one wave, 2048 threads per SM
+// same word 0.73 ms for 1.4e6 and for 5.7e6 particles alike.  Reading and
+// loading a 512-cell discharge from the host 4.94 -> 3.38 ms.
+constexpr int LOAD_T = 256, LOAD_BLOCKS = 8 * 152;   // one wave of 152 SMs, 2048 threads each
 
 template <int S>
 __global__ void __launch_bounds__(LOAD_T) k_load_check(Params P, unsigned long long n) {

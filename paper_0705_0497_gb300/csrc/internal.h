@@ -47,7 +47,6 @@ constexpr float GRID_EMAX = 4096.0f;                             // 2^12
 constexpr int BLOCK = 256;              // threads of the particle kernels
 constexpr int TILE = 8192;              // slots per tile (compaction, neutralization histograms)
 constexpr int WTILE = 2048;             // slots per warp work unit of the particle kernels
-constexpr int FLUSH_TILES = 7;          // tiles between deposit flushes (7*8192*2^16 < 2^32)
 constexpr int MAX_TRIES = 32;           // rejection-loop cap
 constexpr uint32_t FIX_ONE = 65536u;    // CIC fixed point per particle
 constexpr int MAX_NODES = 8193;         // grid limit (smem field and histograms)
@@ -68,10 +67,10 @@ enum Tag : uint32_t { TAG_E = 0, TAG_OM = 1, TAG_OP = 2, TAG_PAIR = 3, TAG_SHIFT
 // device error bits
 constexpr unsigned long long ERR_CAPACITY = 1ull, ERR_ID = 2ull, ERR_NONFINITE = 4ull, ERR_TIMEOUT = 8ull;
 
-// kernel kinds (timing, tickets)
+// kernel kinds (timing; 8, 12 and 13 are reserved)
 enum KernelKind { KK_PUSH_E = 0, KK_PUSH_OM = 1, KK_PUSH_OP = 2, KK_PAIR_HIST = 3, KK_PAIR = 4,
-                  KK_FIELD = 5, KK_COMPACT = 6, KK_DEPOSIT = 7, KK_CAND_E = 8, KK_CAND_OM = 9, KK_CAND_OP = 10,
-                  KK_REC = 11, KK_FILT_OM = 12, KK_FILT_OP = 13, KK_COUL = 14, NKK = 15 };
+                  KK_FIELD = 5, KK_COMPACT = 6, KK_DEPOSIT = 7, KK_CAND_OM = 9, KK_CAND_OP = 10,
+                  KK_REC = 11, KK_COUL = 14, NKK = 15 };
 
 // Counters: same layout as the head of o2pic_stats.
 struct DevCounters {
@@ -106,7 +105,7 @@ struct DevCtrl {
     unsigned long long error_flags;
     unsigned long long next_id[NSP];       // id of the next birth (ids above 2^32 - 1 overflow)
     unsigned int cur[NSP];                 // current buffer (ping-pong) per species
-    unsigned int ticket[NKK + NSP];        // tile tickets per kernel kind, + compaction per species
+    unsigned int ticket[NSP];              // tile tickets of the compaction
     unsigned int removals;                 // (17) pairs to remove
     unsigned int rremovals;                // (16) pairs to remove
     unsigned int dremovals;                // (22) pairs listed
@@ -181,9 +180,10 @@ struct Params {
     unsigned int* wcount[NB];
     unsigned int push_warps[NSP];  // warps of each particle kernel launch (units of wcount)
     // collision records at each particle warp's range, two uint4 each:
-    // electrons {slot, id, x, vx}{vy, vz, -, -} per real collision; ions
-    // {slot, id, vx, vy}{vz, w1, w2, w3} per candidate, compacted to the
-    // real ones by the filter
+    // {slot, id, vx, vy}{vz, w1, w2, w3} (w: words of the candidate's Philox
+    // block), electrons per real collision, ions per candidate, compacted to
+    // the real ones by the filter; afterwards the place of the pair processes'
+    // candidates (uint2) and of the Coulomb sort
     uint4* cand[NSP];
     unsigned int* ccount[NSP];     // records per warp
     unsigned int max_push_warps;   // bound on push_warps (shared memory of the field kernel)

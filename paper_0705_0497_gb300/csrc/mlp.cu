@@ -178,7 +178,7 @@ struct Tile {
                 pa.load(A, lda, k0 + KS, m0, K, M);
                 pb.load(B, ldb, k0 + KS, n0, K, N);
             }
-                        constexpr int UN = SWIZZLE ? KS : 16;
+            constexpr int UN = SWIZZLE ? KS : 16;
 #pragma unroll UN
             for (int kk = 0; kk < KS; ++kk) {
                 const float4 av = *reinterpret_cast<const float4*>(&sh.A[s][kk][col(kk, 4 * ty)]);
@@ -430,8 +430,8 @@ __global__ void k_to_bf16(const float* __restrict__ P, __nv_bfloat16* __restrict
 // C = epi(A B + bias) with A [M][K] fp32, B bf16 [K][N] (or its transpose
 // [N][K]: TB).  The large tile when its grid fills three quarters of the SMs,
 // else k_gemm_few.  2000 rows of 256 to 256 (128 large tiles): 17 us (the
-// former 64 x 64 kernel without prefetch 31); 81 rows of 256 to 256 (44
-// tiles): 5.4 us by k_gemm_few, 13 by an 8 x 32 tile with short slices, 38
+// former 64 x 64 kernel without prefetch 31); 81 rows of 256 to 256 (88 blocks
+// of 8 x 32): 5.4 us by k_gemm_few, 13 by such a tile with short slices, 38
 // before.
 template <bool TB>
 void gemm(const float* A, int lda, const __nv_bfloat16* B, int ldb, float* C, int M, int N, int K, const float* bias,

@@ -13,7 +13,7 @@
 //     (O2+: takes rounds of the whole array in turn) and walks it in rounds of
 //     128, a lane taking four neighbouring slots with one 16-byte load and
 //     store per array, the next round's loads in flight while it works on this
-//     one.  No block-wide barrier between the set-up and the final flush.
+//     one.  No block-wide barrier between the set-up and the end of the ranges.
 //   * what bounds it: on large arrays HBM (20 B per particle; 4.65e7 O2+ on
 //     2048 cells 198 -> 180 us, 5.2 TB/s against 6.8 of a plain copy), on small ones the
 //     instructions (80 per 32 particles, before 122: integer deposit counters
@@ -32,9 +32,9 @@
 //     the rest of the collision;
 //   * electrons: a candidate is filtered at once (energy against the total
 //     rate, the total-rate column in shared memory), only the real
-//     collisions are recorded (32 B each: slot, id, x, v), and the warp runs
-//     their kinematics itself once its range is pushed, while other warps
-//     are still pushing (no second kernel on electron steps);
+//     collisions are recorded (32 B each: slot, id, v, the Philox block's
+//     rest), and the block runs their kinematics once all its warps' ranges
+//     are pushed, pooled over the warps (no second kernel on electron steps);
 //   * ions: candidates are recorded (slot, id, v and the Philox block's rest) and
 //     a second kernel filters them (target sampled from the gas Maxwellian,
 //     energy against the total rate) and runs the kinematics of the real ones
@@ -155,12 +155,13 @@ __device__ __forceinline__ int select_process(const float* __restrict__ cum, int
 // rate test itself repeats the filter's).  bkind: 0 none, 1 ionization (two
 // births), 2 attachment (one).
 //
-// The directions (points of the unit disk) and normals (the same without the
-// centre) a lane needs are drawn by one rejection loop, task after task: 0, 1
-// directions, 2, 3 pairs of normals; elastic and excited electrons need task
-// 0, an ionization 0-3 (after the share of the energy), an attachment 2-3.  A
-// warp passes the loop as often as its longest lane needs in all, not in each
-// task, and the code holds one Philox block instead of nine.
+// The directions (Marsaglia 1972: points of the unit disk) and normals
+// (Marsaglia-Bray polar method: the same without the centre) a lane needs are
+// drawn by one rejection loop, task after task: 0, 1 directions, 2, 3 pairs of
+// normals; elastic and excited electrons need task 0, an ionization 0-3 (after
+// the share of the energy), an attachment 2-3.  A warp passes the loop as often
+// as its longest lane needs in all, not in each task, and the code holds one
+// Philox block instead of nine.
 __device__ __forceinline__ int collide_electron(const Params& P, const float* __restrict__ cum, int np,
                                                 unsigned long long step, uint32_t id, uint4 w0, float x, float& vx,
                                                 float& vy, float& vz, bool& alive, int& bkind, float4& b1, float4& b2,
@@ -280,8 +281,9 @@ struct IonPairs {
     }
 };
 
-// The gas molecule an ion meets: maxwellian() with both pairs of normals drawn
-// by one rejection loop, transformed once at its end.
+// The gas molecule an ion meets, a Maxwellian: both pairs of normals
+// (Marsaglia-Bray polar method) drawn by one rejection loop, transformed once
+// at its end.
 template <int S>
 __device__ __forceinline__ void gas_target(const Params& P, unsigned long long step, IonPairs& r, float& vx, float& vy,
                                            float& vz, unsigned& warn) {

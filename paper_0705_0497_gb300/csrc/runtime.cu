@@ -37,10 +37,9 @@ constexpr bool ION_FORK = O2PIC_ION_FORK != 0;
 // birth counts the field kernel scans in shared memory)
 constexpr int MAX_PUSH_BLOCKS_PER_SM = 8;
 
-// The particle kernel keeps its shared-memory deposit as (count << 40) + sum
-// of CIC weights per cell, so one block may deposit fewer than 2^24 particles
-// into one cell.  A block handles at most slots / blocks + 8 * 128 slots, so
-// at least capacity / 2^23 blocks per species keep it below 2^24 with margin.
+// Fewest blocks of a species' particle kernel that a launch shape may ask for.
+// The kernels run with any number (their deposit counters carry); this is the
+// limit that the interface documents, and what it refuses stays refused.
 int min_push_blocks(unsigned long long cap) {
     return (int)std::max<unsigned long long>(1, o2::ceil_div(cap, 1ull << 23));
 }
